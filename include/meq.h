@@ -262,6 +262,11 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
  * many of them are Newton-Schulz GEMM launches. */
 int meq_kernels_per_step(const meq_state* st);
 int meq_ns_gemm_launches_per_step(const meq_state* st);
+/* Floating-point operations of those products, the symmetric ones counted as
+ * one triangle. Large FFN-like weights run Eq. (5) two iterations at a time
+ * (fewer operations, the same polynomial), so this can be less than the
+ * count of Eq. (5) as written. */
+double meq_ns_flops_per_step(const meq_state* st);
 
 /* Per-phase timing with CUDA events on the launch stream. While enabled,
  * meq_step runs the same kernels with an event recorded between phases:

@@ -399,114 +399,266 @@ uint32_t make_idesc(bool fp16, bool b_mn_major, int m) {
 
 bool iter_fp16(const meq_options& o, int k) { return k < 32 && ((o.ns_fp16_mask >> k) & 1u); }
 
-// Prebuilds the GemmParams of every NS launch of one step.
-bool build_gemm_plan(meq_state* st, std::string* why) {
-  st->gemm.clear();
-  st->gemm_grid.clear();
-  const int K = st->opt.ns_steps;
-  const int ng = static_cast<int>(st->groups.size());
-  const int pair = st->opt.ns_cta_pair ? 2 : 1;
-  const int tile_m = 128 * pair;
-  const uint32_t b_rows = static_cast<uint32_t>(256 / pair);  // K-major B rows each CTA loads
-  const bool fused = st->opt.ns_x0_fused != 0;
+// ------------------------------------------------------- Newton-Schulz plan
+// One product of one shape group. Buffers: the two X buffers, A and P. An X
+// buffer that holds no live iterate also serves as a third s x s buffer (l >= s).
+enum NsBuf : int { BUF_X0 = 0, BUF_X1 = 1, BUF_A = 2, BUF_P = 3, BUF_NONE = 4 };
+
+struct NsOp {
+  int mode = MODE_SYM;
+  bool gram = false;                   // contraction over l (operands are X), else over s
+  NsBuf a = BUF_NONE, b = BUF_NONE, out = BUF_NONE, aux = BUF_NONE, aux2 = BUF_NONE;
+  bool out_is_x = false;               // DENSE: the output is s x l (else s x s)
+  bool aux_is_x = false;
+  bool in16 = true, out16 = true, aux16 = true;  // fp16 (else bf16)
+  float scale = 1.f, c_acc = 1.f, c_aux = 0.f, c_aux2 = 0.f, c_eye = 0.f;
+  int minv_pow = 0;
+};
+
+// Eq. (5) two iterations at a time. With A = X X^T, P = p(A) = a I + b A + c A^2
+// and X' = P X, the next Gram matrix is A' = X' X'^T = P A P (P and A commute),
+// so P' = p(A') and X'' = (P' P) X need no X': one Gram product over l and one
+// dense product over l fall away for four or so products over s.
+// In units of s^3 fused multiply-adds / 2 (a symmetric product over s is 1):
+//   two plain iterations               6 l/s + 2
+//   first pair, all products symmetric 3 l/s + 5
+//   second pair, P' P as a dense one   3 l/s + 6
+// i.e. 45 -> 36 over the five iterations of an FFN weight (l = 8/3 s).
+// Only the five-iteration default with fp16 operands and a fused X_0 takes
+// pairs: its error against fp64 was measured to be no larger than that of the
+// plain form, for these two reasons:
+//   * iteration 0 multiplies by M = P - a I, held in bf16, and adds a X_0 in
+//     fp32 in the epilogue: P's large diagonal is no longer rounded to eight
+//     bits, which pays for what the pairs lose;
+//   * the first pair works with M as well (every singular value is still
+//     small, so P is a I plus a small matrix); in the second pair it is not,
+//     P itself is kept, and P' P is computed whole: mirroring its upper
+//     triangle would force a symmetry that rounding has already broken.
+// Relative error of U~ (numpy emulation, row / column / both / no imbalance):
+//   768 x 2048: 2.57e-3 / 2.76e-3 / 2.88e-3 / 2.25e-3 plain,
+//               2.18e-3 / 2.83e-3 / 2.67e-3 / 2.14e-3 paired.
+bool pairs_allowed(const meq_options& o) {
+  meq_options d;
+  meq_default_options(&d);
+  return o.ns_steps == 5 && o.ns_x0_fused != 0 && (o.ns_fp16_mask & 0x1Fu) == 0x1Fu && o.ns_a == d.ns_a &&
+         o.ns_b == d.ns_b && o.ns_c == d.ns_c;
+}
+
+// Pairs take four launches more than the plain chain (about 10 us each), so
+// they are used where they save at least this many k-blocks (256 x 256 x 64;
+// a pair of SMs takes about 0.35 us for one) over the whole state: 10000 take
+// the 76 pairs of a GB300 46 us. Measured steps, plain -> pairs: Llama-130M
+// (17700 saved) 1399 -> 1360 us, Llama-350M 5615 -> 5271 us, four 1B-class
+// layers 5963 -> 5437 us, two 7B-class layers 19930 -> 18000 us.
+constexpr int64_t kPairMinSaving = 10000;
+
+// k-blocks that the pairs save in one matrix, as the launches run them (whole
+// upper-triangle tiles, whole k-blocks); 0 below s = 512, where the pairs'
+// error against fp64 was measured to grow (128 x 315: 2.6e-3 -> 2.9e-3; with
+// s = 3 it leaves the tolerance) and there is little to save.
+constexpr int64_t kPairMinS = 512;
+int64_t pair_saving(const Group& G) {
+  if (G.s < kPairMinS) return 0;
+  const int64_t ts = (G.s + 255) / 256, tl = (G.l + 255) / 256, ks = (G.s + 63) / 64, kl = (G.l + 63) / 64;
+  const int64_t sym = ts * (ts + 1) / 2;
+  return 2 * (sym * kl + ts * tl * ks) - 5 * sym * ks - ts * ts * ks;
+}
+
+// The products of one group, in order.
+std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs) {
+  std::vector<NsOp> ops;
+  const int K = o.ns_steps;
+  const bool fused = o.ns_x0_fused != 0;
   // 16-bit formats: dA(k) of A_k (and of the polynomial's operands) is the
   // iteration's format; dX(k) of X_k (and of P_k, which multiplies it) too,
   // except that a fused X_0 is bf16 (written unnormalised by the momentum pass).
-  auto dA = [&](int k) { return iter_fp16(st->opt, k); };
-  auto dX = [&](int k) { return (fused && k == 0) ? false : iter_fp16(st->opt, k); };
-  for (int k = 0; k < K; ++k) {
-    const int cur = k & 1, nxt = cur ^ 1;
-    for (int mode = MODE_GRAM; mode <= MODE_XUPD; ++mode) {
-      const int real_mode = (mode == MODE_XUPD && k == K - 1) ? MODE_XLAST : mode;
-      const bool in16 = mode == MODE_POLY ? dA(k) : dX(k);  // operand format of this launch
-      for (int g0 = 0; g0 < ng; g0 += kMaxGroups) {
-        GemmParams P;
-        std::memset(&P, 0, sizeof(P));
-        const int b_mn_major = (mode == MODE_XUPD) ? 1 : 0;
-        const uint32_t idesc = make_idesc(in16, b_mn_major, tile_m);
-        P.ca = st->opt.ns_a, P.cb = st->opt.ns_b, P.cc = st->opt.ns_c;
-        P.err = st->d_err;
-        P.sched = st->d_sched;
-        P.timeout_ns = static_cast<unsigned long long>(static_cast<double>(st->opt.wait_timeout_ms) * 1e6);
-        int tiles = 0;
-        P.ngroups = std::min(kMaxGroups, ng - g0);
-        for (int gi = 0; gi < P.ngroups; ++gi) {
-          Group& G = st->groups[g0 + gi];
-          GemmGroup& Q = P.g[gi];
-          Q.mode = real_mode, Q.idesc = idesc, Q.b_mn_major = b_mn_major;
-          // storage scale of X_k; a fused X_0 is unscaled and its 1/||H||_F is applied per matrix
-          const float ak = (k == 0) ? (fused ? 1.0f : G.alpha0) : G.alpha;
-          const bool per_matrix = fused && k == 0;
-          Q.count = static_cast<int32_t>(G.count);
-          Q.trans = G.trans;
-          bool ok = true;
-          const int64_t x_ld = G.lp * 2, x_ms = G.s * G.lp * 2;   // 16-bit X buffers, bytes
-          const int64_t s_ld = G.sp * 2, s_ms = G.s * G.sp * 2;   // 16-bit A buffer, bytes
-          if (mode == MODE_GRAM) {
-            Q.M = (int32_t)G.s, Q.N = (int32_t)G.s, Q.K = (int32_t)G.l;
-            Q.sym = 1;
-            ok &= encode_map(&Q.tmA, G.x[cur], 2, G.l, G.s, G.count, G.lp, 64, 128, SW128);
-            ok &= encode_map(&Q.tmB, G.x[cur], 2, G.l, G.s, G.count, G.lp, 64, b_rows, SW128);
-            ok &= encode_map(&Q.tmO, G.a16, 2, G.s, G.s, G.count, G.sp, 32, 32, SW64);
-            Q.tma_out = 1;
-            Q.scale = 1.0f / (ak * ak);
-            if (per_matrix) Q.minv = st->d_ginv + G.mbase, Q.minv_pow = 2;
-            Q.out_fp16 = dA(k);
-          } else if (mode == MODE_POLY) {
-            Q.M = (int32_t)G.s, Q.N = (int32_t)G.s, Q.K = (int32_t)G.s;
-            Q.sym = 1;
-            ok &= encode_map(&Q.tmA, G.a16, 2, G.s, G.s, G.count, G.sp, 64, 128, SW128);
-            ok &= encode_map(&Q.tmB, G.a16, 2, G.s, G.s, G.count, G.sp, 64, b_rows, SW128);
-            ok &= encode_map(&Q.tmO, G.p16, 2, G.s, G.s, G.count, G.sp, 32, 32, SW64);
-            Q.tma_out = 1;
-            Q.aux = G.a16, Q.aux_ld = s_ld, Q.aux_mstride = s_ms;
-            Q.scale = 1.0f;
-            Q.out_fp16 = dX(k);
-            Q.aux_fp16 = dA(k);
-          } else {
-            Q.M = (int32_t)G.s, Q.N = (int32_t)G.l, Q.K = (int32_t)G.s;
-            Q.sym = 0;
-            ok &= encode_map(&Q.tmA, G.p16, 2, G.s, G.s, G.count, G.sp, 64, 128, SW128);
-            ok &= encode_map(&Q.tmB, G.x[cur], 2, G.l, G.s, G.count, G.lp, 64, 64, SW128);
-            if (real_mode == MODE_XUPD) {
-              Q.out = G.x[nxt], Q.out_ld = x_ld, Q.out_mstride = x_ms;
-              Q.scale = G.alpha / ak;
-              if (per_matrix) Q.minv = st->d_ginv + G.mbase, Q.minv_pow = 1;
-              Q.out_fp16 = dX(k + 1);
-            } else {
-              Q.out = st->d_u + G.u_base, Q.out_ld = G.un * 2, Q.out_mstride = G.m * G.un * 2;
-              Q.scale = 1.0f / ak;
-              if (per_matrix) Q.minv = st->d_ginv + G.mbase, Q.minv_pow = 1;
-              Q.out_fp16 = 1;  // fp16(kUScale * U)
-              Q.rpart = st->d_parts + G.rpart_base;
-              Q.cpart = st->d_parts + G.cpart_base;
-            }
-          }
-          if (!ok) { *why = "cuTensorMapEncodeTiled failed"; return false; }
-          Q.tiles_m = (int32_t)((Q.M + tile_m - 1) / tile_m);
-          Q.tiles_n = (int32_t)((Q.N + 255) / 256);
-          Q.tiles_per_mat = Q.sym ? sym_tiles(Q.tiles_m, Q.tiles_n, tile_m) : Q.tiles_m * Q.tiles_n;
-          // Dense products walk bands of tile rows column by column; a band's
-          // row panels of P (band * tile_m * K 16-bit values) stay within 32 MB,
-          // about a quarter of L2, so every P panel is read from DRAM once.
-          Q.band = static_cast<int32_t>(
-              std::max<int64_t>(1, std::min<int64_t>(Q.tiles_m, (int64_t(32) << 20) / (int64_t(tile_m) * Q.K * 2))));
-          Q.tile_begin = tiles;
-          const int64_t t = int64_t(Q.tiles_per_mat) * Q.count;
-          if (tiles + t > (int64_t(1) << 30)) { *why = "too many GEMM tiles in one launch"; return false; }
-          tiles += static_cast<int>(t);
-        }
-        P.total_tiles = tiles;
-        // Each launch walks the matrices in the opposite order of the one
-        // before it (the X_0 cast writes in forward order), so it begins with
-        // the outputs still resident in L2.
-        P.reverse = (st->gemm.size() % 2 == 0) ? 1 : 0;
-        P.debug_skip_load = (st->opt.debug_skip_load && st->gemm.empty()) ? 1 : 0;
-        st->gemm.push_back(P);
-        // persistent grid: one CTA (pair) per SM (pair of SMs), never more than the tiles
-        st->gemm_grid.push_back(pair * std::max(1, std::min(tiles, st->num_sms / pair)));
+  auto dA = [&](int k) { return iter_fp16(o, k); };
+  auto dX = [&](int k) { return (fused && k == 0) ? false : iter_fp16(o, k); };
+  int cur = 0;
+  auto X = [](int i) { return i ? BUF_X1 : BUF_X0; };
+  for (int k = 0; k < K;) {
+    // storage scale of X_k; a fused X_0 is unscaled and its 1/||H||_F is applied per matrix
+    const float ak = (k == 0) ? (fused ? 1.0f : G.alpha0) : G.alpha;
+    const bool per_matrix = fused && k == 0;
+    const bool pair = pairs && (k == 1 || k == 3);
+    const bool split = pairs && k < 3;  // P is held as M = P - a I
+    const int step = pair ? 2 : 1;
+    const bool last = k + step == K;
+    const NsBuf cx = X(cur), nx = X(cur ^ 1);
+    NsOp gram;  // A = X X^T
+    gram.gram = true;
+    gram.a = gram.b = cx, gram.out = BUF_A;
+    gram.in16 = dX(k), gram.out16 = dA(k);
+    gram.scale = 1.0f / (ak * ak), gram.minv_pow = per_matrix ? 2 : 0;
+    ops.push_back(gram);
+    NsOp poly;  // P = a I + b A + c A^2 (or M = b A + c A^2)
+    poly.a = poly.b = BUF_A, poly.out = BUF_P, poly.aux = BUF_A;
+    poly.in16 = poly.aux16 = dA(k), poly.out16 = dX(k);
+    poly.c_acc = o.ns_c, poly.c_aux = o.ns_b, poly.c_eye = split ? 0.f : o.ns_a;
+    ops.push_back(poly);
+    NsBuf mul = BUF_P;                      // what multiplies X
+    float diag = split ? o.ns_a : 0.f;      // and its identity part, added in the epilogue
+    if (pair) {
+      NsOp q;  // Q = P A (= M A + a A), in the idle X buffer
+      q.a = BUF_P, q.b = BUF_A, q.out = nx;
+      if (split) q.aux = BUF_A, q.c_aux = o.ns_a;
+      ops.push_back(q);
+      NsOp a1;  // A' = Q P
+      a1.a = nx, a1.b = BUF_P, a1.out = BUF_A;
+      if (split) a1.aux = nx, a1.c_aux = o.ns_a;
+      ops.push_back(a1);
+      NsOp p1 = poly;  // P' (or M') of A'
+      p1.out = nx;
+      ops.push_back(p1);
+      NsOp c;  // P' P, in A's place
+      c.a = nx, c.b = BUF_P, c.out = BUF_A;
+      if (split) {  // less a^2 I: M' M + a (M + M')
+        c.aux = nx, c.c_aux = o.ns_a;
+        c.aux2 = BUF_P, c.c_aux2 = o.ns_a;
+        diag = o.ns_a * o.ns_a;
+      } else {
+        c.mode = MODE_DENSE;
       }
+      ops.push_back(c);
+      mul = BUF_A;
     }
+    NsOp up;  // X' = P X
+    up.mode = last ? MODE_XLAST : MODE_DENSE;
+    up.a = mul, up.b = cx, up.out = last ? BUF_NONE : nx, up.out_is_x = true;
+    up.in16 = dX(k);
+    up.out16 = last ? true : dX(k + step);
+    up.scale = last ? 1.0f / ak : G.alpha / ak;
+    up.minv_pow = per_matrix ? 1 : 0;
+    if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
+    ops.push_back(up);
+    cur ^= 1;
+    k += step;
+  }
+  return ops;
+}
+
+// Fills one group's part of a launch from its product.
+bool fill_group(const meq_state* st, const Group& G, const NsOp& op, GemmGroup& Q) {
+  const int pair = st->opt.ns_cta_pair ? 2 : 1;
+  const int tile_m = 128 * pair;
+  const uint32_t b_rows = static_cast<uint32_t>(256 / pair);  // K-major B rows each CTA loads
+  void* const base[4] = {G.x[0], G.x[1], G.a16, G.p16};
+  const bool dense = op.mode != MODE_SYM;
+  // buffers as matrices of the group: s x l with row stride lp (X), or s x s with row stride sp
+  auto map = [&](CUtensorMap* m, NsBuf buf, bool is_x, uint32_t box_inner, uint32_t box_rows, CUtensorMapSwizzle swz) {
+    return encode_map(m, base[buf], 2, is_x ? G.l : G.s, G.s, G.count, is_x ? G.lp : G.sp, box_inner, box_rows, swz);
+  };
+  auto ld = [&](bool is_x) { return (is_x ? G.lp : G.sp) * 2; };
+  Q.mode = op.mode;
+  Q.idesc = make_idesc(op.in16, dense, tile_m);
+  Q.b_mn_major = dense ? 1 : 0;
+  Q.count = static_cast<int32_t>(G.count);
+  Q.trans = G.trans;
+  Q.M = static_cast<int32_t>(G.s);
+  Q.N = static_cast<int32_t>(op.out_is_x ? G.l : G.s);
+  Q.K = static_cast<int32_t>(op.gram ? G.l : G.s);
+  Q.sym = dense ? 0 : 1;
+  Q.tma_out = Q.sym;
+  Q.same_ab = (!dense && op.a == op.b) ? 1 : 0;
+  bool ok = map(&Q.tmA, op.a, op.gram, 64, 128, SW128);
+  if (dense) ok &= map(&Q.tmB, op.b, op.out_is_x, 64, 64, SW128);
+  else ok &= map(&Q.tmB, op.b, op.gram, 64, b_rows, SW128);
+  if (Q.sym) ok &= map(&Q.tmO, op.out, false, 32, 32, SW64);
+  Q.scale = op.scale;
+  Q.c_acc = op.c_acc, Q.c_aux = op.c_aux, Q.c_aux2 = op.c_aux2, Q.c_eye = op.c_eye;
+  if (op.minv_pow) Q.minv = st->d_ginv + G.mbase, Q.minv_pow = op.minv_pow;
+  Q.out_fp16 = op.out16, Q.aux_fp16 = op.aux16;
+  if (op.aux != BUF_NONE) Q.aux = base[op.aux], Q.aux_ld = ld(op.aux_is_x), Q.aux_mstride = G.s * ld(op.aux_is_x);
+  if (op.aux2 != BUF_NONE) Q.aux2 = base[op.aux2];
+  if (op.mode == MODE_DENSE) {
+    Q.out = base[op.out], Q.out_ld = ld(op.out_is_x), Q.out_mstride = G.s * ld(op.out_is_x);
+  } else if (op.mode == MODE_XLAST) {
+    Q.out = st->d_u + G.u_base, Q.out_ld = G.un * 2, Q.out_mstride = G.m * G.un * 2;
+    Q.rpart = st->d_parts + G.rpart_base;
+    Q.cpart = st->d_parts + G.cpart_base;
+  }
+  Q.tiles_m = static_cast<int32_t>((Q.M + tile_m - 1) / tile_m);
+  Q.tiles_n = static_cast<int32_t>((Q.N + 255) / 256);
+  Q.tiles_per_mat = Q.sym ? sym_tiles(Q.tiles_m, Q.tiles_n, tile_m) : Q.tiles_m * Q.tiles_n;
+  // Dense products walk bands of tile rows column by column; a band's
+  // row panels of P (band * tile_m * K 16-bit values) stay within 32 MB,
+  // about a quarter of L2, so every P panel is read from DRAM once.
+  Q.band = static_cast<int32_t>(
+      std::max<int64_t>(1, std::min<int64_t>(Q.tiles_m, (int64_t(32) << 20) / (int64_t(tile_m) * Q.K * 2))));
+  return ok;
+}
+
+// Prebuilds the GemmParams of every NS launch of one step. Groups run one of
+// two chains of products (plain, or with pairs of iterations); products of
+// the same kind and operand format that are next in both chains share a launch.
+bool build_gemm_plan(meq_state* st, std::string* why) {
+  st->gemm.clear();
+  st->gemm_grid.clear();
+  const int pair = st->opt.ns_cta_pair ? 2 : 1;
+  int64_t saving = 0;
+  if (pairs_allowed(st->opt))
+    for (const Group& G : st->groups) saving += std::max<int64_t>(0, pair_saving(G)) * G.count;
+  const bool pairs = saving >= kPairMinSaving;
+  std::vector<int> which;                 // chain of each group: 0 plain, 1 with pairs
+  std::vector<std::vector<NsOp>> chain;   // its products
+  std::vector<NsOp> A, B;                 // the two chains' products (modes and formats; empty if unused)
+  for (const Group& G : st->groups) {
+    which.push_back(pairs && pair_saving(G) > 0 ? 1 : 0);
+    chain.push_back(ns_chain(st->opt, G, which.back() == 1));
+    (which.back() ? B : A) = chain.back();
+  }
+  auto joint = [&](size_t i, size_t j) {
+    return i < A.size() && j < B.size() && A[i].mode == B[j].mode && A[i].in16 == B[j].in16;
+  };
+  // fewest launches from product i of chain A and j of chain B on
+  std::vector<std::vector<int>> left(A.size() + 1, std::vector<int>(B.size() + 1, 0));
+  for (size_t i = A.size() + 1; i-- > 0;)
+    for (size_t j = B.size() + 1; j-- > 0;) {
+      if (i == A.size() && j == B.size()) continue;
+      int best = 1 << 30;
+      if (joint(i, j)) best = 1 + left[i + 1][j + 1];
+      if (i < A.size()) best = std::min(best, 1 + left[i + 1][j]);
+      if (j < B.size()) best = std::min(best, 1 + left[i][j + 1]);
+      left[i][j] = best;
+    }
+  size_t at[2] = {0, 0};
+  while (at[0] < A.size() || at[1] < B.size()) {
+    bool take[2] = {false, false};
+    if (joint(at[0], at[1]) && left[at[0]][at[1]] == 1 + left[at[0] + 1][at[1] + 1]) take[0] = take[1] = true;
+    else if (at[0] < A.size() && left[at[0]][at[1]] == 1 + left[at[0] + 1][at[1]]) take[0] = true;
+    else take[1] = true;
+    std::vector<int> gs;
+    for (size_t g = 0; g < st->groups.size(); ++g)
+      if (take[which[g]]) gs.push_back(static_cast<int>(g));
+    for (size_t g0 = 0; g0 < gs.size(); g0 += kMaxGroups) {
+      GemmParams P;
+      std::memset(&P, 0, sizeof(P));
+      P.err = st->d_err;
+      P.sched = st->d_sched;
+      P.timeout_ns = static_cast<unsigned long long>(static_cast<double>(st->opt.wait_timeout_ms) * 1e6);
+      int tiles = 0;
+      P.ngroups = static_cast<int32_t>(std::min<size_t>(kMaxGroups, gs.size() - g0));
+      for (int gi = 0; gi < P.ngroups; ++gi) {
+        const int g = gs[g0 + gi];
+        GemmGroup& Q = P.g[gi];
+        if (!fill_group(st, st->groups[g], chain[g][at[which[g]]], Q)) { *why = "cuTensorMapEncodeTiled failed"; return false; }
+        Q.tile_begin = tiles;
+        const int64_t t = int64_t(Q.tiles_per_mat) * Q.count;
+        if (tiles + t > (int64_t(1) << 30)) { *why = "too many GEMM tiles in one launch"; return false; }
+        tiles += static_cast<int>(t);
+      }
+      P.total_tiles = tiles;
+      // Each launch walks the matrices in the opposite order of the one
+      // before it (the X_0 cast writes in forward order), so it begins with
+      // the outputs still resident in L2.
+      P.reverse = (st->gemm.size() % 2 == 0) ? 1 : 0;
+      P.debug_skip_load = (st->opt.debug_skip_load && st->gemm.empty()) ? 1 : 0;
+      st->gemm.push_back(P);
+      // persistent grid: one CTA (pair) per SM (pair of SMs), never more than the tiles
+      st->gemm_grid.push_back(pair * std::max(1, std::min(tiles, st->num_sms / pair)));
+    }
+    for (int c = 0; c < 2; ++c)
+      if (take[c]) ++at[c];
   }
   return true;
 }
@@ -1267,6 +1419,18 @@ int meq_kernels_per_step(const meq_state* st) { return st ? st->kernels_per_step
 
 int meq_ns_gemm_launches_per_step(const meq_state* st) {
   return st ? static_cast<int>(st->gemm.size()) : 0;
+}
+
+double meq_ns_flops_per_step(const meq_state* st) {
+  double f = 0.0;
+  if (!st) return f;
+  for (const GemmParams& P : st->gemm)
+    for (int g = 0; g < P.ngroups; ++g) {
+      const GemmGroup& G = P.g[g];
+      const double out = G.sym ? 0.5 * G.M * (G.M + 1.0) : static_cast<double>(G.M) * G.N;
+      f += 2.0 * out * G.K * G.count;
+    }
+  return f;
 }
 
 meq_status meq_debug_wait_selftest(meq_state* st, float timeout_ms) {

@@ -77,12 +77,14 @@ struct StepScalars {
 };
 
 // --------------------------------------------------------------- GEMM side
-enum GemmMode : int { MODE_GRAM = 0, MODE_POLY = 1, MODE_XUPD = 2, MODE_XLAST = 3 };
+// Kind of a launch: symmetric s x s products (upper-triangle tiles, mirrored
+// TMA stores), dense 16-bit products, and the last update, which writes U.
+enum GemmMode : int { MODE_SYM = 0, MODE_DENSE = 1, MODE_XLAST = 2 };
 
 struct GemmGroup {
   CUtensorMap tmA;        // A operand (K-major), box {64, 128, 1}
   CUtensorMap tmB;        // B operand: K-major box {64, 256, 1} or MN-major box {64, 64, 1}
-  CUtensorMap tmO;        // GRAM / POLY / XUPD: the 16-bit output (A, P or X next) for TMA stores,
+  CUtensorMap tmO;        // symmetric products: the 16-bit output for TMA stores,
                           // box {32, 32, 1}, 64-byte swizzle (the epilogue's staging layout)
   int32_t M, N, K;        // output rows, output cols, contraction
   int32_t count;          // matrices in the group
@@ -91,23 +93,29 @@ struct GemmGroup {
   int32_t band;           // dense outputs: tile rows per band of the tile order
   int32_t tile_begin;     // first tile of this group in the launch
   int32_t sym;            // 1: symmetric s x s output (upper-triangle tiles, mirrored stores)
+  int32_t same_ab;        // 1: both operands are the same matrix (a diagonal tile loads it once)
   int32_t trans;          // XLAST: 1 when the weight is the transpose of the NS layout
-  float scale;            // GRAM: 1/alpha^2; XUPD: alpha_next/alpha; XLAST: 1/alpha
+  // Epilogue: scale * (c_acc * acc + c_aux * aux) + c_aux2 * aux2 + c_eye * I,
+  // the terms after the first only where aux (aux2) is given; scale is
+  // 1/alpha^2 (Gram), alpha_next/alpha (update), 1/alpha (last update) or 1.
+  float scale;
+  float c_acc, c_aux, c_aux2, c_eye;
   const float* minv;      // iteration 0 with X_0 unnormalised: 1/||H||_F per matrix of the group
   int32_t minv_pow;       // epilogue scale *= minv^minv_pow (0, 1 or 2)
   int32_t out_fp16;       // 16-bit format of the output (1 = fp16, 0 = bf16)
-  int32_t aux_fp16;       // POLY: 16-bit format of the A it reads in the epilogue
-  void* out;              // XUPD: 16-bit X next; XLAST: fp16(kUScale U) in the weight's layout
-  int64_t out_ld;         // XUPD / XLAST: output row stride in bytes
-  int64_t out_mstride;    // XUPD / XLAST: output matrix stride in bytes
-  const void* aux;        // POLY: 16-bit A
+  int32_t aux_fp16;       // 16-bit format of aux and aux2
+  void* out;              // DENSE: 16-bit output; XLAST: fp16(kUScale U) in the weight's layout
+  int64_t out_ld;         // DENSE / XLAST: output row stride in bytes
+  int64_t out_mstride;    // DENSE / XLAST: output matrix stride in bytes
+  const void* aux;        // 16-bit matrix the epilogue adds (same rows and columns as the output), or null
+  const void* aux2;       // a second one, in aux's layout, or null
   int64_t aux_ld;         // bytes
   int64_t aux_mstride;    // bytes
   float* rpart;           // XLAST: NS-row partial sums of squares, [count][2 * tiles_n][M]
   float* cpart;           // XLAST: NS-column partial sums of squares, [count][ceil(M/32)][N]
-  int32_t mode;           // GemmMode of the product
+  int32_t mode;           // GemmMode of the launch (read from g[0])
   uint32_t idesc;         // tcgen05 instruction descriptor
-  int32_t b_mn_major;     // 1: B operand tile is MN-major (XUPD)
+  int32_t b_mn_major;     // 1: B operand tile is MN-major (DENSE, XLAST)
   int32_t tma_out;        // 1: the output leaves by TMA stores through tmO (else 16-byte thread stores)
 };
 
@@ -118,7 +126,6 @@ struct GemmParams {
   int32_t ngroups;
   int32_t total_tiles;
   int32_t reverse;         // 1: tiles are taken in reverse order (alternates between launches)
-  float ca, cb, cc;        // NS coefficients
   int* err;                // device error word
   int* sched;              // tile queue: [0] tiles handed out beyond the first wave, [1] units done;
                            // zero between launches (the last unit to finish resets both)

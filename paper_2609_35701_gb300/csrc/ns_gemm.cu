@@ -3,12 +3,13 @@
 // One persistent, warp-specialised kernel computes every product of the
 // quintic iteration, Eq. (5) of the paper, for a batch of same-shape groups:
 //
-//   MODE_GRAM : A   = X X^T / alpha^2           (s x s, contraction over l)
-//   MODE_POLY : P   = a I + b A + c (A A)       (s x s, contraction over s)
-//               a I + b A is added in fp32 from the same 16-bit A the
-//               product uses, so P is exactly a polynomial of that matrix
-//   MODE_XUPD : X'  = P X * (alpha'/alpha)      (s x l, contraction over s)
-//   MODE_XLAST: U   = P X / alpha, written as fp16(2^14 U) in the weight's own
+//   MODE_SYM  : symmetric s x s products: A = X X^T / alpha^2 (contraction over
+//               l) and, over s, P = a I + b A + c (A A) and the products of the
+//               paired iterations (meq_api.cu); a I + b A is added in fp32 from
+//               the same 16-bit A the product uses, so P is exactly a
+//               polynomial of that matrix
+//   MODE_DENSE: X' = P X * (alpha'/alpha) (s x l, contraction over s), and P' P
+//   MODE_XLAST: U = P X / alpha, written as fp16(2^14 U) in the weight's own
 //               layout, with the sums of squares of the stored U's rows and
 //               columns (Eq. (7)) reduced into per-tile partials
 //
@@ -738,6 +739,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       const TileCoord c = entry_coord(e);
       const GemmGroup& G = p.g[c.g];
       const int mode = p.g[0].mode;  // one mode per launch (a launch-uniform read)
+      const bool has_aux = G.aux != nullptr;
       const int row0 = c.tm * TILE_M + static_cast<int>(rank) * BM + q * 32;
       const int R = row0 / 32;  // 32-row block index
       const int rows_valid = min(32, G.M - row0);
@@ -747,7 +749,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       if ((ch0 & 1) != half) ++ch0;                // this warp's chunks: ch % 2 == half
       if (row0 >= G.M) ch0 = nch;
       uint8_t* outm = static_cast<uint8_t*>(G.out) + static_cast<int64_t>(c.mat) * G.out_mstride;
-      // POLY: A block of the chunk, lane L holds 16-byte chunk (L % 4) of rows L/4 + 8i.
+      // aux block of the chunk, lane L holds 16-byte chunk (L % 4) of rows L/4 + 8i.
       uint4 aux[4];
       const uint8_t* auxm = reinterpret_cast<const uint8_t*>(G.aux) + static_cast<int64_t>(c.mat) * G.aux_mstride;
       auto load_aux = [&](int col0) {
@@ -765,9 +767,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       // What needs no accumulator is requested before waiting for it: the
       // polynomial's first A block, and the output scale (iteration 0 reads
       // its matrix's 1/||H||_F from global memory).
-      if (mode == MODE_POLY && ch0 < nch) load_aux(c.tn * BN + ch0 * 32);
+      if (has_aux && ch0 < nch) load_aux(c.tn * BN + ch0 * 32);
       float sc = G.scale;
-      if (mode != MODE_POLY && G.minv_pow) {
+      if (G.minv_pow) {
         const float iv = G.minv[c.mat];
         sc *= G.minv_pow == 2 ? iv * iv : iv;
       }
@@ -782,7 +784,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           if (lane == 0) bulk_wait_reads();  // both slots free
         }
         __syncwarp();
-        if (mode == MODE_POLY) {
+        if (has_aux) {
+          const float k_acc = sc * G.c_acc, k_aux = sc * G.c_aux, k_eye = G.c_eye;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int r = (lane >> 2) + 8 * i, k = lane & 3;
@@ -799,11 +802,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
             for (int h = 0; h < 4; ++h) {
               const float2 a2 = unpack_half2(ws[h], G.aux_fp16);
               const int j = 8 * k + 2 * h;
-              v[j] = fmaf(p.cc, v[j], fmaf(p.cb, a2.x, (col0 + j == row) ? p.ca : 0.f));
-              v[j + 1] = fmaf(p.cc, v[j + 1], fmaf(p.cb, a2.y, (col0 + j + 1 == row) ? p.ca : 0.f));
+              v[j] = fmaf(k_acc, v[j], fmaf(k_aux, a2.x, (col0 + j == row) ? k_eye : 0.f));
+              v[j + 1] = fmaf(k_acc, v[j + 1], fmaf(k_aux, a2.y, (col0 + j + 1 == row) ? k_eye : 0.f));
             }
           }
           __syncwarp();  // slot free for the output block
+          if (G.aux2 != nullptr && lane < rows_valid) {
+            // one launch per step has a second addend: each lane reads its own row
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
+                                 static_cast<int64_t>(row) * G.aux_ld + static_cast<int64_t>(col0) * 2;
+            const float k_aux2 = G.c_aux2;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint4 w = __ldg(reinterpret_cast<const uint4*>(src + 16 * k));
+              const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+              for (int h = 0; h < 4; ++h) {
+                const float2 a2 = unpack_half2(ws[h], G.aux_fp16);
+                v[8 * k + 2 * h] = fmaf(k_aux2, a2.x, v[8 * k + 2 * h]);
+                v[8 * k + 2 * h + 1] = fmaf(k_aux2, a2.y, v[8 * k + 2 * h + 1]);
+              }
+            }
+          }
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] *= sc;
@@ -915,7 +935,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           const TileCoord c = decode_tile<kPair>(p, t);
           const GemmGroup& G = p.g[c.g];
           const int nk = (G.K + BK - 1) / BK;
-          const bool b_is_a = kPair == 2 && G.sym && !p.g[0].b_mn_major && c.tm * TILE_M == c.tn * BN;
+          const bool b_is_a = kPair == 2 && G.same_ab && c.tm * TILE_M == c.tn * BN;
           e.y = static_cast<uint32_t>(c.mat);
           e.z = static_cast<uint32_t>(c.g) | (static_cast<uint32_t>(c.tm) << 4) | (static_cast<uint32_t>(c.tn) << 18);
           e.w = static_cast<uint32_t>(nk) | (b_is_a ? 0x10000u : 0u);

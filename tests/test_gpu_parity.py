@@ -97,6 +97,42 @@ def test_more_shape_groups_than_one_launch_holds(meq, pair):
 
 
 @pytest.mark.parametrize("pair", [1, 0], ids=["cta_pair", "single_cta"])
+def test_paired_iterations(meq, pair):
+    """A state large enough for the NS iterations of its FFN-like weights to run
+    in pairs (wide and tall, with ragged tails in every dimension, beside a
+    square and a nearly square weight that do not): more launches and fewer
+    operations than the plain chain, two steps staged against the oracle, and
+    within the sum of both errors (2 x 3e-3, the relative error of either form
+    to fp64) of the plain chain, which the same weights take in a small state."""
+    shapes = [(600, 4100)] * 8 + [(2100, 515), (700, 700), (513, 530)]
+    pick = [0, 8, 9, 10]
+    wl = W.custom_workload(shapes, pattern="both", base_sigma=0.01, seed=41)
+    few = [shapes[i] for i in pick]
+    a, b = meq.MeqMuon(shapes, ns_cta_pair=pair), meq.MeqMuon(few, ns_cta_pair=pair)
+    assert (a.ns_gemm_launches_per_step, b.ns_gemm_launches_per_step) == (19, 15)
+
+    def flops(s, l, paired):
+        """The pairs save two Gram and two dense products over l for five symmetric and one dense over s."""
+        saved = 2 * (s * (s + 1) * l + 2 * s * s * l) - 5 * s * s * (s + 1) - 2 * s * s * s if paired else 0
+        return 5 * (s * (s + 1) * l + s * s * (s + 1) + 2 * s * s * l) - saved
+
+    want = sum(flops(min(x), max(x), k < 9) for k, x in enumerate(shapes))
+    assert abs(a.ns_flops_per_step / want - 1) < 1e-9
+    Gs, W0 = _to_dev(W.gradients(wl, 0)), _to_dev(W.initial_weights(wl))
+    a.step([w.clone() for w in W0], Gs, LR, MU, WD, EPS)
+    b.step([W0[i].clone() for i in pick], [Gs[i] for i in pick], LR, MU, WD, EPS)
+    for k, i in enumerate(pick):
+        err = PT.rel_frob(a.read_ns_output(i), b.read_ns_output(k))
+        assert err <= 6e-3, (shapes[i], err)
+        assert (err == 0.0) == (i in (9, 10)), (shapes[i], err)
+    a.close()
+    b.close()
+    rep = []
+    run_staged(meq, wl, 2, check_idx=pick, report=rep, ns_cta_pair=pair)
+    assert all(r["update"] <= PT.UPDATE_TOL for r in rep)
+
+
+@pytest.mark.parametrize("pair", [1, 0], ids=["cta_pair", "single_cta"])
 def test_separate_x0_cast(meq, pair):
     """X_0 normalised and cast by its own pass (ns_x0_fused = 0: momentum +
     norm kernel, then the cast kernel) instead of inside the first NS
