@@ -19,7 +19,15 @@
 namespace meq {
 namespace {
 
-constexpr int kThreads = 256;
+__device__ __forceinline__ int64_t mat_begin(const MatInfo& m, int which) {
+  return which == 0   ? m.chunk_begin
+         : which == 1 ? m.tile_begin
+         : which == 2 ? m.hchunk_begin
+         : which == 3 ? m.rblk_begin
+         : which == 4 ? m.slab_begin
+         : which == 5 ? m.xblk_begin
+                      : m.fold_begin;
+}
 
 // Largest i with begin(i) <= key; begin is nondecreasing in i. Entries that
 // own no work of the enumeration share their begin with the next entry (or
@@ -28,13 +36,23 @@ __device__ __forceinline__ int find_mat(const MatInfo* mats, int nmat, int64_t k
   int lo = 0, hi = nmat - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    const int64_t b = which == 0   ? mats[mid].chunk_begin
-                      : which == 1 ? mats[mid].tile_begin
-                      : which == 2 ? mats[mid].hchunk_begin
-                      : which == 3 ? mats[mid].rblk_begin
-                      : which == 4 ? mats[mid].slab_begin
-                                   : mats[mid].xblk_begin;
-    if (b <= key) lo = mid; else hi = mid - 1;
+    if (mat_begin(mats[mid], which) <= key) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// The same by a whole warp: its lanes probe 32 evenly spaced entries at a
+// time, so that 1024 entries take two dependent loads instead of ten.
+__device__ __forceinline__ int find_mat_warp(const MatInfo* mats, int nmat, int64_t key, int which) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = nmat;  // the answer lies in lo .. lo + n - 1
+  while (n > 1) {
+    const int step = (n + 31) / 32;
+    const int i = lo + lane * step;
+    const bool le = lane * step < n && mat_begin(mats[i], which) <= key;
+    const int last = 31 - __clz(__ballot_sync(0xffffffffu, le) | 1u);  // lanes 0 .. last hold
+    n = min(step, n - last * step);
+    lo += last * step;
   }
   return lo;
 }
@@ -517,22 +535,128 @@ __global__ void __launch_bounds__(kThreads) cast_x0_kernel(const MatInfo* __rest
 }
 
 // ----------------------------------------------------------------- statistics
-// sum_{k < count} p[k * stride] with eight independent partial sums (term k
-// goes to partial k % 8) so that the loads overlap; fixed order.
-__device__ __forceinline__ float strided_sum8(const float* __restrict__ p, int64_t count, int64_t stride) {
+// sum_{k0 <= k < k1} p[k * stride] with eight independent partial sums (term
+// k0 + i goes to partial i % 8) so that the loads overlap; fixed order.
+__device__ __forceinline__ float strided_sum8(const float* __restrict__ p, int64_t k0, int64_t k1, int64_t stride) {
   float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  int64_t k = 0;
-  for (; k + 8 <= count; k += 8) {
+  int64_t k = k0;
+  for (; k + 8 <= k1; k += 8) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) a8[u] += p[(k + u) * stride];
   }
-  for (; k < count; ++k) a8[k & 7] += p[k * stride];
+#pragma unroll
+  for (int u = 0; u < 7; ++u)
+    if (k + u < k1) a8[u] += p[(k + u) * stride];
   return ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
 }
 
-// K block sums at once: each value goes through the same warp tree and the
-// same in-order sum over warps as block_sum_f32 gives it alone, with one set
-// of barriers for all of them. sh holds at least 33 * K floats.
+// The vectors of one entry that come from partial sums: r and c of a hidden
+// weight (NS rows and columns, swapped for a transposed one), c of a
+// remaining 2D parameter.
+struct FoldVec {
+  const float* parts;  // [count][len]
+  int64_t count, len;
+  float* dst;
+  float inv;           // 1 / elements summed per entry
+};
+__device__ __forceinline__ FoldVec fold_vec(const MatInfo& M, int which, const float* parts, float* rvec, float* cvec) {
+  FoldVec v;
+  if (M.kind == KIND_HIDDEN) {
+    const bool cols = (which == 1) != (M.trans != 0);  // which: 0 NS rows, 1 NS columns
+    v.parts = parts + (which == 0 ? M.rpart_off : M.cpart_off);
+    v.count = which == 0 ? 2 * ((M.l + 255) / 256) : (M.s + 31) / 32;  // two epilogue halves per 256-column tile
+    v.len = which == 0 ? M.s : M.l;
+    v.dst = (cols ? cvec : rvec) + M.vec_off;
+    v.inv = 1.0f / static_cast<float>(cols ? M.m : M.n);
+  } else {
+    v.parts = parts + M.cpart_off;
+    v.count = (M.m + kColSlab - 1) / kColSlab;
+    v.len = M.n;
+    v.dst = cvec + M.vec_off;
+    v.inv = 1.0f / static_cast<float>(M.m);
+  }
+  return v;
+}
+
+// Row i of remaining 2D parameter mi: its RMS in place of the row's sum of
+// squares (left there by the row pass), and the row scale of Eq. (12).
+__device__ __forceinline__ void two_sided_row(const MatInfo& M, int64_t i, int mi, float delta, float* rvec, float* svec,
+                                              int* nonfinite) {
+  const float ss = rvec[M.vec_off + i];
+  if (!isfinite(ss)) atomicCAS(nonfinite, 0, mi + 1);
+  const float rms = sqrtf(ss * (1.0f / static_cast<float>(M.n)));
+  rvec[M.vec_off + i] = rms;
+  svec[M.vec_off + i] = rms > delta ? 1.0f / rms : 0.f;
+}
+
+// r and c (Eq. (7)) from the partial sums of squares, ahead of finalize: a
+// block takes kFoldCols consecutive entries of one vector, four per lane, and
+// each of its 8 warps an eighth of their partials, added in fixed order. The
+// rows of a remaining 2D parameter come first, one per thread.
+__global__ void __launch_bounds__(kThreads) fold_kernel(const MatInfo* __restrict__ mats, int nmat,
+                                                        const StepScalars* __restrict__ sc,
+                                                        const float* __restrict__ parts, float* __restrict__ rvec,
+                                                        float* __restrict__ cvec, float* __restrict__ svec,
+                                                        float* __restrict__ tvec, int* __restrict__ nonfinite) {
+  pdl_allow_dependents();
+  __shared__ float sh[kThreads / 32][kFoldCols];
+  const int64_t blk = blockIdx.x;
+  const int mi = find_mat_warp(mats, nmat, blk, 6);
+  const MatInfo& M = mats[mi];
+  const int64_t lb = blk - M.fold_begin;
+  const int64_t first = M.kind == KIND_HIDDEN ? (M.s + kFoldCols - 1) / kFoldCols : (M.m + kThreads - 1) / kThreads;
+  const int which = lb >= first ? 1 : 0;
+  if (M.kind == KIND_TWO_SIDED && which == 0) {
+    pdl_wait_predecessor();
+    const int64_t i = lb * kThreads + threadIdx.x;
+    if (i < M.m) two_sided_row(M, i, mi, sc->eps, rvec, svec, nonfinite);
+    return;
+  }
+  const FoldVec v = fold_vec(M, which, parts, rvec, cvec);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t j0 = (lb - (which ? first : 0)) * kFoldCols;
+  const int64_t per = (v.count + 7) / 8;
+  const int64_t k0 = w * per, k1 = min(k0 + per, v.count);
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  pdl_wait_predecessor();
+  const float* p = v.parts + j0 + lane;
+  if (j0 + kFoldCols <= v.len) {
+    int64_t k = k0;
+    for (; k + 4 <= k1; k += 4) {
+      float x[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[i][u] = p[(k + i) * v.len + 32 * u];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] += x[i][u];
+    }
+    for (; k < k1; ++k)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[u] += p[k * v.len + 32 * u];
+  } else {
+    for (int64_t k = k0; k < k1; ++k)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (j0 + lane + 32 * u < v.len) acc[u] += p[k * v.len + 32 * u];
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) sh[w][lane + 32 * u] = acc[u];
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t < kFoldCols && j0 + t < v.len) {
+    const float sum = ((sh[0][t] + sh[1][t]) + (sh[2][t] + sh[3][t])) + ((sh[4][t] + sh[5][t]) + (sh[6][t] + sh[7][t]));
+    const float rms = sqrtf(sum * v.inv);
+    v.dst[j0 + t] = rms;
+    if (M.kind == KIND_TWO_SIDED) tvec[M.vec_off + j0 + t] = rms > sc->eps ? 1.0f / rms : 0.f;
+  }
+}
+
+// K block sums at once, one barrier for all of them: every warp adds the
+// warps' sums up itself (the same tree in each, so all threads get the same
+// values). sh holds 32 * K floats that no other call of the block uses.
 template <int K>
 __device__ __forceinline__ void block_sum_multi(float (&v)[K], float* sh) {
   const unsigned FULL = 0xffffffffu;
@@ -541,49 +665,78 @@ __device__ __forceinline__ void block_sum_multi(float (&v)[K], float* sh) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
   if (l == 0) {
 #pragma unroll
     for (int k = 0; k < K; ++k) sh[32 * k + w] = v[k];
   }
   __syncthreads();
-  if (threadIdx.x < K) {
-    float r = 0.f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += sh[32 * threadIdx.x + i];
-    sh[32 * K + threadIdx.x] = r;
-  }
-  __syncthreads();
 #pragma unroll
-  for (int k = 0; k < K; ++k) v[k] = sh[32 * K + k];
+  for (int k = 0; k < K; ++k) {
+    v[k] = l < static_cast<int>(blockDim.x >> 5) ? sh[32 * k + l] : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
+  }
 }
 
-// Two-pass fp32 CVs of Eq. (8) of a (length la) and b (length lb) over their
-// entries above delta, both at once: the mean pass, then the squared
-// deviations.
-__device__ void block_cv2(const float* a, int64_t la, const float* b, int64_t lb, float delta, float* sh, float* ga,
-                          float* gb) {
-  float p[4] = {0.f, 0.f, 0.f, 0.f};  // count and sum over a, then over b
-  for (int64_t i = threadIdx.x; i < la; i += blockDim.x) {
-    const float x = a[i];
-    if (x > delta) p[0] += 1.f, p[1] += x;
+// r (length la) and c (length lb) of one entry, spread over the block. Up to
+// kStatRegs values per thread are read once and kept in registers for both
+// passes of the CVs and for the scale vector (3 round trips to L2 otherwise).
+constexpr int kStatRegs = 32;
+struct StatVecs {
+  const float *a, *b;
+  int64_t la, lb;
+  int nk;              // values per thread when they are kept in registers, else 0
+  float x[kStatRegs];  // entry threadIdx.x + k * kFinThreads of a followed by b
+
+  __device__ __forceinline__ void load() {
+    const int64_t len = la + lb;
+    nk = len <= static_cast<int64_t>(kStatRegs) * kFinThreads ? static_cast<int>((len + kFinThreads - 1) / kFinThreads) : 0;
+#pragma unroll
+    for (int k = 0; k < kStatRegs; ++k) {
+      if (k >= nk) break;
+      const int i = static_cast<int>(threadIdx.x) + k * kFinThreads;
+      x[k] = i < static_cast<int>(la) ? a[i] : (i < static_cast<int>(len) ? b[i - static_cast<int>(la)] : 0.f);
+    }
   }
-  for (int64_t i = threadIdx.x; i < lb; i += blockDim.x) {
-    const float x = b[i];
-    if (x > delta) p[2] += 1.f, p[3] += x;
+  // f(side, index, value) for every entry of this thread
+  template <typename F>
+  __device__ __forceinline__ void each(F f) const {
+    if (nk) {
+      const int na = static_cast<int>(la), n = static_cast<int>(la + lb);
+#pragma unroll
+      for (int k = 0; k < kStatRegs; ++k) {
+        if (k >= nk) break;
+        const int i = static_cast<int>(threadIdx.x) + k * kFinThreads;
+        if (i < n) f(i < na ? 0 : 1, i < na ? i : i - na, x[k]);
+      }
+    } else {
+#pragma unroll 8
+      for (int64_t i = threadIdx.x; i < la; i += kFinThreads) f(0, i, a[i]);
+#pragma unroll 8
+      for (int64_t i = threadIdx.x; i < lb; i += kFinThreads) f(1, i, b[i]);
+    }
   }
+};
+
+// Two-pass fp32 CVs of Eq. (8) of r and c over their entries above delta,
+// both at once: the mean pass, then the squared deviations.
+__device__ __forceinline__ void block_cv2(const StatVecs& v, float delta, float* sh, float* ga, float* gb) {
+  float p[4] = {0.f, 0.f, 0.f, 0.f};  // count and sum over r, then over c
+  v.each([&](int side, int64_t, float x) {
+    const bool in = x > delta, ia = in && side == 0, ib = in && side == 1;
+    p[0] += ia ? 1.f : 0.f, p[1] += ia ? x : 0.f;
+    p[2] += ib ? 1.f : 0.f, p[3] += ib ? x : 0.f;
+  });
   block_sum_multi<4>(p, sh);
   const float mean_a = p[0] > 0.f ? p[1] / p[0] : 0.f;
   const float mean_b = p[2] > 0.f ? p[3] / p[2] : 0.f;
   float q[2] = {0.f, 0.f};
-  for (int64_t i = threadIdx.x; i < la; i += blockDim.x) {
-    const float x = a[i];
-    if (x > delta) q[0] += (x - mean_a) * (x - mean_a);
-  }
-  for (int64_t i = threadIdx.x; i < lb; i += blockDim.x) {
-    const float x = b[i];
-    if (x > delta) q[1] += (x - mean_b) * (x - mean_b);
-  }
-  block_sum_multi<2>(q, sh);
+  v.each([&](int side, int64_t, float x) {
+    const float d = x - (side == 0 ? mean_a : mean_b);
+    q[0] += x > delta && side == 0 ? d * d : 0.f;
+    q[1] += x > delta && side == 1 ? d * d : 0.f;
+  });
+  block_sum_multi<2>(q, sh + 4 * 32);
   *ga = p[0] > 0.f ? sqrtf(q[0] / p[0]) / mean_a : 0.f;
   *gb = p[2] > 0.f ? sqrtf(q[1] / p[2]) / mean_b : 0.f;
 }
@@ -595,25 +748,26 @@ __device__ void block_cv2(const float* a, int64_t la, const float* b, int64_t lb
 //   remaining 2D: r = row RMS of B, c = column RMS of N_r(B) (Eq. (12)),
 //                1/r in svec, 1/c in tvec, their CVs for inspection;
 //   vector     : r[0] = RMS of B, 1/r[0] in svec (Eq. (13)).
+// folded: r and c of the hidden weights and c of the remaining 2D parameters
+// are there already (fold_kernel).
 // RMS values at or below eps are treated as zero (scale 0).
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const MatInfo* __restrict__ mats,
+__global__ void __launch_bounds__(kFinThreads, 2) finalize_kernel(const MatInfo* __restrict__ mats,
                                                                const StepScalars* __restrict__ sc,
                                                                const float* __restrict__ parts,
                                                                float* __restrict__ rvec, float* __restrict__ cvec,
                                                                float* __restrict__ svec, float* __restrict__ tvec,
                                                                MatStats* __restrict__ stats,
                                                                unsigned long long* __restrict__ dircount,
-                                                               int* __restrict__ nonfinite) {
+                                                               int* __restrict__ nonfinite, int folded) {
   pdl_allow_dependents();
   pdl_wait_predecessor();
-  __shared__ float shf[33 * 4];
+  __shared__ float shf[6 * 32];
   const MatInfo& M = mats[blockIdx.x];
   const float delta = sc->eps;
   float* r = rvec + M.vec_off;
   float* c = cvec + M.vec_off;
   float* s = svec + M.vec_off;
   const float inv_n = 1.0f / static_cast<float>(M.n);
-  const float inv_m = 1.0f / static_cast<float>(M.m);
   if (M.kind == KIND_VECTOR) {
     if (threadIdx.x == 0) {
       if (!isfinite(r[0])) atomicCAS(nonfinite, 0, static_cast<int>(blockIdx.x) + 1);
@@ -626,64 +780,40 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(const MatInfo* __
     }
     return;
   }
-  if (M.kind == KIND_TWO_SIDED) {
-    float* t = tvec + M.vec_off;
-    for (int64_t i = threadIdx.x; i < M.m; i += blockDim.x) {
-      if (!isfinite(r[i])) atomicCAS(nonfinite, 0, static_cast<int>(blockIdx.x) + 1);
-      const float rms = sqrtf(r[i] * inv_n);  // r holds the row sums of squares
-      r[i] = rms;
-      s[i] = rms > delta ? 1.0f / rms : 0.f;
-    }
-    // column sums over the slabs
-    const int64_t nslabs = (M.m + kColSlab - 1) / kColSlab;
-    for (int64_t j = threadIdx.x; j < M.n; j += blockDim.x) {
-      const float tot = strided_sum8(parts + M.cpart_off + j, nslabs, M.n);
-      const float rms = sqrtf(tot * inv_m);
-      c[j] = rms;
-      t[j] = rms > delta ? 1.0f / rms : 0.f;
+  if (!folded) {
+    if (M.kind == KIND_TWO_SIDED)
+      for (int64_t i = threadIdx.x; i < M.m; i += blockDim.x)
+        two_sided_row(M, i, static_cast<int>(blockIdx.x), delta, rvec, svec, nonfinite);
+    for (int which = M.kind == KIND_HIDDEN ? 0 : 1; which < 2; ++which) {
+      const FoldVec v = fold_vec(M, which, parts, rvec, cvec);
+      for (int64_t j = threadIdx.x; j < v.len; j += blockDim.x) {
+        const float rms = sqrtf(strided_sum8(v.parts + j, 0, v.count, v.len) * v.inv);
+        v.dst[j] = rms;
+        if (M.kind == KIND_TWO_SIDED) tvec[M.vec_off + j] = rms > delta ? 1.0f / rms : 0.f;
+      }
     }
     __syncthreads();
-    float gr, gc;
-    block_cv2(r, M.m, c, M.n, delta, shf, &gr, &gc);
-    if (threadIdx.x == 0) {
-      stats[blockIdx.x].gamma_r = static_cast<double>(gr);
-      stats[blockIdx.x].gamma_c = static_cast<double>(gc);
-      stats[blockIdx.x].direction = 2;
-    }
-    return;
   }
-  // NS rows (s of them) are the weight's rows, or its columns when transposed.
-  const int64_t tiles_n = 2 * ((M.l + 255) / 256);  // two epilogue halves per 256-column tile
-  const int64_t nrb = (M.s + 31) / 32;
-  for (int64_t i = threadIdx.x; i < M.s; i += blockDim.x) {
-    const float acc = strided_sum8(parts + M.rpart_off + i, tiles_n, M.s);
-    if (!M.trans) r[i] = sqrtf(acc * inv_n);
-    else c[i] = sqrtf(acc * inv_m);
-  }
-  for (int64_t j = threadIdx.x; j < M.l; j += blockDim.x) {
-    const float acc = strided_sum8(parts + M.cpart_off + j, nrb, M.l);
-    if (!M.trans) c[j] = sqrtf(acc * inv_m);
-    else r[j] = sqrtf(acc * inv_n);
-  }
-  __syncthreads();
   // Eq. (8) over entries > delta: two passes (mean, then squared deviations),
   // fp32 with fixed-order block reductions.
+  StatVecs vecs;
+  vecs.a = r, vecs.b = c, vecs.la = M.m, vecs.lb = M.n;
+  vecs.load();
   float gam0, gam1;
-  block_cv2(r, M.m, c, M.n, delta, shf, &gam0, &gam1);
+  block_cv2(vecs, delta, shf, &gam0, &gam1);
   int dir;
-  if (sc->rule == 1) {
+  if (M.kind == KIND_TWO_SIDED) {
+    dir = 2;  // its scales are written with r and c
+  } else if (sc->rule == 1) {
     // Eq. (6): every row scaled by sqrt(max(m, n)), no equilibration
     dir = 4;
     const float f = sqrtf(static_cast<float>(max(M.m, M.n)));
     for (int64_t i = threadIdx.x; i < M.m; i += blockDim.x) s[i] = f;
   } else {
     dir = gam0 >= gam1 - sc->tie_atol ? 0 : 1;
-    const float* v = dir == 0 ? r : c;
-    const int64_t len = dir == 0 ? M.m : M.n;
-    for (int64_t i = threadIdx.x; i < len; i += blockDim.x) {
-      const float x = v[i];
-      s[i] = x > delta ? 1.0f / x : 0.0f;   // RMS at or below delta: treated as zero
-    }
+    vecs.each([&](int side, int64_t i, float x) {
+      if (side == dir) s[i] = x > delta ? 1.0f / x : 0.0f;  // RMS at or below delta: treated as zero
+    });
   }
   if (threadIdx.x == 0) {
     stats[blockIdx.x].gamma_r = static_cast<double>(gam0);
@@ -865,9 +995,15 @@ cudaError_t launch_cast_x0(const LaunchCtx& L, bool fp16, cudaStream_t st) {
 }
 
 cudaError_t launch_stats(const LaunchCtx& L, cudaStream_t st) {
+  if (L.fold) {
+    const cudaError_t e = launch_pdl(fold_kernel, dim3((unsigned)L.total_folds), dim3(kThreads), 0, st, 1, L.mats,
+                                     L.nmat, L.sc, static_cast<const float*>(L.parts), L.rvec, L.cvec, L.svec, L.tvec,
+                                     L.nonfinite);
+    if (e != cudaSuccess) return e;
+  }
   return launch_pdl(finalize_kernel, dim3(L.nmat), dim3(kFinThreads), 0, st, 1, L.mats, L.sc,
                     static_cast<const float*>(L.parts), L.rvec, L.cvec, L.svec, L.tvec, L.stats, L.dircount,
-                    L.nonfinite);
+                    L.nonfinite, L.fold);
 }
 
 cudaError_t launch_apply(const LaunchCtx& L, cudaStream_t st) {

@@ -90,13 +90,14 @@ struct meq_state {
   int n = 0;
   std::vector<meq_shape> shapes;
   std::vector<int> kinds;                     // meq_kind per entry
-  int n_hidden = 0, n_rows = 0, n_two = 0;    // hidden / row-pass (remaining 2D + vectors) / two-sided
+  int n_hidden = 0;
   meq_options opt{};
   int device = 0;
   int num_sms = 0;
   std::vector<MatInfo> mats;
   std::vector<Group> groups;
-  int64_t total_chunks = 0, total_hchunks = 0, total_tiles = 0, total_rblks = 0, total_slabs = 0, total_xblks = 0;
+  int64_t total_chunks = 0, total_hchunks = 0, total_tiles = 0, total_rblks = 0, total_slabs = 0, total_xblks = 0,
+          total_folds = 0, max_parts = 0;
   int64_t mom_floats = 0, u_halves = 0, vec_floats = 0, parts_floats = 0;
   char* arena = nullptr;
   int64_t arena_bytes = 0;
@@ -236,7 +237,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
   st->mats.assign(n, MatInfo{});
   std::map<std::tuple<int64_t, int64_t, int>, int> gmap;
   st->groups.clear();
-  st->n_hidden = st->n_rows = st->n_two = 0;
+  st->n_hidden = 0;
   for (int i = 0; i < n; ++i) {
     const int64_t m = st->shapes[i].rows, c = st->shapes[i].cols;
     MatInfo& M = st->mats[i];
@@ -245,11 +246,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     M.trans = m > c ? 1 : 0;
     M.kind = st->kinds[i];
     M.group = -1;
-    if (M.kind != KIND_HIDDEN) {
-      ++st->n_rows;
-      if (M.kind == KIND_TWO_SIDED) ++st->n_two;
-      continue;
-    }
+    if (M.kind != KIND_HIDDEN) continue;
     ++st->n_hidden;
     auto key = std::make_tuple(M.s, M.l, M.trans);
     auto it = gmap.find(key);
@@ -273,6 +270,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     st->groups[g].mats.push_back(i);
   }
   int64_t mom = 0, u = 0, vec = 0, parts = 0, chunks = 0, hchunks = 0, tiles = 0, rblks = 0, slabs = 0, xblks = 0;
+  int64_t folds = 0, max_parts = 0;
   int64_t mslots = 0;
   for (auto& G : st->groups) {
     G.mbase = mslots;
@@ -299,6 +297,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     M.xblk_begin = xblks;
     M.rblk_begin = rblks;
     M.slab_begin = slabs;
+    M.fold_begin = folds;
     if (M.kind == KIND_HIDDEN) {
       const Group& G = st->groups[M.group];
       M.un = G.un;
@@ -310,6 +309,8 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
       // momentum + X_0: flat chunks of W, or 64 x 64 tiles when X_0 is W transposed
       xblks += M.trans ? ((M.m + kCastTile - 1) / kCastTile) * ((M.n + kCastTile - 1) / kCastTile)
                        : (M.m * M.n + kChunk - 1) / kChunk;
+      folds += (M.s + kFoldCols - 1) / kFoldCols + (M.l + kFoldCols - 1) / kFoldCols;
+      max_parts = std::max(max_parts, 2 * ((M.l + 255) / 256) * M.s + (M.s + 31) / 32 * M.l);
     } else {
       M.un = M.n;
       rblks += (M.m + 7) / 8;  // 8 rows (warps) per block
@@ -318,12 +319,15 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
         M.cpart_off = parts;
         parts += round_up(ns * M.n, 64);
         slabs += ns * ((M.n + 255) / 256);  // blocks: slab x 256-column chunk
+        folds += (M.m + kThreads - 1) / kThreads + (M.n + kFoldCols - 1) / kFoldCols;
+        max_parts = std::max(max_parts, ns * M.n);
       }
     }
   }
   st->mom_floats = mom, st->u_halves = u, st->vec_floats = vec, st->parts_floats = parts;
   st->total_chunks = chunks, st->total_hchunks = hchunks, st->total_tiles = tiles, st->total_xblks = xblks;
   st->total_rblks = rblks, st->total_slabs = slabs;
+  st->total_folds = folds, st->max_parts = max_parts;
   st->persistent_bytes = 0;
   for (int i = 0; i < n; ++i) st->persistent_bytes += 4 * st->mats[i].m * st->mats[i].n;
 
@@ -870,8 +874,11 @@ meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n
   C.n_hidden = st->n_hidden;
   C.total_rblks = st->total_rblks;
   C.total_slabs = st->total_slabs;
-  st->kernels_per_step = (st->n_hidden ? 2 : 0) + (st->n_rows ? 1 : 0) + (st->n_two ? 1 : 0) + 2 +
-                         static_cast<int>(st->gemm.size());
+  C.total_folds = st->total_folds;
+  C.fold = st->max_parts > kFoldMinParts ? 1 : 0;
+  st->kernels_per_step = (st->n_hidden ? 2 : 0) + (st->total_rblks ? 1 : 0) +
+                         (st->total_slabs ? 1 : 0) + C.fold +
+                         2 + static_cast<int>(st->gemm.size());
   st->step_host.assign(static_cast<size_t>(st->step_bytes), 0);
   st->last_stream = s;
   *out = st;
@@ -940,7 +947,7 @@ static meq_status enqueue_kernels(meq_state* st, cudaStream_t s, cudaEvent_t* ev
       if (e != cudaSuccess) return cuda_fail(st, e, "x0norm launch");
     }
   }
-  if (st->n_rows) {
+  if (st->total_rblks) {
     e = launch_rows(C, s);
     if (e != cudaSuccess) return cuda_fail(st, e, "rows launch");
   }
@@ -955,7 +962,7 @@ static meq_status enqueue_kernels(meq_state* st, cudaStream_t s, cudaEvent_t* ev
     if (e != cudaSuccess) return cuda_fail(st, e, "ns_gemm launch");
   }
   mark(3);
-  if (st->n_two) {
+  if (st->total_slabs) {
     e = launch_colpart(C, s);
     if (e != cudaSuccess) return cuda_fail(st, e, "colpart launch");
   }

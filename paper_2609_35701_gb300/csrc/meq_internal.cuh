@@ -54,6 +54,7 @@ struct MatInfo {
   int64_t slab_begin;    // first row slab of the column pass (remaining 2D only)
   int64_t tile_begin;    // first cast tile (hidden weights only)
   int64_t xblk_begin;    // first momentum-and-X_0 block (hidden weights only)
+  int64_t fold_begin;    // first block of the fold of the partial sums (hidden weights and remaining 2D)
   int64_t rpart_off;     // float offset of NS-row partial sums of squares [2 * ceil(l/256)][s]
   int64_t cpart_off;     // float offset of column partial sums of squares: NS columns
                          // [ceil(s/32)][l] (hidden) or normalised columns [slabs][n] (remaining 2D)

@@ -92,6 +92,17 @@ def test_ragged_mixed_kinds(meq):
     run_kinds(meq, wl, 2)
 
 
+@pytest.mark.parametrize("shapes,kinds", [
+    # hidden weights whose partial sums are folded by their own launch: vector lengths around a
+    # block's 128, counts that are no multiple of its 8 warps, wide and tall
+    ([(257, 1337), (1337, 257), (385, 640), (127, 2049)], [O.HIDDEN] * 4),
+    # longer than the statistics keep in registers (16384 entries), rows longer than 1024
+    ([(20000, 37), (130, 2052), (1, 9)], [O.REMAINING_2D, O.REMAINING_2D, O.VECTOR]),
+])
+def test_folded_statistics(meq, shapes, kinds):
+    run_kinds(meq, W.custom_workload(shapes, pattern="both", seed=53, kinds=kinds), 2)
+
+
 def test_rows_columns_and_vectors_at_the_rms_threshold(meq):
     """The reading of Eq. (9) for rows / columns whose RMS does not exceed
     delta (scale 0, no update from them), on the branches without
