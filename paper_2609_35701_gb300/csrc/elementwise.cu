@@ -9,8 +9,8 @@
 //   finalize      : r, c (Eq. (7)) from the partial sums of squares the last
 //                   NS epilogue wrote, gamma_r, gamma_c (Eq. (8)), the
 //                   direction (Eq. (11)) and the scale vector of Eq. (9).
-//   rows, colpart : momentum, row and column statistics of the remaining 2D
-//                   parameters and vectors (Eqs. (12), (13)).
+//   rowcol, rows, colpart : momentum, row and column statistics of the remaining
+//                   2D parameters and vectors (Eqs. (12), (13)).
 //   apply         : W <- (1 - lr wd) W - rho lr U~ (Eq. (14)).
 #include <algorithm>
 
@@ -26,7 +26,8 @@ __device__ __forceinline__ int64_t mat_begin(const MatInfo& m, int which) {
          : which == 3 ? m.rblk_begin
          : which == 4 ? m.slab_begin
          : which == 5 ? m.xblk_begin
-                      : m.fold_begin;
+         : which == 6 ? m.fold_begin
+                      : m.rc_begin;
 }
 
 // Largest i with begin(i) <= key; begin is nondecreasing in i. Entries that
@@ -336,7 +337,8 @@ __global__ void __launch_bounds__(kThreads) x0norm_kernel(const MatInfo* __restr
 
 // ------------------------------------------- remaining 2D parameters, vectors
 // B <- mu B + G (Eq. (10)) and the row sums of squares of B, one warp per row
-// (a vector is a single row). Row sums go to rvec.
+// (a vector is a single row; remaining 2D parameters with rows longer than
+// kRowColMax). Row sums go to rvec.
 __global__ void __launch_bounds__(kThreads) rows_kernel(const MatInfo* __restrict__ mats, int nmat,
                                                        float* __restrict__ mom, const float* const* __restrict__ grads,
                                                        const StepScalars* __restrict__ sc, float* __restrict__ rvec) {
@@ -370,6 +372,126 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(const MatInfo* __restric
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if (lane == 0) rvec[M.vec_off + row] = ss;
+}
+
+// Both passes over a remaining 2D parameter with rows of up to kRowColMax
+// entries in one: a warp keeps a row of B in registers while its sum of
+// squares is reduced, then adds the squares of the normalised row (Eq. (12),
+// inner operator) to its column sums, so B is read once (12 B / element where
+// rows_kernel and colpart_kernel moved 16). One block per slab of M.slab_rows
+// rows; slab sizes make whole waves of one block per SM.
+template <int kElems, bool kVec>
+__device__ __forceinline__ void rowcol_slab(const MatInfo& M, float* B, const float* G, int64_t r0, int64_t r1, float mu,
+                                            float eps, float* __restrict__ rss, float* __restrict__ cpart,
+                                            float (*sh)[kRowColMax]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int n = static_cast<int>(M.n);
+  // column of value u of this lane
+  auto col = [&](int u) { return kVec ? 128 * (u >> 2) + 4 * lane + (u & 3) : 32 * u + lane; };
+  float acc[kElems];
+#pragma unroll
+  for (int u = 0; u < kElems; ++u) acc[u] = 0.f;
+  for (int64_t row = r0 + w; row < r1; row += kRowColThreads / 32) {
+    float* Br = B + row * n;
+    const float* Gr = G + row * n;
+    float b[kElems];
+    float ss = 0.f;
+    if (kVec) {
+      float4 g4[kElems / 4], b4[kElems / 4];
+#pragma unroll
+      for (int k = 0; k < kElems / 4; ++k)
+        if (col(4 * k) < n) {
+          g4[k] = __ldcs(reinterpret_cast<const float4*>(Gr + col(4 * k)));
+          b4[k] = *reinterpret_cast<const float4*>(Br + col(4 * k));
+        }
+#pragma unroll
+      for (int k = 0; k < kElems / 4; ++k) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (col(4 * k) < n) {
+          x = make_float4(fmaf(mu, b4[k].x, g4[k].x), fmaf(mu, b4[k].y, g4[k].y), fmaf(mu, b4[k].z, g4[k].z),
+                          fmaf(mu, b4[k].w, g4[k].w));
+          *reinterpret_cast<float4*>(Br + col(4 * k)) = x;
+        }
+        b[4 * k] = x.x, b[4 * k + 1] = x.y, b[4 * k + 2] = x.z, b[4 * k + 3] = x.w;
+      }
+    } else {
+      float g[kElems];
+#pragma unroll
+      for (int u = 0; u < kElems; ++u) {
+        g[u] = b[u] = 0.f;
+        if (col(u) < n) g[u] = __ldcs(Gr + col(u)), b[u] = Br[col(u)];
+      }
+#pragma unroll
+      for (int u = 0; u < kElems; ++u) {
+        b[u] = fmaf(mu, b[u], g[u]);
+        if (col(u) < n) Br[col(u)] = b[u];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) ss += b[u] * b[u];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) rss[row] = ss;
+    const float rms = sqrtf(ss / static_cast<float>(n));
+    const float rinv = rms > eps ? 1.0f / rms : 0.f;
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) {
+      const float x = b[u] * rinv;
+      acc[u] = fmaf(x, x, acc[u]);
+    }
+  }
+  // the warps' column sums, in a fixed order: w and w + 8 first, then 0 .. 7
+  constexpr int kHalf = kRowColThreads / 64;
+  if (w >= kHalf) {
+#pragma unroll
+    for (int u = 0; u < kElems; ++u)
+      if (col(u) < n) sh[w - kHalf][col(u)] = acc[u];
+  }
+  __syncthreads();
+  if (w < kHalf) {
+#pragma unroll
+    for (int u = 0; u < kElems; ++u)
+      if (col(u) < n) sh[w][col(u)] += acc[u];
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < n; c += kRowColThreads) {
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < kHalf; ++i) t += sh[i][c];
+    cpart[c] = t;
+  }
+}
+
+__global__ void __launch_bounds__(kRowColThreads, 1) rowcol_kernel(const MatInfo* __restrict__ mats, int nmat,
+                                                                  float* __restrict__ mom,
+                                                                  const float* const* __restrict__ grads,
+                                                                  const StepScalars* __restrict__ sc,
+                                                                  float* __restrict__ rvec, float* __restrict__ parts) {
+  pdl_allow_dependents();
+  __shared__ float sh[kRowColThreads / 64][kRowColMax];
+  const int64_t blk = blockIdx.x;
+  const int mi = find_mat(mats, nmat, blk, 7);
+  const MatInfo& M = mats[mi];
+  const int64_t ls = blk - M.rc_begin;
+  const int64_t r0 = ls * M.slab_rows;
+  const int64_t r1 = min(r0 + M.slab_rows, M.m);
+  pdl_wait_predecessor();
+  const float mu = sc->mu, eps = sc->eps;
+  float* B = mom + M.mom_off;
+  const float* G = grads[mi];
+  float* rss = rvec + M.vec_off;
+  float* cp = parts + M.cpart_off + ls * M.n;
+  if ((M.n & 3) == 0) {
+    if (M.n <= 256) rowcol_slab<8, true>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+    else if (M.n <= 512) rowcol_slab<16, true>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+    else if (M.n <= 768) rowcol_slab<24, true>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+    else rowcol_slab<32, true>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+  } else {
+    if (M.n <= 256) rowcol_slab<8, false>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+    else if (M.n <= 512) rowcol_slab<16, false>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+    else if (M.n <= 768) rowcol_slab<24, false>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+    else rowcol_slab<32, false>(M, B, G, r0, r1, mu, eps, rss, cp, sh);
+  }
 }
 
 // Column sums of squares of N_r(B) (Eq. (12), inner operator): one block per
@@ -570,7 +692,7 @@ __device__ __forceinline__ FoldVec fold_vec(const MatInfo& M, int which, const f
     v.inv = 1.0f / static_cast<float>(cols ? M.m : M.n);
   } else {
     v.parts = parts + M.cpart_off;
-    v.count = (M.m + kColSlab - 1) / kColSlab;
+    v.count = (M.m + M.slab_rows - 1) / M.slab_rows;
     v.len = M.n;
     v.dst = cvec + M.vec_off;
     v.inv = 1.0f / static_cast<float>(M.m);
@@ -979,6 +1101,11 @@ cudaError_t launch_x0norm(const LaunchCtx& L, cudaStream_t st) {
 cudaError_t launch_rows(const LaunchCtx& L, cudaStream_t st) {
   return launch_pdl(rows_kernel, dim3((unsigned)L.total_rblks), dim3(kThreads), 0, st, 1, L.mats, L.nmat, L.mom,
                     L.grads, L.sc, L.rvec);
+}
+
+cudaError_t launch_rowcol(const LaunchCtx& L, cudaStream_t st) {
+  return launch_pdl(rowcol_kernel, dim3((unsigned)L.total_rcs), dim3(kRowColThreads), 0, st, 1, L.mats, L.nmat, L.mom,
+                    L.grads, L.sc, L.rvec, L.parts);
 }
 
 cudaError_t launch_colpart(const LaunchCtx& L, cudaStream_t st) {

@@ -97,7 +97,7 @@ struct meq_state {
   std::vector<MatInfo> mats;
   std::vector<Group> groups;
   int64_t total_chunks = 0, total_hchunks = 0, total_tiles = 0, total_rblks = 0, total_slabs = 0, total_xblks = 0,
-          total_folds = 0, max_parts = 0;
+          total_folds = 0, max_parts = 0, total_rcs = 0;
   int64_t mom_floats = 0, u_halves = 0, vec_floats = 0, parts_floats = 0;
   char* arena = nullptr;
   int64_t arena_bytes = 0;
@@ -228,6 +228,23 @@ bool valid_shapes(const meq_shape* shapes, int n, std::string* why) {
 
 float pow2_round(double x) { return static_cast<float>(std::ldexp(1.0, static_cast<int>(std::lround(std::log2(std::max(x, 1.0)))))); }
 
+// Rows per block of the one-pass form over the remaining 2D parameters: at
+// least kColSlab (the partial sums are sized for that), and as many more as
+// it takes for the blocks, one per SM at a time, to fill whole waves.
+int64_t rowcol_slab_rows(const meq_state* st) {
+  auto blocks = [&](int64_t rows) {
+    int64_t b = 0;
+    for (int i = 0; i < st->n; ++i)
+      if (st->kinds[i] == KIND_TWO_SIDED && st->shapes[i].cols <= kRowColMax) b += (st->shapes[i].rows + rows - 1) / rows;
+    return b;
+  };
+  int64_t rows = kColSlab;
+  const int64_t waves = st->num_sms > 0 ? blocks(rows) / st->num_sms : 0;
+  if (waves > 0)
+    while (blocks(rows) > waves * st->num_sms && rows < 4 * kColSlab) rows += kRowColThreads / 32;
+  return rows;
+}
+
 // Builds the whole plan (shapes -> groups, offsets, sizes). Allocation-free.
 void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* off_vec4, int64_t* off_cpart,
           int64_t* off_partials, int64_t* off_counters, int64_t* off_x0s, int64_t* off_stats, int64_t* off_step,
@@ -270,7 +287,8 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     st->groups[g].mats.push_back(i);
   }
   int64_t mom = 0, u = 0, vec = 0, parts = 0, chunks = 0, hchunks = 0, tiles = 0, rblks = 0, slabs = 0, xblks = 0;
-  int64_t folds = 0, max_parts = 0;
+  int64_t folds = 0, max_parts = 0, rcs = 0;
+  const int64_t slab_rows = rowcol_slab_rows(st);
   int64_t mslots = 0;
   for (auto& G : st->groups) {
     G.mbase = mslots;
@@ -298,6 +316,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     M.rblk_begin = rblks;
     M.slab_begin = slabs;
     M.fold_begin = folds;
+    M.rc_begin = rcs;
     if (M.kind == KIND_HIDDEN) {
       const Group& G = st->groups[M.group];
       M.un = G.un;
@@ -313,12 +332,15 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
       max_parts = std::max(max_parts, 2 * ((M.l + 255) / 256) * M.s + (M.s + 31) / 32 * M.l);
     } else {
       M.un = M.n;
-      rblks += (M.m + 7) / 8;  // 8 rows (warps) per block
+      const bool one_pass = M.kind == KIND_TWO_SIDED && M.n <= kRowColMax;
+      M.slab_rows = one_pass ? slab_rows : kColSlab;
+      if (one_pass) rcs += (M.m + M.slab_rows - 1) / M.slab_rows;
+      else rblks += (M.m + 7) / 8;  // 8 rows (warps) per block
       if (M.kind == KIND_TWO_SIDED) {
         const int64_t ns = (M.m + kColSlab - 1) / kColSlab;
         M.cpart_off = parts;
         parts += round_up(ns * M.n, 64);
-        slabs += ns * ((M.n + 255) / 256);  // blocks: slab x 256-column chunk
+        if (!one_pass) slabs += ns * ((M.n + 255) / 256);  // blocks: slab x 256-column chunk
         folds += (M.m + kThreads - 1) / kThreads + (M.n + kFoldCols - 1) / kFoldCols;
         max_parts = std::max(max_parts, ns * M.n);
       }
@@ -327,7 +349,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
   st->mom_floats = mom, st->u_halves = u, st->vec_floats = vec, st->parts_floats = parts;
   st->total_chunks = chunks, st->total_hchunks = hchunks, st->total_tiles = tiles, st->total_xblks = xblks;
   st->total_rblks = rblks, st->total_slabs = slabs;
-  st->total_folds = folds, st->max_parts = max_parts;
+  st->total_folds = folds, st->max_parts = max_parts, st->total_rcs = rcs;
   st->persistent_bytes = 0;
   for (int i = 0; i < n; ++i) st->persistent_bytes += 4 * st->mats[i].m * st->mats[i].n;
 
@@ -875,8 +897,9 @@ meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n
   C.total_rblks = st->total_rblks;
   C.total_slabs = st->total_slabs;
   C.total_folds = st->total_folds;
+  C.total_rcs = st->total_rcs;
   C.fold = st->max_parts > kFoldMinParts ? 1 : 0;
-  st->kernels_per_step = (st->n_hidden ? 2 : 0) + (st->total_rblks ? 1 : 0) +
+  st->kernels_per_step = (st->n_hidden ? 2 : 0) + (st->total_rcs ? 1 : 0) + (st->total_rblks ? 1 : 0) +
                          (st->total_slabs ? 1 : 0) + C.fold +
                          2 + static_cast<int>(st->gemm.size());
   st->step_host.assign(static_cast<size_t>(st->step_bytes), 0);
@@ -946,6 +969,10 @@ static meq_status enqueue_kernels(meq_state* st, cudaStream_t s, cudaEvent_t* ev
       e = launch_x0norm(C, s);
       if (e != cudaSuccess) return cuda_fail(st, e, "x0norm launch");
     }
+  }
+  if (st->total_rcs) {
+    e = launch_rowcol(C, s);
+    if (e != cudaSuccess) return cuda_fail(st, e, "rowcol launch");
   }
   if (st->total_rblks) {
     e = launch_rows(C, s);

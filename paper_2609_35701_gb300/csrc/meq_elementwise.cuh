@@ -9,7 +9,9 @@ constexpr int kThreads = 256;      // block size of most kernels
 constexpr int64_t kChunk = 4096;   // elements per momentum / apply block
 constexpr int kCastTile = 64;      // X_0 cast tile (64 x 64 of W)
 constexpr int kFinThreads = 512;   // finalize block size (two blocks per SM)
-constexpr int kColSlab = 128;      // rows per block of the remaining-2D column pass
+constexpr int kColSlab = 128;      // rows per block of the remaining-2D column pass (at least, in the one-pass form)
+constexpr int kRowColMax = 1024;   // longest row of the one-pass form: 32 values per lane, and as many column sums
+constexpr int kRowColThreads = 512;
 // The partial sums get a launch of their own (fold_kernel) when an entry has
 // more of them than this; below, one finalize block reads them in less time
 // than a launch takes. Statistics phase, one block per entry -> fold, then
@@ -49,7 +51,7 @@ struct LaunchCtx {
   MatStats* stats;
   unsigned long long* dircount;  // per entry: Eq. (11) row choices, column choices
   int* nonfinite;                // 1 + index of the first entry whose momentum had a non-finite norm, or 0
-  int64_t total_chunks, total_hchunks, total_tiles, total_rblks, total_slabs, total_xblks, total_folds;
+  int64_t total_chunks, total_hchunks, total_tiles, total_rblks, total_slabs, total_xblks, total_folds, total_rcs;
   int fold;                      // 1: the partial sums are folded by a launch of their own before finalize
   int n_hidden;
 };
@@ -59,8 +61,9 @@ constexpr int KIND_HIDDEN = 0, KIND_TWO_SIDED = 1, KIND_VECTOR = 2;
 cudaError_t launch_momentum_norm(const LaunchCtx& L, cudaStream_t st);
 cudaError_t launch_momentum_x0(const LaunchCtx& L, cudaStream_t st);  // fused momentum + bf16 X_0
 cudaError_t launch_x0norm(const LaunchCtx& L, cudaStream_t st);       // 1 / ||H||_F from its partials
-cudaError_t launch_rows(const LaunchCtx& L, cudaStream_t st);      // remaining 2D + vectors
-cudaError_t launch_colpart(const LaunchCtx& L, cudaStream_t st);   // remaining 2D
+cudaError_t launch_rowcol(const LaunchCtx& L, cudaStream_t st);    // remaining 2D, rows up to kRowColMax
+cudaError_t launch_rows(const LaunchCtx& L, cudaStream_t st);      // remaining 2D with longer rows, vectors
+cudaError_t launch_colpart(const LaunchCtx& L, cudaStream_t st);   // remaining 2D with longer rows
 cudaError_t launch_cast_x0(const LaunchCtx& L, bool fp16, cudaStream_t st);
 cudaError_t launch_stats(const LaunchCtx& L, cudaStream_t st);  // [fold and] finalize of the fused statistics
 cudaError_t launch_apply(const LaunchCtx& L, cudaStream_t st);

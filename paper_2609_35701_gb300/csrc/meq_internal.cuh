@@ -50,8 +50,10 @@ struct MatInfo {
   int64_t vec_off;       // float offset of r (m), c (n) and scale (max(m, n))
   int64_t chunk_begin;   // first apply chunk (all kinds)
   int64_t hchunk_begin;  // first momentum-and-norm chunk (hidden weights only)
-  int64_t rblk_begin;    // first 8-row block of the row pass (remaining 2D and vectors)
-  int64_t slab_begin;    // first row slab of the column pass (remaining 2D only)
+  int64_t rblk_begin;    // first 8-row block of the row pass (remaining 2D with long rows, vectors)
+  int64_t slab_begin;    // first row slab of the column pass (remaining 2D with long rows)
+  int64_t rc_begin;      // first slab of the one-pass form (remaining 2D with rows up to kRowColMax)
+  int64_t slab_rows;     // rows per slab (remaining 2D)
   int64_t tile_begin;    // first cast tile (hidden weights only)
   int64_t xblk_begin;    // first momentum-and-X_0 block (hidden weights only)
   int64_t fold_begin;    // first block of the fold of the partial sums (hidden weights and remaining 2D)

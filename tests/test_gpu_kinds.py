@@ -103,6 +103,20 @@ def test_folded_statistics(meq, shapes, kinds):
     run_kinds(meq, W.custom_workload(shapes, pattern="both", seed=53, kinds=kinds), 2)
 
 
+@pytest.mark.parametrize("n", [1, 3, 4, 31, 128, 255, 256, 260, 512, 513, 767, 768, 1000, 1021, 1024])
+def test_remaining_2d_in_one_pass(meq, n):
+    """Rows of up to 1024 entries: every width class and its edges, aligned and not, with slabs
+    shorter and longer than a block's 16 warps."""
+    rows = [1, 15, 129, 300]
+    kinds = [O.REMAINING_2D] * len(rows)
+    run_kinds(meq, W.custom_workload([(m, n) for m in rows], pattern="both", seed=n, kinds=kinds), 2)
+
+
+def test_remaining_2d_slabs_of_whole_waves(meq):
+    shapes = [(27000, 20), (130, 20)]
+    run_kinds(meq, W.custom_workload(shapes, pattern="both", seed=59, kinds=[O.REMAINING_2D] * 2), 2)
+
+
 def test_rows_columns_and_vectors_at_the_rms_threshold(meq):
     """The reading of Eq. (9) for rows / columns whose RMS does not exceed
     delta (scale 0, no update from them), on the branches without
