@@ -19,7 +19,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmeq.so")
 SOURCES = ["ns_gemm.cu", "elementwise.cu", "meq_api.cu", "noalloc.cu"]
-HEADERS = ["meq_internal.cuh", "meq_elementwise.cuh"]
+HEADERS = ["meq_internal.cuh", "meq_elementwise.cuh", "meq_stats.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE]
 

@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "meq_elementwise.cuh"
+#include "meq_stats.cuh"
 
 namespace meq {
 namespace {
@@ -649,21 +650,6 @@ __global__ void __launch_bounds__(kThreads) cast_x0_kernel(const MatInfo* __rest
 }
 
 // ----------------------------------------------------------------- statistics
-// sum_{k0 <= k < k1} p[k * stride] with eight independent partial sums (term
-// k0 + i goes to partial i % 8) so that the loads overlap; fixed order.
-__device__ __forceinline__ float strided_sum8(const float* __restrict__ p, int64_t k0, int64_t k1, int64_t stride) {
-  float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  int64_t k = k0;
-  for (; k + 8 <= k1; k += 8) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) a8[u] += p[(k + u) * stride];
-  }
-#pragma unroll
-  for (int u = 0; u < 7; ++u)
-    if (k + u < k1) a8[u] += p[(k + u) * stride];
-  return ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
-}
-
 // The vectors of one entry that come from partial sums: r and c of a hidden
 // weight (NS rows and columns, swapped for a transposed one), c of a
 // remaining 2D parameter.
@@ -727,132 +713,15 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(const MatInfo* __restric
     return;
   }
   const FoldVec v = fold_vec(M, which, parts, rvec, cvec);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t j0 = (lb - (which ? first : 0)) * kFoldCols;
-  const int64_t per = (v.count + 7) / 8;
-  const int64_t k0 = w * per, k1 = min(k0 + per, v.count);
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  pdl_wait_predecessor();
-  const float* p = v.parts + j0 + lane;
-  if (j0 + kFoldCols <= v.len) {
-    int64_t k = k0;
-    for (; k + 4 <= k1; k += 4) {
-      float x[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[i][u] = p[(k + i) * v.len + 32 * u];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] += x[i][u];
-    }
-    for (; k < k1; ++k)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] += p[k * v.len + 32 * u];
-  } else {
-    for (int64_t k = k0; k < k1; ++k)
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (j0 + lane + 32 * u < v.len) acc[u] += p[k * v.len + 32 * u];
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) sh[w][lane + 32 * u] = acc[u];
-  __syncthreads();
   const int t = threadIdx.x;
+  pdl_wait_predecessor();
+  const float sum = fold_block(v.parts, v.count, v.len, j0, sh);
   if (t < kFoldCols && j0 + t < v.len) {
-    const float sum = ((sh[0][t] + sh[1][t]) + (sh[2][t] + sh[3][t])) + ((sh[4][t] + sh[5][t]) + (sh[6][t] + sh[7][t]));
     const float rms = sqrtf(sum * v.inv);
     v.dst[j0 + t] = rms;
     if (M.kind == KIND_TWO_SIDED) tvec[M.vec_off + j0 + t] = rms > sc->eps ? 1.0f / rms : 0.f;
   }
-}
-
-// K block sums at once, one barrier for all of them: every warp adds the
-// warps' sums up itself (the same tree in each, so all threads get the same
-// values). sh holds 32 * K floats that no other call of the block uses.
-template <int K>
-__device__ __forceinline__ void block_sum_multi(float (&v)[K], float* sh) {
-  const unsigned FULL = 0xffffffffu;
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) sh[32 * k + w] = v[k];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    v[k] = l < static_cast<int>(blockDim.x >> 5) ? sh[32 * k + l] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
-  }
-}
-
-// r (length la) and c (length lb) of one entry, spread over the block. Up to
-// kStatRegs values per thread are read once and kept in registers for both
-// passes of the CVs and for the scale vector (3 round trips to L2 otherwise).
-constexpr int kStatRegs = 32;
-struct StatVecs {
-  const float *a, *b;
-  int64_t la, lb;
-  int nk;              // values per thread when they are kept in registers, else 0
-  float x[kStatRegs];  // entry threadIdx.x + k * kFinThreads of a followed by b
-
-  __device__ __forceinline__ void load() {
-    const int64_t len = la + lb;
-    nk = len <= static_cast<int64_t>(kStatRegs) * kFinThreads ? static_cast<int>((len + kFinThreads - 1) / kFinThreads) : 0;
-#pragma unroll
-    for (int k = 0; k < kStatRegs; ++k) {
-      if (k >= nk) break;
-      const int i = static_cast<int>(threadIdx.x) + k * kFinThreads;
-      x[k] = i < static_cast<int>(la) ? a[i] : (i < static_cast<int>(len) ? b[i - static_cast<int>(la)] : 0.f);
-    }
-  }
-  // f(side, index, value) for every entry of this thread
-  template <typename F>
-  __device__ __forceinline__ void each(F f) const {
-    if (nk) {
-      const int na = static_cast<int>(la), n = static_cast<int>(la + lb);
-#pragma unroll
-      for (int k = 0; k < kStatRegs; ++k) {
-        if (k >= nk) break;
-        const int i = static_cast<int>(threadIdx.x) + k * kFinThreads;
-        if (i < n) f(i < na ? 0 : 1, i < na ? i : i - na, x[k]);
-      }
-    } else {
-#pragma unroll 8
-      for (int64_t i = threadIdx.x; i < la; i += kFinThreads) f(0, i, a[i]);
-#pragma unroll 8
-      for (int64_t i = threadIdx.x; i < lb; i += kFinThreads) f(1, i, b[i]);
-    }
-  }
-};
-
-// Two-pass fp32 CVs of Eq. (8) of r and c over their entries above delta,
-// both at once: the mean pass, then the squared deviations.
-__device__ __forceinline__ void block_cv2(const StatVecs& v, float delta, float* sh, float* ga, float* gb) {
-  float p[4] = {0.f, 0.f, 0.f, 0.f};  // count and sum over r, then over c
-  v.each([&](int side, int64_t, float x) {
-    const bool in = x > delta, ia = in && side == 0, ib = in && side == 1;
-    p[0] += ia ? 1.f : 0.f, p[1] += ia ? x : 0.f;
-    p[2] += ib ? 1.f : 0.f, p[3] += ib ? x : 0.f;
-  });
-  block_sum_multi<4>(p, sh);
-  const float mean_a = p[0] > 0.f ? p[1] / p[0] : 0.f;
-  const float mean_b = p[2] > 0.f ? p[3] / p[2] : 0.f;
-  float q[2] = {0.f, 0.f};
-  v.each([&](int side, int64_t, float x) {
-    const float d = x - (side == 0 ? mean_a : mean_b);
-    q[0] += x > delta && side == 0 ? d * d : 0.f;
-    q[1] += x > delta && side == 1 ? d * d : 0.f;
-  });
-  block_sum_multi<2>(q, sh + 4 * 32);
-  *ga = p[0] > 0.f ? sqrtf(q[0] / p[0]) / mean_a : 0.f;
-  *gb = p[2] > 0.f ? sqrtf(q[1] / p[2]) / mean_b : 0.f;
 }
 
 // Statistics and normalisation scales, one block per parameter.

@@ -11,24 +11,27 @@
 // library holds until the process exits.
 //
 // It sums squares over blocks of 32 rows x 1024 columns, folds the partials
-// with one thread per row and per column (blocks in order), and forms the
-// CVs in two passes, all in
-// fp32 like the full step's statistics, so results agree with meq_read_stats
-// up to fp32 summation order. The same kernels, given scratch that the caller
-// allocated, give the first point of the CV trajectory (meq_ns_cv_trajectory).
+// with the step's own fold (small matrices: in the last kernel), and forms the
+// CVs in two passes, all in fp32 like the full step's statistics, so results
+// agree with meq_read_stats up to fp32 summation order. The same kernels, given
+// scratch that the caller allocated, give the first point of the CV trajectory
+// (meq_ns_cv_trajectory).
+//
+// Bound by the one read of U. 4096 x 11008 (180 MB, 26.6 us at the measured
+// copy rate): 98 us with scalar loads, one thread per column of the fold, a
+// CV block that went to L2 six times, and full launch gaps; 41 us now.
 #include <mutex>
 #include <string>
 
 #include "../../include/meq.h"
-#include "meq_elementwise.cuh"
+#include "meq_stats.cuh"
 
 namespace {
 
-constexpr int kNaThreads = 256;
+using namespace meq;
+
 constexpr int kNaSlab = 32;        // rows per block
 constexpr int kNaChunk = 1024;     // columns per block (four per thread)
-constexpr int kNaFoldThreads = 256;
-constexpr int kNaFinThreads = 1024;
 constexpr int kMaxDevices = 64;
 
 // 8 MiB of scratch: the row partial sums of squares (ceil(cols / 1024) x
@@ -39,29 +42,18 @@ static __device__ __align__(256) float g_stats_scratch[kScratchFloats];
 std::mutex g_setup_mu;
 float* g_scratch_addr[kMaxDevices] = {nullptr};
 
-__device__ __forceinline__ float na_block_sum_f32(float v, float* sh) {
-  const unsigned FULL = 0xffffffffu;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float r = 0.f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += sh[i];
-    sh[0] = r;
-  }
-  __syncthreads();
-  return sh[0];
-}
-
 // One block per 32-row slab (blockIdx.x) and 1024-column chunk (blockIdx.y):
 // the slab's column partial sums of squares over the chunk's columns, and
-// the chunk's partial sums of squares of the slab's rows.
-__global__ void __launch_bounds__(kNaThreads) na_stats_kernel(const float* __restrict__ U, int64_t m, int64_t n,
-                                                              float* __restrict__ scratch) {
-  __shared__ float shr[kNaThreads / 32][32];
+// the chunk's partial sums of squares of the slab's rows. kVec: rows are a
+// multiple of 4 long and U is 16-byte aligned, so a thread takes four
+// neighbouring columns, eight 16-byte loads in flight (else four columns 256
+// apart, one after the other).
+template <bool kVec>
+__global__ void __launch_bounds__(kThreads, 3) na_stats_kernel(const float* __restrict__ U, int64_t m, int64_t n,
+                                                               float* __restrict__ scratch) {
+  pdl_allow_dependents();
+  pdl_wait_predecessor();
+  __shared__ float shr[kThreads / 32][32];
   const int64_t slab = blockIdx.x, chunk = blockIdx.y;
   const int64_t r0 = slab * kNaSlab;
   const int nr = static_cast<int>(m - r0 < kNaSlab ? m - r0 : kNaSlab);
@@ -73,18 +65,42 @@ __global__ void __launch_bounds__(kNaThreads) na_stats_kernel(const float* __res
   float racc[kNaSlab];
 #pragma unroll
   for (int r = 0; r < kNaSlab; ++r) racc[r] = 0.f;
-  for (int64_t c = chunk * kNaChunk + threadIdx.x; c < c1; c += kNaThreads) {
-    float cacc = 0.f;
+  if (kVec) {
+    const int64_t c = chunk * kNaChunk + 4 * threadIdx.x;
+    if (c < c1) {
+      float4 cacc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int r = 0; r < kNaSlab; ++r) {
-      if (r < nr) {
-        const float u = Us[r * n + c];
-        const float u2 = u * u;
-        cacc += u2;
-        racc[r] += u2;
+      for (int rb = 0; rb < kNaSlab; rb += 8) {
+        float4 u[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          u[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (rb + i < nr) u[i] = __ldcs(reinterpret_cast<const float4*>(Us + (rb + i) * n + c));
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float x = u[i].x * u[i].x, y = u[i].y * u[i].y, z = u[i].z * u[i].z, w = u[i].w * u[i].w;
+          cacc.x += x, cacc.y += y, cacc.z += z, cacc.w += w;
+          racc[rb + i] = (x + y) + (z + w);
+        }
       }
+      // the scratch's column part need not be 16-byte aligned (it follows nchunks * m floats)
+      cp[c] = cacc.x, cp[c + 1] = cacc.y, cp[c + 2] = cacc.z, cp[c + 3] = cacc.w;
     }
-    cp[c] = cacc;
+  } else {
+    for (int64_t c = chunk * kNaChunk + threadIdx.x; c < c1; c += kThreads) {
+      float cacc = 0.f;
+#pragma unroll
+      for (int r = 0; r < kNaSlab; ++r) {
+        if (r < nr) {
+          const float u = Us[r * n + c];
+          const float u2 = u * u;
+          cacc += u2;
+          racc[r] += u2;
+        }
+      }
+      cp[c] = cacc;
+    }
   }
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -102,95 +118,77 @@ __global__ void __launch_bounds__(kNaThreads) na_stats_kernel(const float* __res
   __syncthreads();
   if (threadIdx.x < nr) {
     float s = 0.f;
-    for (int i = 0; i < kNaThreads / 32; ++i) s += shr[i][threadIdx.x];
+    for (int i = 0; i < kThreads / 32; ++i) s += shr[i][threadIdx.x];
     rowss[r0 + threadIdx.x] = s;
   }
 }
 
-// r (Eq. (7)) from the row partials and c from the column partials, one
-// thread per row / column, each summing its partials in block order; the
-// row sums of squares are kept (first row of the scratch) for the CV kernel.
-__global__ void __launch_bounds__(kNaFoldThreads) na_fold_kernel(int64_t m, int64_t n, float* __restrict__ scratch,
-                                                                 float* __restrict__ r, float* __restrict__ c) {
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * kNaFoldThreads + threadIdx.x;
+// r (Eq. (7)) from the row partials and c from the column partials, blocks of
+// kFoldCols rows first, then of columns; the row sums of squares are kept
+// (first row of the scratch) for the CV kernel.
+__global__ void __launch_bounds__(kThreads) na_fold_kernel(int64_t m, int64_t n, float* __restrict__ scratch,
+                                                           float* __restrict__ r, float* __restrict__ c) {
+  pdl_allow_dependents();
+  pdl_wait_predecessor();
+  __shared__ float sh[kThreads / 32][kFoldCols];
   const int64_t nslabs = (m + kNaSlab - 1) / kNaSlab;
   const int64_t nchunks = (n + kNaChunk - 1) / kNaChunk;
-  const float* cpart = scratch + nchunks * m;
-  if (t < m) {
-    float acc = 0.f;
-    for (int64_t k = 0; k < nchunks; ++k) acc += scratch[k * m + t];
-    scratch[t] = acc;  // only this thread reads or writes row t's partials
-    r[t] = sqrtf(acc * (1.0f / static_cast<float>(n)));
-  }
-  if (t < n) {
-    float acc = 0.f;
-    int64_t k = 0;
-    for (; k + 4 <= nslabs; k += 4) {  // four loads in flight, added in slab order
-      const float a0 = cpart[k * n + t], a1 = cpart[(k + 1) * n + t];
-      const float a2 = cpart[(k + 2) * n + t], a3 = cpart[(k + 3) * n + t];
-      acc += a0;
-      acc += a1;
-      acc += a2;
-      acc += a3;
-    }
-    for (; k < nslabs; ++k) acc += cpart[k * n + t];
-    c[t] = sqrtf(acc * (1.0f / static_cast<float>(m)));
+  const int64_t row_blocks = (m + kFoldCols - 1) / kFoldCols;
+  const bool rows = blockIdx.x < row_blocks;
+  const int64_t len = rows ? m : n;
+  const int64_t j0 = (rows ? blockIdx.x : blockIdx.x - row_blocks) * static_cast<int64_t>(kFoldCols);
+  const float sum = fold_block(rows ? scratch : scratch + nchunks * m, rows ? nchunks : nslabs, len, j0, sh);
+  const int64_t j = j0 + threadIdx.x;
+  if (threadIdx.x < kFoldCols && j < len) {
+    if (rows) scratch[j] = sum;  // only this block reads or writes these rows' partials
+    (rows ? r : c)[j] = sqrtf(sum * (1.0f / static_cast<float>(rows ? n : m)));
   }
 }
 
 // gamma_r, gamma_c (Eq. (8), over entries > delta) and the side (Eq. (11)),
 // all fp32, in one block. With frob set, r and c are first divided by
 // ||U||_F (from the row sums of squares, fixed order), so that they and the
-// threshold describe X = U / ||U||_F; a zero U gives zeros.
-__global__ void __launch_bounds__(kNaFinThreads) na_cv_kernel(int64_t m, int64_t n, float delta, float tie_atol, int frob,
-                                                              const float* __restrict__ scratch, float* __restrict__ r,
-                                                              float* __restrict__ c, double* __restrict__ gammas,
-                                                              int* __restrict__ direction) {
-  __shared__ float shf[32];
-  if (frob) {
-    float tot = 0.f;
-    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) tot += scratch[i];
-    tot = na_block_sum_f32(tot, shf);
-    const float inv = tot > 0.f ? 1.0f / sqrtf(tot) : 0.f;
-    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) r[i] *= inv;
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) c[j] *= inv;
+// threshold describe X = U / ||U||_F; a zero U gives zeros. Without a fold
+// launch before it, the block folds the partials itself.
+__global__ void __launch_bounds__(kFinThreads) na_cv_kernel(int64_t m, int64_t n, float delta, float tie_atol, int frob,
+                                                            int folded, float* __restrict__ scratch,
+                                                            float* __restrict__ r, float* __restrict__ c,
+                                                            double* __restrict__ gammas, int* __restrict__ direction) {
+  pdl_allow_dependents();
+  pdl_wait_predecessor();
+  __shared__ float shf[7 * 32];
+  if (!folded) {
+    const int64_t nslabs = (m + kNaSlab - 1) / kNaSlab;
+    const int64_t nchunks = (n + kNaChunk - 1) / kNaChunk;
+    const float* cpart = scratch + nchunks * m;
+    for (int64_t i = threadIdx.x; i < m; i += kFinThreads) {
+      const float s = strided_sum8(scratch + i, 0, nchunks, m);
+      scratch[i] = s;  // only this thread reads or writes row i's partials
+      r[i] = sqrtf(s * (1.0f / static_cast<float>(n)));
+    }
+    for (int64_t j = threadIdx.x; j < n; j += kFinThreads)
+      c[j] = sqrtf(strided_sum8(cpart + j, 0, nslabs, n) * (1.0f / static_cast<float>(m)));
     __syncthreads();
   }
-  float gam[2];
-  for (int side = 0; side < 2; ++side) {
-    const float* v = side == 0 ? r : c;
-    const int64_t len = side == 0 ? m : n;
-    float cnt = 0.f, sum = 0.f;
-    for (int64_t i = threadIdx.x; i < len; i += blockDim.x) {
-      const float x = v[i];
-      if (x > delta) cnt += 1.f, sum += x;
-    }
-    cnt = na_block_sum_f32(cnt, shf);
-    sum = na_block_sum_f32(sum, shf);
-    const float mean = cnt > 0.f ? sum / cnt : 0.f;
-    float var = 0.f;
-    for (int64_t i = threadIdx.x; i < len; i += blockDim.x) {
-      const float x = v[i];
-      if (x > delta) var += (x - mean) * (x - mean);
-    }
-    var = na_block_sum_f32(var, shf);
-    gam[side] = cnt > 0.f ? sqrtf(var / cnt) / mean : 0.f;
+  if (frob) {
+    float tot[1] = {0.f};
+    for (int64_t i = threadIdx.x; i < m; i += kFinThreads) tot[0] += scratch[i];
+    block_sum_multi<1>(tot, shf + 6 * 32);
+    const float inv = tot[0] > 0.f ? 1.0f / sqrtf(tot[0]) : 0.f;
+    for (int64_t i = threadIdx.x; i < m; i += kFinThreads) r[i] *= inv;
+    for (int64_t j = threadIdx.x; j < n; j += kFinThreads) c[j] *= inv;
+    __syncthreads();
   }
+  StatVecs vecs;
+  vecs.a = r, vecs.b = c, vecs.la = m, vecs.lb = n;
+  vecs.load();
+  float g0, g1;
+  block_cv2(vecs, delta, shf, &g0, &g1);
   if (threadIdx.x == 0) {
-    gammas[0] = static_cast<double>(gam[0]);
-    gammas[1] = static_cast<double>(gam[1]);
-    *direction = gam[0] >= gam[1] - tie_atol ? 0 : 1;
+    gammas[0] = static_cast<double>(g0);
+    gammas[1] = static_cast<double>(g1);
+    *direction = g0 >= g1 - tie_atol ? 0 : 1;
   }
-}
-
-// Plain launch (no attributes) that returns this launch's own status.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_plain(void (*kernel)(KArgs...), dim3 grid, unsigned block, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(block);
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 // Device address of the scratch array on the current device, looked up once
@@ -231,17 +229,22 @@ cudaError_t launch_row_col_stats(const float* U, int64_t rows, int64_t cols, flo
   const int64_t nslabs = (rows + kNaSlab - 1) / kNaSlab;
   const int64_t nchunks = (cols + kNaChunk - 1) / kNaChunk;
   *failed = "statistics launch";
-  cudaError_t e = launch_plain(na_stats_kernel, dim3(static_cast<unsigned>(nslabs), static_cast<unsigned>(nchunks)),
-                               kNaThreads, st, U, rows, cols, scratch);
+  const bool vec = (cols & 3) == 0 && (reinterpret_cast<uintptr_t>(U) & 15u) == 0;
+  cudaError_t e = launch_pdl(vec ? na_stats_kernel<true> : na_stats_kernel<false>,
+                             dim3(static_cast<unsigned>(nslabs), static_cast<unsigned>(nchunks)), dim3(kThreads), 0, st,
+                             1, U, rows, cols, scratch);
   if (e != cudaSuccess) return e;
-  *failed = "fold launch";
-  const int64_t len = rows > cols ? rows : cols;
-  e = launch_plain(na_fold_kernel, dim3(static_cast<unsigned>((len + kNaFoldThreads - 1) / kNaFoldThreads)),
-                   kNaFoldThreads, st, rows, cols, scratch, r, c);
-  if (e != cudaSuccess) return e;
+  const int folded = row_col_stats_scratch_floats(rows, cols) > kFoldMinParts ? 1 : 0;
+  if (folded) {
+    *failed = "fold launch";
+    const int64_t blocks = (rows + kFoldCols - 1) / kFoldCols + (cols + kFoldCols - 1) / kFoldCols;
+    e = launch_pdl(na_fold_kernel, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, st, 1, rows, cols, scratch, r,
+                   c);
+    if (e != cudaSuccess) return e;
+  }
   *failed = "CV launch";
-  return launch_plain(na_cv_kernel, dim3(1), kNaFinThreads, st, rows, cols, eps, tie_atol, frob,
-                      static_cast<const float*>(scratch), r, c, gammas, direction);
+  return launch_pdl(na_cv_kernel, dim3(1), dim3(kFinThreads), 0, st, 1, rows, cols, eps, tie_atol, frob, folded, scratch,
+                    r, c, gammas, direction);
 }
 
 }  // namespace meq

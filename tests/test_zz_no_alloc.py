@@ -79,6 +79,39 @@ def test_noalloc_stats_match_oracle_and_step_twice_in_a_row():
     opt.close()
 
 
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 4096), (4096, 1), (31, 1020), (33, 1028), (64, 127), (32, 1024), (97, 1025),
+                                 (256, 256), (1000, 3001), (20000, 36)])
+@pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "one_float_in"])
+def test_noalloc_stats_edges(m, n, shift):
+    """Edges of the 32 x 1024 blocks, of 16-byte rows and bases, of the fold (with and without its own
+    launch) and of what the CV block keeps in registers; CUDA stream capture and replay of the last."""
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import torch
+
+    from paper_2609_35701_gb300 import meq
+
+    gen = torch.Generator().manual_seed(m * 7919 + n)
+    U_h = torch.randn(m, n, generator=gen) * torch.exp(torch.empty(m, 1).uniform_(-2.0, 2.0, generator=gen))
+    flat = torch.zeros(m * n + 4, device="cuda")
+    U = flat[shift:shift + m * n].view(m, n)
+    U.copy_(U_h)
+    r, c, g, d = _outputs(torch, m, n)
+    assert meq.row_col_stats_noalloc(U, r, c, g, d, eps=EPS, tie_atol=TIE) == 0
+    torch.cuda.synchronize()
+    _check_against_oracle(U_h.double().numpy(), r, c, g, d, (m, n))
+    want = [t.clone() for t in (r, c, g, d)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        assert meq.row_col_stats_noalloc(U, r, c, g, d, eps=EPS, tie_atol=TIE) == 0
+    for t in (r, c, g):
+        t.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(want, (r, c, g, d)))
+
+
 def test_noalloc_llama7b_shapes_and_size_limit():
     """The Llama-7B hidden shapes (the largest the fixed scratch takes for
     these widths), timed with CUDA events; a shape just past the limit is
