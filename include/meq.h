@@ -251,8 +251,8 @@ meq_status meq_debug_corrupt_canary(meq_state* st, int index);
  * every later iterate, are compared with eps after the normalisation. h:
  * device fp32, rows x cols row-major, 16-byte aligned, read only. gamma_r,
  * gamma_c: host arrays of steps + 1 doubles. steps: 0..32. Synchronous;
- * allocates and frees its own device scratch (about rows x cols x 4 bytes
- * plus one optimizer state per k), so concurrent calls do not share memory;
+ * allocates and frees its own device scratch (the statistics' partial sums
+ * and one optimizer state), so concurrent calls do not share memory;
  * every shape meq_init_state accepts is accepted. Errors:
  * MEQ_ERR_INVALID_ARG (NULL, misaligned, bad sizes), MEQ_ERR_OOM, or the
  * error of the step it runs (text in meq_last_error(NULL)). */

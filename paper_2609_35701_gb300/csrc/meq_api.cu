@@ -92,6 +92,7 @@ struct meq_state {
   std::vector<int> kinds;                     // meq_kind per entry
   int n_hidden = 0;
   meq_options opt{};
+  bool trajectory = false;                    // statistics after every NS iteration
   int device = 0;
   int num_sms = 0;
   std::vector<MatInfo> mats;
@@ -491,7 +492,7 @@ int64_t pair_saving(const Group& G) {
 }
 
 // The products of one group, in order.
-std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs) {
+std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, bool trajectory) {
   std::vector<NsOp> ops;
   const int K = o.ns_steps;
   const bool fused = o.ns_x0_fused != 0;
@@ -548,15 +549,19 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs) {
       ops.push_back(c);
       mul = BUF_A;
     }
-    NsOp up;  // X' = P X
-    up.mode = last ? MODE_XLAST : MODE_DENSE;
-    up.a = mul, up.b = cx, up.out = last ? BUF_NONE : nx, up.out_is_x = true;
-    up.in16 = dX(k);
-    up.out16 = last ? true : dX(k + step);
-    up.scale = last ? 1.0f / ak : G.alpha / ak;
-    up.minv_pow = per_matrix ? 1 : 0;
-    if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
-    ops.push_back(up);
+    for (int w = 0; w < 2; ++w) {  // U = P X, X' = P X
+      const bool u = w == 0;
+      if (u ? !(last || trajectory) : last) continue;
+      NsOp up;
+      up.mode = u ? MODE_XLAST : MODE_DENSE;
+      up.a = mul, up.b = cx, up.out = u ? BUF_NONE : nx, up.out_is_x = true;
+      up.in16 = dX(k);
+      up.out16 = u ? true : dX(k + step);
+      up.scale = u ? 1.0f / ak : G.alpha / ak;
+      up.minv_pow = per_matrix ? 1 : 0;
+      if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
+      ops.push_back(up);
+    }
     cur ^= 1;
     k += step;
   }
@@ -622,7 +627,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
   st->gemm_grid.clear();
   const int pair = st->opt.ns_cta_pair ? 2 : 1;
   int64_t saving = 0;
-  if (pairs_allowed(st->opt))
+  if (pairs_allowed(st->opt) && !st->trajectory)
     for (const Group& G : st->groups) saving += std::max<int64_t>(0, pair_saving(G)) * G.count;
   const bool pairs = saving >= kPairMinSaving;
   std::vector<int> which;                 // chain of each group: 0 plain, 1 with pairs
@@ -630,7 +635,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
   std::vector<NsOp> A, B;                 // the two chains' products (modes and formats; empty if unused)
   for (const Group& G : st->groups) {
     which.push_back(pairs && pair_saving(G) > 0 ? 1 : 0);
-    chain.push_back(ns_chain(st->opt, G, which.back() == 1));
+    chain.push_back(ns_chain(st->opt, G, which.back() == 1, st->trajectory));
     (which.back() ? B : A) = chain.back();
   }
   auto joint = [&](size_t i, size_t j) {
@@ -692,6 +697,9 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
 }  // namespace
 
 extern "C" {
+
+static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
+                             void* cuda_stream, bool trajectory, meq_state** out);
 
 void meq_default_options(meq_options* o) {
   if (!o) return;
@@ -761,6 +769,13 @@ meq_status meq_init_state(const meq_shape* shapes, int n, const meq_options* opt
 
 meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
                                 void* cuda_stream, meq_state** out) {
+  return init_state(shapes, kinds, n, opt, cuda_stream, false, out);
+}
+
+// trajectory: the NS plan gives U's statistics after every iteration
+// (meq_ns_cv_trajectory), not after the last one only.
+static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
+                             void* cuda_stream, bool trajectory, meq_state** out) {
   if (!out) return fail(nullptr, MEQ_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
   meq_options o;
@@ -772,13 +787,16 @@ meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return fail(nullptr, MEQ_ERR_UNSUPPORTED, std::string("no CUDA device: ") + cudaGetErrorString(e));
-  cudaDeviceProp prop;
-  e = cudaGetDeviceProperties(&prop, dev);
-  if (e != cudaSuccess) return fail(nullptr, MEQ_ERR_CUDA, std::string("cudaGetDeviceProperties: ") + cudaGetErrorString(e));
-  if (prop.major != 10 || prop.minor != 3)
+  int major = 0, minor = 0, smem_optin = 0, num_sms = 0;
+  e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return fail(nullptr, MEQ_ERR_CUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
+  if (major != 10 || minor != 3)
     return fail(nullptr, MEQ_ERR_UNSUPPORTED,
-                "this library is built for sm_103a (GB300); device is sm_" + std::to_string(prop.major) + std::to_string(prop.minor));
-  if (prop.sharedMemPerBlockOptin < static_cast<size_t>(ns_gemm_smem_bytes(o.ns_cta_pair ? 2 : 1)))
+                "this library is built for sm_103a (GB300); device is sm_" + std::to_string(major) + std::to_string(minor));
+  if (smem_optin < ns_gemm_smem_bytes(o.ns_cta_pair ? 2 : 1))
     return fail(nullptr, MEQ_ERR_UNSUPPORTED, "not enough opt-in shared memory per block");
   if (!get_encode()) return fail(nullptr, MEQ_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled is not available from the driver");
 
@@ -792,7 +810,8 @@ meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n
   if (kinds) st->kinds.assign(kinds, kinds + n);
   st->opt = o;
   st->device = dev;
-  st->num_sms = prop.multiProcessorCount;
+  st->num_sms = num_sms;
+  st->trajectory = trajectory;
 
   Layout L(o.debug_canaries != 0);
   int64_t off_mom, off_u, off_vec4, off_cpart, off_partials, off_counters, off_x0s, off_stats, off_step, off_err, off_mats,
@@ -1000,6 +1019,26 @@ static meq_status enqueue_kernels(meq_state* st, cudaStream_t s, cudaEvent_t* ev
   e = launch_apply(C, s);
   if (e != cudaSuccess) return cuda_fail(st, e, "apply launch");
   mark(5);
+  return MEQ_OK;
+}
+
+// The CV trajectory: momentum and X_0, then the NS products in order, the
+// statistics after every product that writes U (MatStats k of t for the k-th).
+static meq_status enqueue_trajectory(meq_state* st, MatStats* t, cudaStream_t s) {
+  LaunchCtx C = st->ctx;
+  const bool fused = st->opt.ns_x0_fused != 0;
+  cudaError_t e = fused ? launch_momentum_x0(C, s) : launch_momentum_norm(C, s);
+  if (e == cudaSuccess) e = fused ? launch_x0norm(C, s) : launch_cast_x0(C, iter_fp16(st->opt, 0), s);
+  if (e != cudaSuccess) return cuda_fail(st, e, "momentum launch");
+  C.stats = t;
+  for (size_t i = 0; i < st->gemm.size(); ++i) {
+    e = launch_ns_gemm(st->gemm[i], st->gemm_grid[i], st->opt.ns_cta_pair ? 2 : 1, s);
+    if (e != cudaSuccess) return cuda_fail(st, e, "ns_gemm launch");
+    if (st->gemm[i].g[0].mode != MODE_XLAST) continue;
+    e = launch_stats(C, s);
+    if (e != cudaSuccess) return cuda_fail(st, e, "finalize launch");
+    ++C.stats;
+  }
   return MEQ_OK;
 }
 
@@ -1322,54 +1361,53 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
   o.ns_steps = 1;
   if (!valid_options(o, &why)) return fail(nullptr, MEQ_ERR_INVALID_ARG, why);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  // scratch: W (rows x cols, left unchanged by lr = 0), r, c, the two CVs and
-  // the direction, then the statistics kernels' partial sums
-  const int64_t wb = round_up(rows * cols * 4, 256), rb = round_up(rows * 4, 256), cb = round_up(cols * 4, 256);
+  // scratch: r, c, the direction and the two CVs of k = 0, one MatStats per
+  // k >= 1, then the statistics kernels' partial sums
+  const int64_t rb = round_up(rows * 4, 256), cb = round_up(cols * 4, 256);
+  const int64_t tb = round_up(static_cast<int64_t>(sizeof(MatStats)) * (steps + 1), 256);
   const int64_t pb = round_up(row_col_stats_scratch_floats(rows, cols) * 4, 256);
   char* tmp = nullptr;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&tmp), static_cast<size_t>(wb + rb + cb + 256 + pb));
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&tmp), static_cast<size_t>(rb + cb + tb + pb));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, MEQ_ERR_OOM, "scratch allocation failed");
   }
-  float* w = reinterpret_cast<float*>(tmp);
-  float* r = reinterpret_cast<float*>(tmp + wb);
-  float* c = reinterpret_cast<float*>(tmp + wb + rb);
-  double* g = reinterpret_cast<double*>(tmp + wb + rb + cb);
-  int* d = reinterpret_cast<int*>(g + 2);
-  float* parts = reinterpret_cast<float*>(tmp + wb + rb + cb + 256);
+  float* r = reinterpret_cast<float*>(tmp);
+  float* c = reinterpret_cast<float*>(tmp + rb);
+  MatStats* t = reinterpret_cast<MatStats*>(tmp + rb + cb);
+  float* parts = reinterpret_cast<float*>(tmp + rb + cb + tb);
   meq_status ms = MEQ_OK;
-  e = cudaMemsetAsync(w, 0, static_cast<size_t>(rows * cols * 4), s);
-  if (e != cudaSuccess) ms = cuda_fail(nullptr, e, "cudaMemsetAsync");
   // k = 0: the statistics of X_0 = H / ||H||_F (the threshold eps applies to
   // the RMS of X_0, as for every later iterate), in this call's own scratch
-  if (ms == MEQ_OK) {
-    const char* what = "";
-    e = launch_row_col_stats(h, rows, cols, eps, o.tie_atol, 1, parts, r, c, g, d, s, &what);
-    if (e != cudaSuccess) ms = cuda_fail(nullptr, e, what);
+  const char* what = "";
+  e = launch_row_col_stats(h, rows, cols, eps, o.tie_atol, 1, parts, r, c, &t[0].gamma_r, &t[0].direction, s, &what);
+  if (e != cudaSuccess) ms = cuda_fail(nullptr, e, what);
+  // k >= 1: one chain of NS products over a one-matrix state fed H with no
+  // momentum history and mu = 0 (so its NS input is H). After each iteration
+  // U = X_k is written as the step writes it and its statistics go to t[k];
+  // then X_k itself, for the next iteration. (One state per k took 3 (1 + ..
+  // + steps) products and as many set-ups: 14.2 ms for 20 iterations of a
+  // 1024 x 2736 matrix, 1.7 ms this way.)
+  meq_state* st = nullptr;
+  if (ms == MEQ_OK && steps > 0) {
+    o.ns_steps = steps;
+    ms = init_state(&shape, nullptr, 1, &o, cuda_stream, true, &st);
   }
-  double hg[2] = {0.0, 0.0};
-  if (ms == MEQ_OK) {
-    e = cudaMemcpyAsync(hg, g, sizeof(hg), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) ms = cuda_fail(nullptr, e, "cudaMemcpyAsync");
-  }
-  if (ms == MEQ_OK) gamma_r[0] = hg[0], gamma_c[0] = hg[1];
-  // k >= 1: the statistics of the k-step NS output of a one-matrix state fed
-  // H with no momentum history and mu = 0 (so its NS input is H), lr = 0
-  for (int k = 1; ms == MEQ_OK && k <= steps; ++k) {
-    o.ns_steps = k;
-    meq_state* st = nullptr;
-    ms = meq_init_state(&shape, 1, &o, cuda_stream, &st);
-    if (ms != MEQ_OK) break;
-    float* wp = w;
-    const float* hp = h;
-    ms = meq_step(&wp, &hp, st, &shape, 1, 0.f, 0.f, 0.f, eps, cuda_stream);
+  if (ms == MEQ_OK && st) {
+    ms = upload_step(st, nullptr, &h, &shape, 1, 0.f, 0.f, 0.f, eps, s);
+    if (ms == MEQ_OK) ms = enqueue_trajectory(st, t + 1, s);
     if (ms == MEQ_OK) ms = meq_sync(st);
-    if (ms == MEQ_OK) ms = meq_read_stats(st, 0, nullptr, nullptr, gamma_r + k, gamma_c + k, nullptr);
     if (ms != MEQ_OK) g_init_error = st->last_error;
-    meq_free(st);
   }
+  // (the CVs of k = 0 are delivered whatever became of the iterates)
+  std::vector<MatStats> ht(static_cast<size_t>(steps) + 1);
+  e = cudaMemcpyAsync(ht.data(), t, ht.size() * sizeof(MatStats), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess && ms == MEQ_OK) ms = cuda_fail(nullptr, e, "cudaMemcpyAsync");
+  if (e == cudaSuccess)
+    for (int k = 0; k <= (ms == MEQ_OK ? steps : 0); ++k)
+      gamma_r[k] = ht[static_cast<size_t>(k)].gamma_r, gamma_c[k] = ht[static_cast<size_t>(k)].gamma_c;
+  meq_free(st);
   cudaFree(tmp);
   return ms;
 }

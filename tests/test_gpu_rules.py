@@ -146,6 +146,24 @@ def test_ns_cv_trajectory_matches_oracle(meq):
     torch.cuda.synchronize()
 
 
+@pytest.mark.parametrize("shape", [(200, 333), (333, 200), (256, 256), (64, 9000)])
+@pytest.mark.parametrize("opts", [{}, {"ns_x0_fused": 0}, {"ns_fp16_mask": 0}, {"ns_fp16_mask": 0b01101},
+                                  {"nesterov": 1, "ns_cta_pair": 0}], ids=str)
+def test_ns_cv_trajectory_is_that_of_separate_steps(meq, shape, opts):
+    """Point k of the trajectory equals, bit for bit, the CVs that a k-iteration step from the same
+    matrix reports (tall and wide, operand formats that change between iterations)."""
+    import torch
+
+    H = torch.randn(shape, generator=torch.Generator().manual_seed(5)) * torch.logspace(-1, 1, shape[0])[:, None]
+    gr, gc = meq.ns_cv_trajectory(H.cuda(), steps=6, **opts)
+    for k in (1, 2, 5, 6):
+        opt = meq.MeqMuon([shape], ns_steps=k, **opts)
+        opt.step([torch.zeros(shape, device="cuda")], [H.cuda()], 0.0, 0.0, 0.0)
+        st = opt.read_stats(0)
+        assert (gr[k], gc[k]) == (st["gamma_r"], st["gamma_c"]), k
+        opt.close()
+
+
 def test_ns_cv_trajectory_threshold_applies_to_x0(meq):
     """Section 3.1 replays Eq. (5) from X_0 = H / ||H||_F, and Eq. (8)
     counts the rows and columns whose RMS exceeds delta: the threshold is on
