@@ -132,6 +132,35 @@ def test_paired_iterations(meq, pair):
     assert all(r["update"] <= PT.UPDATE_TOL for r in rep)
 
 
+@pytest.mark.parametrize("shapes", [[(257, 131)], [(1, 1)], [(1, 999)], [(640, 64)] * 3 + [(64, 640)]], ids=str)
+@pytest.mark.parametrize("canaries", [0, 1])
+def test_read_back_in_pieces(meq, shapes, canaries):
+    """U and the update read to the host, through the state's scratch in as many pieces as it takes
+    (one matrix per group: two), equal what the kernel writes into device memory, are the fp16
+    values the library holds, and leave the next step as it is."""
+    import torch
+
+    wl = W.custom_workload(shapes, pattern="both", base_sigma=0.01, seed=43)
+    a, b = (meq.MeqMuon(shapes, debug_canaries=canaries) for _ in range(2))
+    pa, pb = _to_dev(W.initial_weights(wl)), _to_dev(W.initial_weights(wl))
+    for t in range(2):
+        Gs = _to_dev(W.gradients(wl, t))
+        a.step(pa, Gs, LR, MU, WD, EPS)
+        b.step(pb, Gs, LR, MU, WD, EPS)
+        for i, (m, n) in enumerate(shapes):
+            d = torch.empty(m, n, device="cuda")
+            for read, host in ((meq.lib.meq_read_ns_output, a.read_ns_output(i)), (meq.lib.meq_read_update, a.read_update(i))):
+                assert read(a._st, i, d.data_ptr()) == 0
+                assert np.array_equal(d.cpu().numpy(), host), (i, t)
+            U = a.read_ns_output(i) * 16384.0
+            assert np.array_equal(U, U.astype(np.float16).astype(np.float32))
+        assert all(torch.equal(x, y) for x, y in zip(pa, pb))  # b is never read
+        if canaries:
+            a.check_canaries()
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("pair", [1, 0], ids=["cta_pair", "single_cta"])
 def test_separate_x0_cast(meq, pair):
     """X_0 normalised and cast by its own pass (ns_x0_fused = 0: momentum +
