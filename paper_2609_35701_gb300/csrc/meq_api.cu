@@ -47,8 +47,13 @@ struct Group {
   int64_t m = 0, n = 0, un = 0;  // weight shape of every member, U row stride
   int64_t u_base = 0;      // element offset of the group's fp16 U block [count][m][un]
   int64_t mbase = 0;       // first slot of the group in the per-matrix inverse-norm array
-  int64_t rpart_base = 0;  // float offsets of the fused-statistics partials
+  // Fused-statistics partials: the column sums (float offset in the slab), and
+  // the row sums, rparts per row, in the X buffer that the last update leaves
+  // idle (CV trajectory, where each update writes U: in the slab).
   int64_t cpart_base = 0;
+  int64_t rpart_base = 0;
+  int64_t rparts = 0;
+  float* rpart = nullptr;
   std::vector<int> mats;
   uint16_t* x[2] = {nullptr, nullptr};
   uint16_t* a16 = nullptr;
@@ -128,6 +133,7 @@ struct meq_state {
   // launch plan
   std::vector<GemmParams> gemm;  // in launch order
   std::vector<int> gemm_grid;
+  std::vector<GemmTile> gemm_tile;
   LaunchCtx ctx{};
   bool graph_ready = false;
   cudaGraph_t graph = nullptr;
@@ -287,8 +293,9 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
   for (auto& G : st->groups) {  // U is stored group by group: [count][m][un]
     G.u_base = u;
     u += round_up(G.count * G.m * G.un, 64);
+    G.rparts = 2 * ((G.l + 63) / 64);  // at most: 64-column tiles
     G.rpart_base = parts;
-    parts += round_up(G.count * 2 * ((G.l + 255) / 256) * G.s, 64);
+    if (st->trajectory) parts += round_up(G.count * G.rparts * G.s, 64);
     G.cpart_base = parts;
     parts += round_up(G.count * ((G.s + 31) / 32) * G.l, 64);
   }
@@ -311,7 +318,6 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
       const Group& G = st->groups[M.group];
       M.un = G.un;
       M.u_off = G.u_base + M.gidx * M.m * M.un;
-      M.rpart_off = G.rpart_base + M.gidx * 2 * ((G.l + 255) / 256) * G.s;
       M.cpart_off = G.cpart_base + M.gidx * ((G.s + 31) / 32) * G.l;
       hchunks += (M.m * M.n + kChunk - 1) / kChunk;
       tiles += ((M.m + kCastTile - 1) / kCastTile) * ((M.n + kCastTile - 1) / kCastTile);
@@ -398,18 +404,20 @@ bool encode_map(CUtensorMap* m, void* base, int elem_bytes, int64_t inner, int64
 constexpr CUtensorMapSwizzle SW128 = CU_TENSOR_MAP_SWIZZLE_128B;
 constexpr CUtensorMapSwizzle SW64 = CU_TENSOR_MAP_SWIZZLE_64B;
 
-// Tiles (tile_m rows x 256 columns) holding a 32 x 32 block on or above the diagonal.
-int sym_tiles(int tiles_m, int tiles_n, int tile_m) {
-  int t = 0;
-  for (int tn = 0; tn < tiles_n; ++tn) t += std::min(tiles_m, ((tn + 1) * 256) / tile_m);
-  return t;
+// Tiles of one M x N product; symmetric: those holding a 32 x 32 block on or above the diagonal.
+int64_t tile_count(int64_t M, int64_t N, bool sym, const GemmTile& t) {
+  const int64_t tile_m = 128 * t.pair, tm = (M + tile_m - 1) / tile_m, tn = (N + t.bn - 1) / t.bn;
+  if (!sym) return tm * tn;
+  int64_t c = 0;
+  for (int64_t j = 0; j < tn; ++j) c += std::min(tm, ((j + 1) * t.bn + tile_m - 1) / tile_m);
+  return c;
 }
 
 // tcgen05 kind::f16 instruction descriptor: D fp32, A/B fp16 (0) or bf16 (1),
-// A K-major, B K-major or MN-major, N = 256, M = 128 (one CTA) or 256 (pair).
-uint32_t make_idesc(bool fp16, bool b_mn_major, int m) {
+// A K-major, B K-major or MN-major, N columns, M = 128 (one CTA) or 256 (pair).
+uint32_t make_idesc(bool fp16, bool b_mn_major, int m, int n) {
   const uint32_t fmt = fp16 ? 0u : 1u;
-  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((256u >> 3) << 17) |
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((static_cast<uint32_t>(n) >> 3) << 17) |
          ((static_cast<uint32_t>(m) >> 4) << 24);
 }
 
@@ -557,11 +565,36 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
   return ops;
 }
 
+// Rows and columns of a product's output.
+int64_t op_rows(const Group& G, const NsOp&) { return G.s; }
+int64_t op_cols(const Group& G, const NsOp& op) { return op.out_is_x ? G.l : G.s; }
+
+// Estimated duration (us) of a launch, to choose between 64-column tiles on
+// single CTAs and 256-column tiles on CTA pairs: whole waves of tiles, each a
+// fixed part (first operands, epilogue, hand-over; longer for the mirrored
+// stores of symmetric products) and a part per k-block. Constants fitted to
+// steps of 1 to 48 equal weights, all with one variant, us (256-column /
+// 64-column): 256 x 256: one 111 / 80, eight 120 / 81, 32 123 / 110; 512 x 512:
+// four 146 / 105, 16 162 / 201; 128 x 512: 48 129 / 102; 1024 x 1024: one 180 /
+// 138, two 184 / 158, four 199 / 287; 1024 x 2736: two 265 / 246, eight 519 / 656.
+double launch_cost(const std::vector<std::pair<const Group*, const NsOp*>>& ops, const GemmTile& t, int num_sms) {
+  double tiles = 0, us = 0;
+  for (const auto& x : ops) {
+    const Group& G = *x.first;
+    const NsOp& op = *x.second;
+    const bool sym = op.mode == MODE_SYM;
+    const double n = static_cast<double>(tile_count(op_rows(G, op), op_cols(G, op), sym, t)) * G.count;
+    const double nk = static_cast<double>(((op.gram ? G.l : G.s) + 63) / 64);
+    tiles += n;
+    us += n * (t.bn == 64 ? 1.2 + 0.22 * nk : (sym ? 3.2 : 2.8) + 0.35 * nk);
+  }
+  return std::ceil(tiles * t.pair / num_sms) * us / tiles;
+}
+
 // Fills one group's part of a launch from its product.
-bool fill_group(const meq_state* st, const Group& G, const NsOp& op, GemmGroup& Q) {
-  const int pair = st->opt.ns_cta_pair ? 2 : 1;
-  const int tile_m = 128 * pair;
-  const uint32_t b_rows = static_cast<uint32_t>(256 / pair);  // K-major B rows each CTA loads
+bool fill_group(const meq_state* st, const Group& G, const NsOp& op, const GemmTile& t, GemmGroup& Q) {
+  const int tile_m = 128 * t.pair;
+  const uint32_t b_rows = static_cast<uint32_t>(t.bn / t.pair);  // K-major B rows each CTA loads
   void* const base[4] = {G.x[0], G.x[1], G.a16, G.p16};
   const bool dense = op.mode != MODE_SYM;
   // buffers as matrices of the group: s x l with row stride lp (X), or s x s with row stride sp
@@ -570,12 +603,12 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, GemmGroup& 
   };
   auto ld = [&](bool is_x) { return (is_x ? G.lp : G.sp) * 2; };
   Q.mode = op.mode;
-  Q.idesc = make_idesc(op.in16, dense, tile_m);
+  Q.idesc = make_idesc(op.in16, dense, tile_m, t.bn);
   Q.b_mn_major = dense ? 1 : 0;
   Q.count = static_cast<int32_t>(G.count);
   Q.trans = G.trans;
-  Q.M = static_cast<int32_t>(G.s);
-  Q.N = static_cast<int32_t>(op.out_is_x ? G.l : G.s);
+  Q.M = static_cast<int32_t>(op_rows(G, op));
+  Q.N = static_cast<int32_t>(op_cols(G, op));
   Q.K = static_cast<int32_t>(op.gram ? G.l : G.s);
   Q.sym = dense ? 0 : 1;
   Q.tma_out = Q.sym;
@@ -594,12 +627,12 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, GemmGroup& 
     Q.out = base[op.out], Q.out_ld = ld(op.out_is_x), Q.out_mstride = G.s * ld(op.out_is_x);
   } else if (op.mode == MODE_XLAST) {
     Q.out = st->d_u + G.u_base, Q.out_ld = G.un * 2, Q.out_mstride = G.m * G.un * 2;
-    Q.rpart = st->d_parts + G.rpart_base;
+    Q.rpart = G.rpart;
     Q.cpart = st->d_parts + G.cpart_base;
   }
   Q.tiles_m = static_cast<int32_t>((Q.M + tile_m - 1) / tile_m);
-  Q.tiles_n = static_cast<int32_t>((Q.N + 255) / 256);
-  Q.tiles_per_mat = Q.sym ? sym_tiles(Q.tiles_m, Q.tiles_n, tile_m) : Q.tiles_m * Q.tiles_n;
+  Q.tiles_n = static_cast<int32_t>((Q.N + t.bn - 1) / t.bn);
+  Q.tiles_per_mat = static_cast<int32_t>(tile_count(Q.M, Q.N, !dense, t));
   // Dense products walk bands of tile rows column by column; a band's
   // row panels of P (band * tile_m * K 16-bit values) stay within 32 MB,
   // about a quarter of L2, so every P panel is read from DRAM once.
@@ -614,7 +647,8 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, GemmGroup& 
 bool build_gemm_plan(meq_state* st, std::string* why) {
   st->gemm.clear();
   st->gemm_grid.clear();
-  const int pair = st->opt.ns_cta_pair ? 2 : 1;
+  st->gemm_tile.clear();
+  const GemmTile large{st->opt.ns_cta_pair ? 2 : 1, 256}, small{1, 64};
   int64_t saving = 0;
   if (pairs_allowed(st->opt) && !st->trajectory)
     for (const Group& G : st->groups) saving += std::max<int64_t>(0, pair_saving(G)) * G.count;
@@ -658,14 +692,30 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
       P.timeout_ns = static_cast<unsigned long long>(static_cast<double>(st->opt.wait_timeout_ms) * 1e6);
       int tiles = 0;
       P.ngroups = static_cast<int32_t>(std::min<size_t>(kMaxGroups, gs.size() - g0));
+      std::vector<std::pair<const Group*, const NsOp*>> ops;
+      for (int gi = 0; gi < P.ngroups; ++gi) {
+        const int g = gs[g0 + gi];
+        ops.emplace_back(&st->groups[g], &chain[g][at[which[g]]]);
+      }
+      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load &&
+                             launch_cost(ops, small, st->num_sms) < launch_cost(ops, large, st->num_sms);
+      const GemmTile& t = use_small ? small : large;
       for (int gi = 0; gi < P.ngroups; ++gi) {
         const int g = gs[g0 + gi];
         GemmGroup& Q = P.g[gi];
-        if (!fill_group(st, st->groups[g], chain[g][at[which[g]]], Q)) { *why = "cuTensorMapEncodeTiled failed"; return false; }
+        Group& G = st->groups[g];
+        const NsOp& op = chain[g][at[which[g]]];
+        if (op.mode == MODE_XLAST) {
+          // two row partials per tile column
+          G.rparts = 2 * ((op_cols(G, op) + t.bn - 1) / t.bn);
+          G.rpart = st->trajectory ? st->d_parts + G.rpart_base
+                                   : reinterpret_cast<float*>(G.x[op.b == BUF_X0 ? 1 : 0]);
+        }
+        if (!fill_group(st, G, op, t, Q)) { *why = "cuTensorMapEncodeTiled failed"; return false; }
         Q.tile_begin = tiles;
-        const int64_t t = int64_t(Q.tiles_per_mat) * Q.count;
-        if (tiles + t > (int64_t(1) << 30)) { *why = "too many GEMM tiles in one launch"; return false; }
-        tiles += static_cast<int>(t);
+        const int64_t n = int64_t(Q.tiles_per_mat) * Q.count;
+        if (tiles + n > (int64_t(1) << 30)) { *why = "too many GEMM tiles in one launch"; return false; }
+        tiles += static_cast<int>(n);
       }
       P.total_tiles = tiles;
       // Each launch walks the matrices in the opposite order of the one
@@ -674,8 +724,9 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
       P.reverse = (st->gemm.size() % 2 == 0) ? 1 : 0;
       P.debug_skip_load = (st->opt.debug_skip_load && st->gemm.empty()) ? 1 : 0;
       st->gemm.push_back(P);
+      st->gemm_tile.push_back(t);
       // persistent grid: one CTA (pair) per SM (pair of SMs), never more than the tiles
-      st->gemm_grid.push_back(pair * std::max(1, std::min(tiles, st->num_sms / pair)));
+      st->gemm_grid.push_back(t.pair * std::max(1, std::min(tiles, st->num_sms / t.pair)));
     }
     for (int c = 0; c < 2; ++c)
       if (take[c]) ++at[c];
@@ -848,6 +899,17 @@ static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, c
     G.p16 = reinterpret_cast<uint16_t*>(A + goffs[4 * g + 3]);
   }
 
+  if (!build_gemm_plan(st, &why)) {
+    cudaFree(st->arena);
+    delete st;
+    return fail(nullptr, MEQ_ERR_UNSUPPORTED, why);
+  }
+  for (MatInfo& M : st->mats)
+    if (M.kind == KIND_HIDDEN) {
+      const Group& G = st->groups[M.group];
+      M.rparts = G.rparts;
+      M.rpart_off = (G.rpart - st->d_parts) + M.gidx * G.rparts * G.s;
+    }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   std::vector<GroupInfo> gi(st->groups.size());
   for (size_t g = 0; g < st->groups.size(); ++g) {
@@ -871,11 +933,6 @@ static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, c
     return fail(nullptr, MEQ_ERR_CUDA, std::string("initialising the state failed: ") + cudaGetErrorString(ee));
   }
 
-  if (!build_gemm_plan(st, &why)) {
-    cudaFree(st->arena);
-    delete st;
-    return fail(nullptr, MEQ_ERR_UNSUPPORTED, why);
-  }
   LaunchCtx& C = st->ctx;
   C.mats = st->d_mats;
   C.nmat = n;
@@ -993,7 +1050,7 @@ static meq_status enqueue_kernels(meq_state* st, cudaStream_t s, cudaEvent_t* ev
   }
   mark(2);
   for (size_t i = 0; i < st->gemm.size(); ++i) {
-    e = launch_ns_gemm(st->gemm[i], st->gemm_grid[i], st->opt.ns_cta_pair ? 2 : 1, s);
+    e = launch_ns_gemm(st->gemm[i], st->gemm_tile[i], st->gemm_grid[i], s);
     if (e != cudaSuccess) return cuda_fail(st, e, "ns_gemm launch");
   }
   mark(3);
@@ -1021,7 +1078,7 @@ static meq_status enqueue_trajectory(meq_state* st, MatStats* t, cudaStream_t s)
   if (e != cudaSuccess) return cuda_fail(st, e, "momentum launch");
   C.stats = t;
   for (size_t i = 0; i < st->gemm.size(); ++i) {
-    e = launch_ns_gemm(st->gemm[i], st->gemm_grid[i], st->opt.ns_cta_pair ? 2 : 1, s);
+    e = launch_ns_gemm(st->gemm[i], st->gemm_tile[i], st->gemm_grid[i], s);
     if (e != cudaSuccess) return cuda_fail(st, e, "ns_gemm launch");
     if (st->gemm[i].g[0].mode != MODE_XLAST) continue;
     e = launch_stats(C, s);

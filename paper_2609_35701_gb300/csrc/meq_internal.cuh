@@ -57,7 +57,8 @@ struct MatInfo {
   int64_t tile_begin;    // first cast tile (hidden weights only)
   int64_t xblk_begin;    // first momentum-and-X_0 block (hidden weights only)
   int64_t fold_begin;    // first block of the fold of the partial sums (hidden weights and remaining 2D)
-  int64_t rpart_off;     // float offset of NS-row partial sums of squares [2 * ceil(l/256)][s]
+  int64_t rpart_off;     // float offset of NS-row partial sums of squares [rparts][s]
+  int64_t rparts;        // two per tile column of the last update
   int64_t cpart_off;     // float offset of column partial sums of squares: NS columns
                          // [ceil(s/32)][l] (hidden) or normalised columns [slabs][n] (remaining 2D)
 };
@@ -86,7 +87,7 @@ enum GemmMode : int { MODE_SYM = 0, MODE_DENSE = 1, MODE_XLAST = 2 };
 
 struct GemmGroup {
   CUtensorMap tmA;        // A operand (K-major), box {64, 128, 1}
-  CUtensorMap tmB;        // B operand: K-major box {64, 256, 1} or MN-major box {64, 64, 1}
+  CUtensorMap tmB;        // B operand: K-major box {64, bn / pair, 1} or MN-major box {64, 64, 1}
   CUtensorMap tmO;        // symmetric products: the 16-bit output for TMA stores,
                           // box {32, 32, 1}, 64-byte swizzle (the epilogue's staging layout)
   int32_t M, N, K;        // output rows, output cols, contraction
@@ -120,6 +121,12 @@ struct GemmGroup {
   uint32_t idesc;         // tcgen05 instruction descriptor
   int32_t b_mn_major;     // 1: B operand tile is MN-major (DENSE, XLAST)
   int32_t tma_out;        // 1: the output leaves by TMA stores through tmO (else 16-byte thread stores)
+};
+
+// Tile variant of a launch: pair 1 or 2 CTAs per tile of 128 * pair rows and
+// bn columns.
+struct GemmTile {
+  int pair, bn;
 };
 
 // One GEMM launch: one product's shape groups, taken as one tile queue in
@@ -170,8 +177,8 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 // Launchers (defined in the .cu files).
-cudaError_t prepare_ns_gemm();  // sets the kernel's dynamic shared-memory limit (per device)
-cudaError_t launch_ns_gemm(const GemmParams& p, int grid, int pair, cudaStream_t st);  // pair: 1 or 2 CTAs per tile
+cudaError_t prepare_ns_gemm();  // sets the kernels' dynamic shared-memory limits (per device)
+cudaError_t launch_ns_gemm(const GemmParams& p, const GemmTile& t, int grid, cudaStream_t st);
 int ns_gemm_smem_bytes(int pair);
 
 // Row / column statistics of one fp32 matrix (Eqs. (7), (8), (11)) with

@@ -57,28 +57,34 @@
 namespace meq {
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, UK = 16;  // per-CTA rows, tile columns, k-block, MMA K
+constexpr int BM = 128, BK = 64, UK = 16;            // per-CTA rows, k-block, MMA K
 constexpr int A_BYTES = BM * BK * 2;                 // 16 KB
 constexpr int NUM_EPI_WARPS = kNsEpilogueWarps;      // two per TMEM lane quarter
 constexpr int SCHED_WARP = 2 + NUM_EPI_WARPS;
 constexpr int NUM_THREADS = 64 + 32 * NUM_EPI_WARPS + 32;
-constexpr uint32_t TMEM_COLS = 512;
 constexpr int SLOT_BYTES = 2048;                     // one 32 x 32 16-bit block (two per epilogue warp)
 constexpr int SCHED_D = 16;                          // entries of the tile ring (16 bytes each)
 constexpr float kUInvScale2 = 1.0f / (kUScale * kUScale);  // exact: kUScale is a power of two
 
-// kPair = 1: one CTA computes a 128 x 256 tile (tcgen05 cta_group::1).
-// kPair = 2: a cluster of two CTAs computes a 256 x 256 tile with
+// kPair = 1: one CTA computes a 128 x kBN tile (tcgen05 cta_group::1).
+// kPair = 2: a cluster of two CTAs computes a 256 x kBN tile with
 // cta_group::2 MMAs: each CTA holds its own 128 rows of A and half of B
-// (128 rows / columns), so a stage is 32 KB instead of 48 KB per SM and six
-// stages fit.
-template <int kPair>
+// (kBN / 2 rows / columns), so at kBN = 256 a stage is 32 KB instead of 48 KB
+// per SM and six stages fit.
+// <2, 256> is the variant for launches that fill the chip. <1, 64> is for
+// launches of so few tiles that each SM gets at most one: there the launch is
+// a chain of latencies, of which the epilogue of a 256-column tile (four
+// 32-column chunks per warp, 0.6-1 us each) is the longest; a 64-column tile
+// has one chunk per warp, more SMs work, and eight stages hold the operands
+// of 512 contraction steps at once. <1, 256> is the option ns_cta_pair = 0.
+template <int kPair, int kBN>
 struct Cfg {
   static constexpr int TILE_M = BM * kPair;
-  static constexpr int BN_LOCAL = BN / kPair;
+  static constexpr int BN_LOCAL = kBN / kPair;
   static constexpr int B_BYTES = BN_LOCAL * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = kPair == 1 ? 4 : 6;
+  static constexpr int STAGES = kBN == 64 ? 8 : kPair == 1 ? 4 : 6;
+  static constexpr uint32_t TMEM_COLS = 2 * kBN;  // two accumulators
   // full, empty, tmem full x2, tmem empty x2, drain, tile ring full / empty,
   // entry taken by the producer
   static constexpr int NUM_BARS = 2 * STAGES + 4 + 1 + 2 * SCHED_D + 1;
@@ -313,7 +319,7 @@ struct TileCoord {
 // band's panels of P, where a row-by-row walk re-read every column panel of
 // a wide X once per tile row (measured at 4096 x 11008: 4.5 times the
 // launch's algorithmic bytes from DRAM). Symmetric outputs (Gram, polynomial) run tn-major over
-// the tiles with tm * TILE_M < (tn + 1) * 256, i.e. those holding a 32 x 32
+// the tiles with tm * TILE_M < (tn + 1) * kBN, i.e. those holding a 32 x 32
 // block on or above the diagonal.
 __device__ __forceinline__ int find_segment(const GemmParams& p, int t) {
   int lo = 0, hi = p.ngroups - 1;  // the last segment whose tile_begin <= t
@@ -324,7 +330,7 @@ __device__ __forceinline__ int find_segment(const GemmParams& p, int t) {
   }
   return lo;
 }
-template <int kPair>
+template <int kPair, int kBN>
 __device__ __forceinline__ TileCoord decode_tile(const GemmParams& p, int t) {
   if (p.reverse) t = p.total_tiles - 1 - t;
   const int g = find_segment(p, t);
@@ -344,7 +350,7 @@ __device__ __forceinline__ TileCoord decode_tile(const GemmParams& p, int t) {
   } else {
     int tn = 0;
     for (;;) {
-      const int cnt = min(G.tiles_m, ((tn + 1) * BN) / Cfg<kPair>::TILE_M);
+      const int cnt = min(G.tiles_m, ((tn + 1) * kBN + Cfg<kPair, kBN>::TILE_M - 1) / Cfg<kPair, kBN>::TILE_M);
       if (r < cnt) break;
       r -= cnt;
       ++tn;
@@ -458,9 +464,11 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_reads() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // Every committed store has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-template <int kPair>
+template <int kPair, int kBN>
 __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_constant__ GemmParams p) {
-  using C_ = Cfg<kPair>;
+  using C_ = Cfg<kPair, kBN>;
+  constexpr int BN = kBN;
+  constexpr uint32_t TMEM_COLS = C_::TMEM_COLS;
   constexpr int STAGES = C_::STAGES;
   constexpr int STAGE_BYTES = C_::STAGE_BYTES;
   constexpr int TILE_M = C_::TILE_M;
@@ -745,7 +753,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       const int rows_valid = min(32, G.M - row0);
       float rsum = 0.f;            // XLAST: this lane's row, sum of squares over the tile
       const int nch = min(BN / 32, (G.N - c.tn * BN + 31) / 32);
-      int ch0 = G.sym ? max(0, R - c.tn * 8) : 0;  // blocks strictly below the diagonal come from mirrors
+      int ch0 = G.sym ? max(0, R - c.tn * (BN / 32)) : 0;  // blocks strictly below the diagonal come from mirrors
       if ((ch0 & 1) != half) ++ch0;                // this warp's chunks: ch % 2 == half
       if (row0 >= G.M) ch0 = nch;
       uint8_t* outm = static_cast<uint8_t*>(G.out) + static_cast<int64_t>(c.mat) * G.out_mstride;
@@ -777,7 +785,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       tc_fence_after();
       for (int ch = ch0; ch < nch; ch += 2) {
         const int col0 = c.tn * BN + ch * 32;
-        const int C = c.tn * 8 + ch;
+        const int C = c.tn * (BN / 32) + ch;
         float v[32];
         tmem_ld_32cols(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * BN + ch * 32), v);
         if (G.tma_out) {
@@ -906,7 +914,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         }
         __syncwarp();  // reconverge before the next warp-wide tcgen05.ld
       }
-      if (mode == MODE_XLAST && row0 < G.M && row0 + lane < G.M)  // one partial per (tile column, half)
+      if (mode == MODE_XLAST && row0 + lane < G.M)  // one partial per (tile column, half)
         G.rpart[(static_cast<int64_t>(c.mat) * G.tiles_n * 2 + c.tn * 2 + half) * G.M + row0 + lane] = rsum * kUInvScale2;
       tc_fence_before();
       __syncwarp();
@@ -932,7 +940,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         }
         uint4 e = make_uint4(static_cast<uint32_t>(t), 0u, 0u, 0u);
         if (t < p.total_tiles) {
-          const TileCoord c = decode_tile<kPair>(p, t);
+          const TileCoord c = decode_tile<kPair, kBN>(p, t);
           const GemmGroup& G = p.g[c.g];
           const int nk = (G.K + BK - 1) / BK;
           const bool b_is_a = kPair == 2 && G.same_ab && c.tm * TILE_M == c.tn * BN;
@@ -947,6 +955,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         // queue counter, which that kernel's last unit resets, only after it.
         if (n == 0) pdl_wait_predecessor();
         fetched = atomicAdd(p.sched, 1);  // read when the producer has taken this entry
+      }
+      // This unit claims nothing more (its claims have returned). The last
+      // unit to get here resets the queue; the next launch reads it only after
+      // this grid has completed. (Counting out at the CTA's end, behind a
+      // fence, held every launch up by 0.5-0.8 us.)
+      pdl_wait_predecessor();
+      if (atomicAdd(p.sched + 1, 1) == nunits - 1) {
+        p.sched[0] = 0;
+        p.sched[1] = 0;
       }
     }
     __syncwarp();
@@ -970,16 +987,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
   __syncthreads();
   if (kPair == 2) cluster_sync_all();  // no CTA leaves while its peer may still signal it
   tc_fence_after();
-  if (threadIdx.x == 0 && leader) {
-    // The last unit to finish resets the tile queue. Every unit's fetches
-    // precede its count here, and the next launch reads the queue only after
-    // this grid has completed.
-    __threadfence();
-    if (atomicAdd(p.sched + 1, 1) == nunits - 1) {
-      p.sched[0] = 0;
-      p.sched[1] = 0;
-    }
-  }
   if (warp == 1) {
     if (kPair == 2)
       asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
@@ -990,17 +997,23 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
 
 }  // namespace
 
-int ns_gemm_smem_bytes(int pair) { return pair == 2 ? Cfg<2>::SMEM_BYTES : Cfg<1>::SMEM_BYTES; }
+int ns_gemm_smem_bytes(int pair) { return pair == 2 ? Cfg<2, 256>::SMEM_BYTES : Cfg<1, 256>::SMEM_BYTES; }
 
 cudaError_t prepare_ns_gemm() {
-  cudaError_t e = cudaFuncSetAttribute(ns_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1>::SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(ns_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<2>::SMEM_BYTES);
+  auto set = [](auto kernel, int bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  cudaError_t e = set(ns_gemm_kernel<1, 256>, Cfg<1, 256>::SMEM_BYTES);
+  if (e == cudaSuccess) e = set(ns_gemm_kernel<1, 64>, Cfg<1, 64>::SMEM_BYTES);
+  if (e == cudaSuccess) e = set(ns_gemm_kernel<2, 256>, Cfg<2, 256>::SMEM_BYTES);
+  return e;
 }
 
-cudaError_t launch_ns_gemm(const GemmParams& p, int grid, int pair, cudaStream_t st) {
-  if (pair == 2) return launch_pdl(ns_gemm_kernel<2>, dim3(grid), dim3(NUM_THREADS), Cfg<2>::SMEM_BYTES, st, 2, p);
-  return launch_pdl(ns_gemm_kernel<1>, dim3(grid), dim3(NUM_THREADS), Cfg<1>::SMEM_BYTES, st, 1, p);
+cudaError_t launch_ns_gemm(const GemmParams& p, const GemmTile& t, int grid, cudaStream_t st) {
+  const dim3 g(grid), b(NUM_THREADS);
+  if (t.pair == 2) return launch_pdl(ns_gemm_kernel<2, 256>, g, b, Cfg<2, 256>::SMEM_BYTES, st, 2, p);
+  if (t.bn == 64) return launch_pdl(ns_gemm_kernel<1, 64>, g, b, Cfg<1, 64>::SMEM_BYTES, st, 1, p);
+  return launch_pdl(ns_gemm_kernel<1, 256>, g, b, Cfg<1, 256>::SMEM_BYTES, st, 1, p);
 }
 
 }  // namespace meq

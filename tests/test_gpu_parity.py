@@ -132,6 +132,33 @@ def test_paired_iterations(meq, pair):
     assert all(r["update"] <= PT.UPDATE_TOL for r in rep)
 
 
+@pytest.mark.parametrize("shapes", [
+    [(200, 333), (333, 200), (130, 130)], [(257, 513), (513, 257), (64, 1000), (1000, 64)],
+    [(384, 768), (768, 384), (768, 768), (129, 385)], [(63, 65), (64, 64), (65, 63), (128, 129), (192, 200)],
+], ids=str)
+def test_tile_variants_agree(meq, shapes):
+    """A state of a few matrices runs its products on 64-column tiles of single CTAs, one of sixty
+    times as many on 256-column tiles of CTA pairs: the same U bit for bit on ragged shapes, and
+    statistics within fp32 summation order (1e-5); the large state staged against the oracle."""
+    many = shapes * 60
+    wl = W.custom_workload(shapes, pattern="both", base_sigma=0.01, seed=47)
+    Gs, W0 = _to_dev(W.gradients(wl, 0)), _to_dev(W.initial_weights(wl))
+    a, b = meq.MeqMuon(shapes), meq.MeqMuon(many)
+    a.step([w.clone() for w in W0], Gs, LR, MU, WD, EPS)
+    pb = [w.clone() for _ in range(60) for w in W0]
+    b.step(pb, Gs * 60, LR, MU, WD, EPS)
+    for i in range(len(shapes)):
+        for k in (i, len(many) - len(shapes) + i):
+            U = b.read_ns_output(k)
+            assert np.array_equal(a.read_ns_output(i), U), (shapes[i], k)
+            sa, sb = a.read_stats(i), b.read_stats(k)
+            assert PT.max_rel(sa["r"], sb["r"]) <= 1e-5 and PT.max_rel(sa["c"], sb["c"]) <= 1e-5
+            PT.check_step(W0[i].cpu().numpy(), Gs[i].cpu().double().numpy(), np.zeros(shapes[i]), pb[k].cpu().numpy(),
+                          b.read_momentum(k), U, sb, LR, MU, WD, EPS, Ut_gpu=b.read_update(k))
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("shapes", [[(257, 131)], [(1, 1)], [(1, 999)], [(640, 64)] * 3 + [(64, 640)]], ids=str)
 @pytest.mark.parametrize("canaries", [0, 1])
 def test_read_back_in_pieces(meq, shapes, canaries):
