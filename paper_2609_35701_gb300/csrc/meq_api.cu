@@ -460,7 +460,9 @@ struct NsOp {
 //     triangle would force a symmetry that rounding has already broken.
 // Relative error of U~ (numpy emulation, row / column / both / no imbalance):
 //   768 x 2048: 2.57e-3 / 2.76e-3 / 2.88e-3 / 2.25e-3 plain,
-//               2.18e-3 / 2.83e-3 / 2.67e-3 / 2.14e-3 paired.
+//               2.18e-3 / 2.83e-3 / 2.67e-3 / 2.14e-3 paired;
+// on a GB300, 2048 x 5461 with Student-t scales on both sides (5461 x 2048):
+//               2.41e-3 (2.91e-3) plain, 2.09e-3 (2.83e-3) paired.
 bool pairs_allowed(const meq_options& o) {
   meq_options d;
   meq_default_options(&d);
@@ -498,6 +500,11 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
   // except that a fused X_0 is bf16 (written unnormalised by the momentum pass).
   auto dA = [&](int k) { return iter_fp16(o, k); };
   auto dX = [&](int k) { return (fused && k == 0) ? false : iter_fp16(o, k); };
+  // The paired chain holds its s x s matrices times 2^11: their entries stay
+  // below 32 (|P' P| <= a^2 = 11.9), and those that couple a row of tiny norm
+  // to the others keep fp16's full precision down to 3e-8 instead of 6e-5.
+  // (Unscaled, rows at 1e-4 of the typical norm lost up to 8% of U~.)
+  const float gs = pairs ? 2048.f : 1.f;
   int cur = 0;
   auto X = [](int i) { return i ? BUF_X1 : BUF_X0; };
   for (int k = 0; k < K;) {
@@ -513,29 +520,29 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
     gram.gram = true;
     gram.a = gram.b = cx, gram.out = BUF_A;
     gram.in16 = dX(k), gram.out16 = dA(k);
-    gram.scale = 1.0f / (ak * ak), gram.minv_pow = per_matrix ? 2 : 0;
+    gram.scale = gs / (ak * ak), gram.minv_pow = per_matrix ? 2 : 0;
     ops.push_back(gram);
     NsOp poly;  // P = a I + b A + c A^2 (or M = b A + c A^2)
     poly.a = poly.b = BUF_A, poly.out = BUF_P, poly.aux = BUF_A;
     poly.in16 = poly.aux16 = dA(k), poly.out16 = dX(k);
-    poly.c_acc = o.ns_c, poly.c_aux = o.ns_b, poly.c_eye = split ? 0.f : o.ns_a;
+    poly.c_acc = o.ns_c / gs, poly.c_aux = o.ns_b, poly.c_eye = split ? 0.f : o.ns_a * gs;
     ops.push_back(poly);
     NsBuf mul = BUF_P;                      // what multiplies X
     float diag = split ? o.ns_a : 0.f;      // and its identity part, added in the epilogue
     if (pair) {
       NsOp q;  // Q = P A (= M A + a A), in the idle X buffer
-      q.a = BUF_P, q.b = BUF_A, q.out = nx;
+      q.a = BUF_P, q.b = BUF_A, q.out = nx, q.c_acc = 1.0f / gs;
       if (split) q.aux = BUF_A, q.c_aux = o.ns_a;
       ops.push_back(q);
       NsOp a1;  // A' = Q P
-      a1.a = nx, a1.b = BUF_P, a1.out = BUF_A;
+      a1.a = nx, a1.b = BUF_P, a1.out = BUF_A, a1.c_acc = 1.0f / gs;
       if (split) a1.aux = nx, a1.c_aux = o.ns_a;
       ops.push_back(a1);
       NsOp p1 = poly;  // P' (or M') of A'
       p1.out = nx;
       ops.push_back(p1);
       NsOp c;  // P' P, in A's place
-      c.a = nx, c.b = BUF_P, c.out = BUF_A;
+      c.a = nx, c.b = BUF_P, c.out = BUF_A, c.c_acc = 1.0f / gs;
       if (split) {  // less a^2 I: M' M + a (M + M')
         c.aux = nx, c.c_aux = o.ns_a;
         c.aux2 = BUF_P, c.c_aux2 = o.ns_a;
@@ -555,6 +562,7 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
       up.in16 = dX(k);
       up.out16 = u ? true : dX(k + step);
       up.scale = u ? 1.0f / ak : G.alpha / ak;
+      up.c_acc = 1.0f / gs;
       up.minv_pow = per_matrix ? 1 : 0;
       if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
       ops.push_back(up);
@@ -617,7 +625,7 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, const GemmT
   if (dense) ok &= map(&Q.tmB, op.b, op.out_is_x, 64, 64, SW128);
   else ok &= map(&Q.tmB, op.b, op.gram, 64, b_rows, SW128);
   if (Q.sym) ok &= map(&Q.tmO, op.out, false, 32, 32, SW64);
-  Q.scale = op.scale;
+  Q.scale = op.aux == BUF_NONE ? op.scale * op.c_acc : op.scale;  // without aux the epilogue takes one factor
   Q.c_acc = op.c_acc, Q.c_aux = op.c_aux, Q.c_aux2 = op.c_aux2, Q.c_eye = op.c_eye;
   if (op.minv_pow) Q.minv = st->d_ginv + G.mbase, Q.minv_pow = op.minv_pow;
   Q.out_fp16 = op.out16, Q.aux_fp16 = op.aux16;

@@ -99,9 +99,9 @@ struct GemmGroup {
   int32_t sym;            // 1: symmetric s x s output (upper-triangle tiles, mirrored stores)
   int32_t same_ab;        // 1: both operands are the same matrix (a diagonal tile loads it once)
   int32_t trans;          // XLAST: 1 when the weight is the transpose of the NS layout
-  // Epilogue: scale * (c_acc * acc + c_aux * aux) + c_aux2 * aux2 + c_eye * I,
-  // the terms after the first only where aux (aux2) is given; scale is
-  // 1/alpha^2 (Gram), alpha_next/alpha (update), 1/alpha (last update) or 1.
+  // Epilogue: with aux, scale * (c_acc * acc + c_aux * aux) + c_aux2 * aux2 +
+  // c_eye * I (aux2 where given), else scale * acc; scale holds 1/alpha^2
+  // (Gram), alpha_next/alpha (update), 1/alpha (last update) or 1.
   float scale;
   float c_acc, c_aux, c_aux2, c_eye;
   const float* minv;      // iteration 0 with X_0 unnormalised: 1/||H||_F per matrix of the group

@@ -132,6 +132,43 @@ def test_paired_iterations(meq, pair):
     assert all(r["update"] <= PT.UPDATE_TOL for r in rep)
 
 
+@pytest.mark.parametrize("shape,rows", [((600, 4100), True), ((4100, 600), False)], ids=str)
+def test_paired_iterations_keep_tiny_lines(meq, shape, rows):
+    """NS rows of 1e-3 to 1e-4 of the typical norm couple to the others through entries far below
+    fp16's normal range; in the paired iterations every such line of U keeps the precision it has in
+    the plain chain (their relative error to fp64 at most 1.2 times the plain chain's, and the
+    whole matrix's no larger)."""
+    import torch
+
+    m, n = shape
+    g = torch.Generator().manual_seed(61)
+    H = torch.randn(shape, generator=g) * 0.01
+    tiny = torch.logspace(-4, -3, 16)
+    if rows:
+        H[:16] *= tiny[:, None]
+    else:
+        H[:, :16] *= tiny[None, :]
+    X = H.double().cuda() if rows else H.double().cuda().T.contiguous()
+    X = X / X.norm()
+    for _ in range(5):
+        A = X @ X.T
+        X = 3.4445 * X + (-4.7750 * A + 2.0315 * (A @ A)) @ X
+    Hd = H.cuda()
+    errs = []
+    for count, launches in ((8, 17), (1, 15)):
+        opt = meq.MeqMuon([shape] * count)
+        assert opt.ns_gemm_launches_per_step == launches
+        opt.step([torch.zeros(shape, device="cuda") for _ in range(count)], [Hd] * count, 0.0, 0.0, 0.0)
+        U = torch.from_numpy(opt.read_ns_output(0)).cuda().double()
+        U = U if rows else U.T
+        e = (U - X).square().sum(1).sqrt() / X.square().sum(1).sqrt()
+        errs.append((e[:16].cpu().numpy(), float((U - X).norm() / X.norm())))
+        opt.close()
+    (lines, whole), (lines0, whole0) = errs
+    assert whole <= whole0 <= 4e-3
+    assert np.all(lines <= 1.2 * lines0), (lines, lines0)
+
+
 @pytest.mark.parametrize("shapes", [
     [(200, 333), (333, 200), (130, 130)], [(257, 513), (513, 257), (64, 1000), (1000, 64)],
     [(384, 768), (768, 384), (768, 768), (129, 385)], [(63, 65), (64, 64), (65, 63), (128, 129), (192, 200)],
