@@ -373,16 +373,21 @@ __device__ __forceinline__ TileCoord entry_coord(uint4 e) {
   return c;
 }
 
-__device__ __forceinline__ uint32_t pack_half2(float a, float b, int fp16) {
-  if (fp16) {
+// The 16-bit formats are template arguments of the epilogue's loops, chosen by
+// one branch per block: as a runtime flag per pair they took twice the
+// conversions.
+template <bool kFp16>
+__device__ __forceinline__ uint32_t pack_half2(float a, float b) {
+  if (kFp16) {
     __half2 h = __floats2half2_rn(a, b);
     return *reinterpret_cast<uint32_t*>(&h);
   }
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&h);
 }
-__device__ __forceinline__ float2 unpack_half2(uint32_t w, int fp16) {
-  if (fp16) {
+template <bool kFp16>
+__device__ __forceinline__ float2 unpack_half2(uint32_t w) {
+  if (kFp16) {
     __half2 h = *reinterpret_cast<__half2*>(&w);
     return __half22float2(h);
   }
@@ -398,15 +403,38 @@ __device__ __forceinline__ float2 unpack_half2(uint32_t w, int fp16) {
 
 // Row-major 32 x 32 16-bit block, 64-byte rows, 64B swizzle (16-byte chunk k
 // of row r sits at chunk k ^ ((r >> 1) & 3)).
-__device__ __forceinline__ void fill_half_rows(uint8_t* slot, int r, const float* v, int fp16) {
+template <bool kFp16>
+__device__ __forceinline__ void fill_half_rows(uint8_t* slot, int r, const float* v) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     uint4 w;
-    w.x = pack_half2(v[8 * k + 0], v[8 * k + 1], fp16);
-    w.y = pack_half2(v[8 * k + 2], v[8 * k + 3], fp16);
-    w.z = pack_half2(v[8 * k + 4], v[8 * k + 5], fp16);
-    w.w = pack_half2(v[8 * k + 6], v[8 * k + 7], fp16);
+    w.x = pack_half2<kFp16>(v[8 * k + 0], v[8 * k + 1]);
+    w.y = pack_half2<kFp16>(v[8 * k + 2], v[8 * k + 3]);
+    w.z = pack_half2<kFp16>(v[8 * k + 4], v[8 * k + 5]);
+    w.w = pack_half2<kFp16>(v[8 * k + 6], v[8 * k + 7]);
     *reinterpret_cast<uint4*>(slot + r * 64 + ((k ^ ((r >> 1) & 3)) << 4)) = w;
+  }
+}
+__device__ __forceinline__ void fill_half_rows(uint8_t* slot, int r, const float* v, int fp16) {
+  if (fp16) fill_half_rows<true>(slot, r, v);
+  else fill_half_rows<false>(slot, r, v);
+}
+// v = k_acc v + k_aux a (+ k_eye at column j = diag of this lane's row; only
+// the blocks on the diagonal look for it), a being row r of the block in slot.
+template <bool kFp16, bool kDiag>
+__device__ __forceinline__ void add_aux(const uint8_t* slot, int r, float* v, float k_acc, float k_aux, float k_eye,
+                                        int diag) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint4 w = *reinterpret_cast<const uint4*>(slot + r * 64 + ((k ^ ((r >> 1) & 3)) << 4));
+    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float2 a = unpack_half2<kFp16>(ws[h]);
+      const int j = 8 * k + 2 * h;
+      v[j] = fmaf(k_acc, v[j], fmaf(k_aux, a.x, kDiag && j == diag ? k_eye : 0.f));
+      v[j + 1] = fmaf(k_acc, v[j + 1], fmaf(k_aux, a.y, kDiag && j + 1 == diag ? k_eye : 0.f));
+    }
   }
 }
 // The transposed block: element (row j, col r) = v[j] of lane r.
@@ -801,24 +829,20 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           }
           __syncwarp();
           if (ch + 2 < nch) load_aux(col0 + 64);  // in flight while this chunk is processed
-          const int row = row0 + lane;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint4 w = *reinterpret_cast<const uint4*>(slot + lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4));
-            const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              const float2 a2 = unpack_half2(ws[h], G.aux_fp16);
-              const int j = 8 * k + 2 * h;
-              v[j] = fmaf(k_acc, v[j], fmaf(k_aux, a2.x, (col0 + j == row) ? k_eye : 0.f));
-              v[j + 1] = fmaf(k_acc, v[j + 1], fmaf(k_aux, a2.y, (col0 + j + 1 == row) ? k_eye : 0.f));
-            }
+          // row0 and col0 are multiples of 32: the diagonal is lane = j of the block C == R
+          const bool diag = G.sym && C == R;
+          if (G.aux_fp16) {
+            if (diag) add_aux<true, true>(slot, lane, v, k_acc, k_aux, k_eye, lane);
+            else add_aux<true, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
+          } else {
+            if (diag) add_aux<false, true>(slot, lane, v, k_acc, k_aux, k_eye, lane);
+            else add_aux<false, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
           }
           __syncwarp();  // slot free for the output block
           if (G.aux2 != nullptr && lane < rows_valid) {
             // one launch per step has a second addend: each lane reads its own row
             const uint8_t* src = reinterpret_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
-                                 static_cast<int64_t>(row) * G.aux_ld + static_cast<int64_t>(col0) * 2;
+                                 static_cast<int64_t>(row0 + lane) * G.aux_ld + static_cast<int64_t>(col0) * 2;
             const float k_aux2 = G.c_aux2;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -826,7 +850,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
               const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
               for (int h = 0; h < 4; ++h) {
-                const float2 a2 = unpack_half2(ws[h], G.aux_fp16);
+                const float2 a2 = unpack_half2<true>(ws[h]);  // (fp16 chains only)
                 v[8 * k + 2 * h] = fmaf(k_aux2, a2.x, v[8 * k + 2 * h]);
                 v[8 * k + 2 * h + 1] = fmaf(k_aux2, a2.y, v[8 * k + 2 * h + 1]);
               }
