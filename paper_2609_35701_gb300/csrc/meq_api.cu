@@ -670,7 +670,8 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
     (which.back() ? B : A) = chain.back();
   }
   auto joint = [&](size_t i, size_t j) {
-    return i < A.size() && j < B.size() && A[i].mode == B[j].mode && A[i].in16 == B[j].in16;
+    return i < A.size() && j < B.size() && A[i].mode == B[j].mode && A[i].in16 == B[j].in16 &&
+           A[i].aux2 == B[j].aux2;
   };
   // fewest launches from product i of chain A and j of chain B on
   std::vector<std::vector<int>> left(A.size() + 1, std::vector<int>(B.size() + 1, 0));
@@ -705,9 +706,11 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
         const int g = gs[g0 + gi];
         ops.emplace_back(&st->groups[g], &chain[g][at[which[g]]]);
       }
-      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load &&
+      const bool aux2 = ops[0].second->aux2 != BUF_NONE;
+      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load && !aux2 &&
                              launch_cost(ops, small, st->num_sms) < launch_cost(ops, large, st->num_sms);
-      const GemmTile& t = use_small ? small : large;
+      GemmTile t = use_small ? small : large;
+      t.aux2 = aux2;
       for (int gi = 0; gi < P.ngroups; ++gi) {
         const int g = gs[g0 + gi];
         GemmGroup& Q = P.g[gi];

@@ -127,6 +127,7 @@ struct GemmGroup {
 // bn columns.
 struct GemmTile {
   int pair, bn;
+  bool aux2 = false;  // every group has a second addend (256-column tiles only)
 };
 
 // One GEMM launch: one product's shape groups, taken as one tile queue in

@@ -492,7 +492,11 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_reads() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // Every committed store has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-template <int kPair, int kBN>
+// kAux2: the launch adds a second 16-bit matrix in its epilogue (one product
+// of the paired iterations). Its loads are requested ahead of the accumulator;
+// in the kernel that every launch runs, the branch and the registers for them
+// cost all other launches 0.5%.
+template <int kPair, int kBN, bool kAux2>
 __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_constant__ GemmParams p) {
   using C_ = Cfg<kPair, kBN>;
   constexpr int BN = kBN;
@@ -815,6 +819,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         const int col0 = c.tn * BN + ch * 32;
         const int C = c.tn * (BN / 32) + ch;
         float v[32];
+        uint4 aux2[4];
+        if (kAux2) {  // each lane its own row
+          const uint8_t* src = static_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
+                               static_cast<int64_t>(row0 + min(lane, rows_valid - 1)) * G.aux_ld +
+                               static_cast<int64_t>(col0) * 2;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) aux2[k] = __ldg(reinterpret_cast<const uint4*>(src) + k);
+        }
         tmem_ld_32cols(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * BN + ch * 32), v);
         if (G.tma_out) {
           if (lane == 0) bulk_wait_reads();  // both slots free
@@ -839,15 +851,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
             else add_aux<false, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
           }
           __syncwarp();  // slot free for the output block
-          if (G.aux2 != nullptr && lane < rows_valid) {
-            // one launch per step has a second addend: each lane reads its own row
-            const uint8_t* src = reinterpret_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
-                                 static_cast<int64_t>(row0 + lane) * G.aux_ld + static_cast<int64_t>(col0) * 2;
+          if (kAux2) {
             const float k_aux2 = G.c_aux2;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const uint4 w = __ldg(reinterpret_cast<const uint4*>(src + 16 * k));
-              const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+              const uint32_t ws[4] = {aux2[k].x, aux2[k].y, aux2[k].z, aux2[k].w};
 #pragma unroll
               for (int h = 0; h < 4; ++h) {
                 const float2 a2 = unpack_half2<true>(ws[h]);  // (fp16 chains only)
@@ -1027,17 +1035,22 @@ cudaError_t prepare_ns_gemm() {
   auto set = [](auto kernel, int bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  cudaError_t e = set(ns_gemm_kernel<1, 256>, Cfg<1, 256>::SMEM_BYTES);
-  if (e == cudaSuccess) e = set(ns_gemm_kernel<1, 64>, Cfg<1, 64>::SMEM_BYTES);
-  if (e == cudaSuccess) e = set(ns_gemm_kernel<2, 256>, Cfg<2, 256>::SMEM_BYTES);
+  cudaError_t e = set(ns_gemm_kernel<1, 256, false>, Cfg<1, 256>::SMEM_BYTES);
+  if (e == cudaSuccess) e = set(ns_gemm_kernel<1, 256, true>, Cfg<1, 256>::SMEM_BYTES);
+  if (e == cudaSuccess) e = set(ns_gemm_kernel<1, 64, false>, Cfg<1, 64>::SMEM_BYTES);
+  if (e == cudaSuccess) e = set(ns_gemm_kernel<2, 256, false>, Cfg<2, 256>::SMEM_BYTES);
+  if (e == cudaSuccess) e = set(ns_gemm_kernel<2, 256, true>, Cfg<2, 256>::SMEM_BYTES);
   return e;
 }
 
 cudaError_t launch_ns_gemm(const GemmParams& p, const GemmTile& t, int grid, cudaStream_t st) {
   const dim3 g(grid), b(NUM_THREADS);
-  if (t.pair == 2) return launch_pdl(ns_gemm_kernel<2, 256>, g, b, Cfg<2, 256>::SMEM_BYTES, st, 2, p);
-  if (t.bn == 64) return launch_pdl(ns_gemm_kernel<1, 64>, g, b, Cfg<1, 64>::SMEM_BYTES, st, 1, p);
-  return launch_pdl(ns_gemm_kernel<1, 256>, g, b, Cfg<1, 256>::SMEM_BYTES, st, 1, p);
+  if (t.bn == 64) return launch_pdl(ns_gemm_kernel<1, 64, false>, g, b, Cfg<1, 64>::SMEM_BYTES, st, 1, p);
+  if (t.pair == 2)
+    return launch_pdl(t.aux2 ? ns_gemm_kernel<2, 256, true> : ns_gemm_kernel<2, 256, false>, g, b,
+                      Cfg<2, 256>::SMEM_BYTES, st, 2, p);
+  return launch_pdl(t.aux2 ? ns_gemm_kernel<1, 256, true> : ns_gemm_kernel<1, 256, false>, g, b,
+                    Cfg<1, 256>::SMEM_BYTES, st, 1, p);
 }
 
 }  // namespace meq
