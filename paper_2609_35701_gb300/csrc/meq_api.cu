@@ -612,14 +612,12 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, const GemmT
   auto ld = [&](bool is_x) { return (is_x ? G.lp : G.sp) * 2; };
   Q.mode = op.mode;
   Q.idesc = make_idesc(op.in16, dense, tile_m, t.bn);
-  Q.b_mn_major = dense ? 1 : 0;
   Q.count = static_cast<int32_t>(G.count);
   Q.trans = G.trans;
   Q.M = static_cast<int32_t>(op_rows(G, op));
   Q.N = static_cast<int32_t>(op_cols(G, op));
   Q.K = static_cast<int32_t>(op.gram ? G.l : G.s);
   Q.sym = dense ? 0 : 1;
-  Q.tma_out = Q.sym;
   Q.same_ab = (!dense && op.a == op.b) ? 1 : 0;
   bool ok = map(&Q.tmA, op.a, op.gram, 64, 128, SW128);
   if (dense) ok &= map(&Q.tmB, op.b, op.out_is_x, 64, 64, SW128);
@@ -706,11 +704,13 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
         const int g = gs[g0 + gi];
         ops.emplace_back(&st->groups[g], &chain[g][at[which[g]]]);
       }
-      const bool aux2 = ops[0].second->aux2 != BUF_NONE;
-      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load && !aux2 &&
+      int aux = ops[0].second->aux2 != BUF_NONE ? 2 : 0;
+      for (const auto& x : ops)
+        if (x.second->aux != BUF_NONE) aux = std::max(aux, 1);
+      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load && aux < 2 &&
                              launch_cost(ops, small, st->num_sms) < launch_cost(ops, large, st->num_sms);
       GemmTile t = use_small ? small : large;
-      t.aux2 = aux2;
+      t.aux = aux;
       for (int gi = 0; gi < P.ngroups; ++gi) {
         const int g = gs[g0 + gi];
         GemmGroup& Q = P.g[gi];

@@ -119,15 +119,13 @@ struct GemmGroup {
   float* cpart;           // XLAST: NS-column partial sums of squares, [count][ceil(M/32)][N]
   int32_t mode;           // GemmMode of the launch (read from g[0])
   uint32_t idesc;         // tcgen05 instruction descriptor
-  int32_t b_mn_major;     // 1: B operand tile is MN-major (DENSE, XLAST)
-  int32_t tma_out;        // 1: the output leaves by TMA stores through tmO (else 16-byte thread stores)
 };
 
 // Tile variant of a launch: pair 1 or 2 CTAs per tile of 128 * pair rows and
 // bn columns.
 struct GemmTile {
   int pair, bn;
-  bool aux2 = false;  // every group has a second addend (256-column tiles only)
+  int aux = 0;  // addends of the epilogue: 0, 1 (in some group) or 2 (in every group; 256-column tiles only)
 };
 
 // One GEMM launch: one product's shape groups, taken as one tile queue in

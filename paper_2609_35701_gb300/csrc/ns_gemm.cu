@@ -155,23 +155,22 @@ __device__ bool wait_bounded_drain(uint32_t bar, uint32_t parity, int* err, int 
 }
 
 // Warp-uniform bounded wait (all 32 lanes call it; all get the same answer).
-__device__ bool wait_bounded_warp(uint32_t bar, uint32_t parity, int* err, int code, uint64_t timeout_ns) {
+// Every branch is taken by the whole warp: the tcgen05 loads that follow are
+// .sync.aligned, and a warp that a lane-0 branch has split need not be one
+// again there, __syncwarp or not (seen: lane 0 alone at the load, whose
+// results were then used before they had arrived).
+__device__ __forceinline__ bool wait_bounded_warp(uint32_t bar, uint32_t parity, int* err, int code, uint64_t timeout_ns) {
   const unsigned FULL = 0xffffffffu;
   if (__all_sync(FULL, mbar_try_wait(bar, parity))) return true;
   const uint64_t t0 = global_ns();
   for (uint32_t it = 1;; ++it) {
     if (__all_sync(FULL, mbar_try_wait(bar, parity))) return true;
     if ((it & 127u) == 0) {
-      int stop = 0;
-      if ((threadIdx.x & 31) == 0) {
-        if (*reinterpret_cast<volatile int*>(err) != 0) {
-          stop = 1;
-        } else if (global_ns() - t0 > timeout_ns || it >= (1u << 28)) {
-          atomicCAS(err, 0, code);
-          stop = 1;
-        }
+      if (__any_sync(FULL, *reinterpret_cast<volatile int*>(err) != 0)) return false;
+      if (__any_sync(FULL, global_ns() - t0 > timeout_ns || it >= (1u << 28))) {
+        atomicCAS(err, 0, code);  // every lane: the first one writes, the others find it written
+        return false;
       }
-      if (__shfl_sync(FULL, stop, 0)) return false;
     }
   }
 }
@@ -204,7 +203,8 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t ran
   return r;
 }
 __device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // not .aligned: the single-lane roles may leave a warp split
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 // Accumulator release by the epilogue. Only the warp's tcgen05.ld reads must
 // precede it, and tcgen05.wait::ld has already completed them; a release
@@ -212,6 +212,15 @@ __device__ __forceinline__ void cluster_sync_all() {
 // the cluster, which the MMA issuer does not need.
 __device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar_cluster) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
+}
+// The same by lane 0 of a converged warp, as a predicated instruction (no
+// branch: see wait_bounded_warp).
+__device__ __forceinline__ void mbar_arrive_relaxed_cluster_lane0(uint32_t bar_cluster, int lane) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, 0;\n\t"
+      "@p mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar_cluster),
+      "r"(lane)
+      : "memory");
 }
 // Writes a 16-byte tile-ring entry into the peer CTA's shared memory and
 // completes it as a 16-byte transaction on the peer's barrier, which this
@@ -289,19 +298,22 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;
 }
 
-// 32 lanes x 32 consecutive fp32 columns from TMEM.
+// 32 lanes x 32 consecutive fp32 columns from TMEM. The load and its wait are
+// one asm statement: between two, the compiler may place arithmetic on the
+// registers, which hold their old values until the wait.
 __device__ __forceinline__ void tmem_ld_32cols(uint32_t taddr, float* v) {
   uint32_t r[32];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      : "r"(taddr)
+      : "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -330,7 +342,7 @@ __device__ __forceinline__ int find_segment(const GemmParams& p, int t) {
   }
   return lo;
 }
-template <int kPair, int kBN>
+template <int kPair, int kBN, bool kSym>
 __device__ __forceinline__ TileCoord decode_tile(const GemmParams& p, int t) {
   if (p.reverse) t = p.total_tiles - 1 - t;
   const int g = find_segment(p, t);
@@ -341,7 +353,7 @@ __device__ __forceinline__ TileCoord decode_tile(const GemmParams& p, int t) {
   TileCoord c;
   c.g = g;
   c.mat = mat;
-  if (!G.sym) {
+  if (!kSym) {
     const int band = r / (G.band * G.tiles_n);
     const int in = r - band * G.band * G.tiles_n;
     const int rows = min(G.band, G.tiles_m - band * G.band);
@@ -480,11 +492,15 @@ __device__ __forceinline__ void store_block64(const uint8_t* slot, int lane, uin
 // 64-byte swizzle = the staging layout). Rows and columns outside the
 // tensor's extent are not written. The writing threads make their
 // shared-memory stores visible to the TMA unit first (fence.proxy.async).
-__device__ __forceinline__ void tma_store_block(const CUtensorMap* tm, const uint8_t* src, int x, int y, int z) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(tm)),
-               "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z)
-               : "memory");
+// Issued by lane 0 where `on` is set, as a predicated instruction.
+__device__ __forceinline__ void tma_store_block_lane0(const CUtensorMap* tm, const uint8_t* src, int x, int y, int z, int lane,
+                                                      bool on) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\t"
+      "@p cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];\n\t}" ::"l"(
+          reinterpret_cast<uint64_t>(tm)),
+      "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z), "r"(static_cast<int>(on && lane == 0))
+      : "memory");
 }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
@@ -492,15 +508,18 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_reads() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // Every committed store has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// kAux2: the launch adds a second 16-bit matrix in its epilogue (one product
-// of the paired iterations). Its loads are requested ahead of the accumulator;
-// in the kernel that every launch runs, the branch and the registers for them
-// cost all other launches 0.5%.
-template <int kPair, int kBN, bool kAux2>
+// One instance per kind of launch: kMode (GemmMode) and kAux, the 16-bit
+// matrices added in the epilogue (0: none; 1: one, in some groups; 2: two, in
+// every group, one product of the paired iterations). As runtime values the
+// operand layout, the output path and the addends cost the producer, the MMA
+// issuer and the epilogue registers and branches in every launch; the chains
+// of dependent instructions are what small launches and launch tails wait for.
+template <int kPair, int kBN, int kMode, int kAux>
 __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_constant__ GemmParams p) {
   using C_ = Cfg<kPair, kBN>;
   constexpr int BN = kBN;
   constexpr uint32_t TMEM_COLS = C_::TMEM_COLS;
+  constexpr bool kSym = kMode == MODE_SYM;  // K-major B, upper-triangle tiles, TMA stores
   constexpr int STAGES = C_::STAGES;
   constexpr int STAGE_BYTES = C_::STAGE_BYTES;
   constexpr int TILE_M = C_::TILE_M;
@@ -552,7 +571,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
     for (int g = 0; g < p.ngroups; ++g) {
       prefetch_tmap(&p.g[g].tmA);
       prefetch_tmap(&p.g[g].tmB);
-      if (p.g[g].sym) prefetch_tmap(&p.g[g].tmO);
+      if (kSym) prefetch_tmap(&p.g[g].tmO);
     }
   }
   if (warp == 1) {
@@ -609,6 +628,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
     return true;
   };
 
+  // The same for a whole epilogue warp, without a branch that splits it.
+  auto sched_take_warp = [&](int n, uint4& e) -> bool {
+    const int i = n & (SCHED_D - 1);
+    if (!wait_bounded_warp(SFULL_BAR(i), (n / SCHED_D) & 1, err, DEV_TIMEOUT_SCHED_TAKE, tmo)) return false;
+    e = ld_shared_v4(ring + 16u * i);
+    __syncwarp();  // every lane has read it
+    mbar_arrive_relaxed_cluster_lane0((kPair == 2 && !leader) ? map_to_rank(SEMPTY_BAR(i), 0) : SEMPTY_BAR(i), lane);
+    return true;
+  };
+
   if (warp == 0) {
     if (lane == 0) {
       // ---------------------------------------------------------------- TMA producer
@@ -625,16 +654,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         const TileCoord c = entry_coord(e);
         const GemmGroup& G = p.g[c.g];
         const int nk = static_cast<int>(e.w & 0xFFFFu);
-        // Mode, descriptor and B layout are per launch: reading them at a
-        // fixed index keeps them launch-uniform for the compiler (measured:
-        // 2% of the step).
-        const int b_mn_major = p.g[0].b_mn_major;
         const int arow = c.tm * TILE_M + static_cast<int>(rank) * BM;
         const int bcol = c.tn * BN + static_cast<int>(rank) * C_::BN_LOCAL;
         // A diagonal tile of a symmetric product (X X^T, A A) has each CTA's
         // B half equal to its A half (same rows of the same buffer, same box):
         // only A is loaded, and the MMA reads it as B too.
-        const bool b_is_a = (e.w >> 16) & 1u;
+        const bool b_is_a = kSym && ((e.w >> 16) & 1u);
         for (int kb = 0; kb < nk; ++kb) {
           if (!wait_bounded(EMPTY_BAR(stage), phase ^ 1u, err, DEV_TIMEOUT_PRODUCER, tmo)) {
             ok = false;
@@ -645,7 +670,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           if (kPair == 1) {
             mbar_expect_tx(FULL_BAR(stage), STAGE_BYTES);
             tma_load_3d(sa, &G.tmA, FULL_BAR(stage), kb * BK, arow, c.mat);
-            if (!b_mn_major) {
+            if (kSym) {
               tma_load_3d(sb, &G.tmB, FULL_BAR(stage), kb * BK, bcol, c.mat);
             } else {
 #pragma unroll
@@ -664,7 +689,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
               tma_load_3d_pair(sa, &G.tmA, fb, kb * BK, arow, c.mat);
               if (b_is_a) {
                 // B is this stage's A
-              } else if (!b_mn_major) {
+              } else if (kSym) {
                 tma_load_3d_pair(sb, &G.tmB, fb, kb * BK, bcol, c.mat);
               } else {
 #pragma unroll
@@ -701,11 +726,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         uint4 e;
         if (!sched_take(n, e) || static_cast<int>(e.x) >= p.total_tiles) break;
         const int nk = static_cast<int>(e.w & 0xFFFFu);
-        const int b_mn_major = p.g[0].b_mn_major;
+        // the descriptor is per launch: read at a fixed index, it stays uniform
         const uint32_t idesc = p.g[0].idesc;
-        const uint32_t b_lbo = b_mn_major ? (64u * BK * 2u) : 16u;
+        constexpr uint32_t b_lbo = kSym ? 16u : (64u * BK * 2u);
         // diagonal tile of a symmetric product: B is read from the A half (the producer loads A only)
-        const bool b_is_a = (e.w >> 16) & 1u;
+        const bool b_is_a = kSym && ((e.w >> 16) & 1u);
         if (!wait_bounded(TEMPTY_BAR(acc), acc_phase ^ 1u, err, DEV_TIMEOUT_MMA_TMEM, tmo)) break;
         tc_fence_after();
         const uint32_t d = tmem_base + static_cast<uint32_t>(acc * BN);
@@ -720,8 +745,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
 #pragma unroll
           for (int k = 0; k < BK / UK; ++k) {
             const uint64_t adesc = smem_desc(sa + k * (UK * 2), 16u, 1024u);
-            const uint64_t bdesc = b_mn_major ? smem_desc(sb + k * (UK * 128), b_lbo, 1024u)
-                                                : smem_desc(sb + k * (UK * 2), 16u, 1024u);
+            const uint64_t bdesc = smem_desc(sb + k * (kSym ? UK * 2 : UK * 128), b_lbo, 1024u);
             if (kPair == 2) tc_mma_pair(d, adesc, bdesc, idesc, (kb > 0 || k > 0) ? 1u : 0u);
             else tc_mma(d, adesc, bdesc, idesc, (kb > 0 || k > 0) ? 1u : 0u);
           }
@@ -768,24 +792,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
     const uint32_t tempty_target0 = (kPair == 2 && !leader) ? map_to_rank(TEMPTY_BAR(0), 0) : TEMPTY_BAR(0);
     const uint32_t tempty_target1 = (kPair == 2 && !leader) ? map_to_rank(TEMPTY_BAR(1), 0) : TEMPTY_BAR(1);
     for (int n = 0;; ++n) {
-      uint4 e = make_uint4(0u, 0u, 0u, 0u);
-      int got = 1;
-      if (lane == 0) got = sched_take(n, e) ? 1 : 0;
-      got = __shfl_sync(0xffffffffu, got, 0);
-      e.x = __shfl_sync(0xffffffffu, e.x, 0);
-      e.y = __shfl_sync(0xffffffffu, e.y, 0);
-      e.z = __shfl_sync(0xffffffffu, e.z, 0);
-      if (!got || static_cast<int>(e.x) >= p.total_tiles) break;
+      uint4 e;
+      if (!sched_take_warp(n, e) || static_cast<int>(e.x) >= p.total_tiles) break;
       const TileCoord c = entry_coord(e);
       const GemmGroup& G = p.g[c.g];
-      const int mode = p.g[0].mode;  // one mode per launch (a launch-uniform read)
-      const bool has_aux = G.aux != nullptr;
+      const bool has_aux = kAux == 2 || (kAux == 1 && G.aux != nullptr);
       const int row0 = c.tm * TILE_M + static_cast<int>(rank) * BM + q * 32;
       const int R = row0 / 32;  // 32-row block index
       const int rows_valid = min(32, G.M - row0);
       float rsum = 0.f;            // XLAST: this lane's row, sum of squares over the tile
       const int nch = min(BN / 32, (G.N - c.tn * BN + 31) / 32);
-      int ch0 = G.sym ? max(0, R - c.tn * (BN / 32)) : 0;  // blocks strictly below the diagonal come from mirrors
+      int ch0 = kSym ? max(0, R - c.tn * (BN / 32)) : 0;  // blocks strictly below the diagonal come from mirrors
       if ((ch0 & 1) != half) ++ch0;                // this warp's chunks: ch % 2 == half
       if (row0 >= G.M) ch0 = nch;
       uint8_t* outm = static_cast<uint8_t*>(G.out) + static_cast<int64_t>(c.mat) * G.out_mstride;
@@ -820,18 +837,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         const int C = c.tn * (BN / 32) + ch;
         float v[32];
         uint4 aux2[4];
-        if (kAux2) {  // each lane its own row
+        if (kAux == 2) {  // each lane its own row
           const uint8_t* src = static_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
                                static_cast<int64_t>(row0 + min(lane, rows_valid - 1)) * G.aux_ld +
                                static_cast<int64_t>(col0) * 2;
 #pragma unroll
           for (int k = 0; k < 4; ++k) aux2[k] = __ldg(reinterpret_cast<const uint4*>(src) + k);
         }
+        __syncwarp();  // the load is warp-wide (.sync.aligned)
         tmem_ld_32cols(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * BN + ch * 32), v);
-        if (G.tma_out) {
-          if (lane == 0) bulk_wait_reads();  // both slots free
+        if (kSym) {
+          bulk_wait_reads();  // both slots free (only lane 0 has stores to wait for)
+          __syncwarp();
         }
-        __syncwarp();
         if (has_aux) {
           const float k_acc = sc * G.c_acc, k_aux = sc * G.c_aux, k_eye = G.c_eye;
 #pragma unroll
@@ -842,7 +860,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           __syncwarp();
           if (ch + 2 < nch) load_aux(col0 + 64);  // in flight while this chunk is processed
           // row0 and col0 are multiples of 32: the diagonal is lane = j of the block C == R
-          const bool diag = G.sym && C == R;
+          const bool diag = kSym && C == R;
           if (G.aux_fp16) {
             if (diag) add_aux<true, true>(slot, lane, v, k_acc, k_aux, k_eye, lane);
             else add_aux<true, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
@@ -851,7 +869,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
             else add_aux<false, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
           }
           __syncwarp();  // slot free for the output block
-          if (kAux2) {
+          if (kAux == 2) {
             const float k_aux2 = G.c_aux2;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -868,7 +886,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] *= sc;
         }
-        if (mode == MODE_XLAST) {
+        if (kMode == MODE_XLAST) {
           // U is stored as fp16(kUScale U). The sums of squares are taken from
           // those stored values and scaled back by kUScale^-2 (a power of
           // two) when written, so the statistics describe the U the update
@@ -924,40 +942,36 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
             store_block64(slot_t, lane, outm + static_cast<int64_t>(col0) * G.out_ld + row0 * 2, G.out_ld,
                           min(32, G.N - col0), min(4, (G.M - row0 + 7) / 8));
           }
-        } else if (!G.tma_out) {
+        } else if (!kSym) {
           // X rows are padded to a multiple of 64 elements: whole 32-column blocks stay inside them
           fill_half_rows(slot, lane, v, G.out_fp16);
           __syncwarp();
           store_block64(slot, lane, outm + static_cast<int64_t>(row0) * G.out_ld + col0 * 2, G.out_ld, rows_valid, 4);
         } else {
           fill_half_rows(slot, lane, v, G.out_fp16);
-          const bool mirror = G.sym && C > R;  // strictly above the diagonal: also store the transpose
+          const bool mirror = C > R;  // strictly above the diagonal: also store the transpose
           if (mirror) {
             __syncwarp();
             transpose_slot(slot, slot_t, lane);
           }
           fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) {
-            tma_store_block(&G.tmO, slot, col0, row0, c.mat);
-            if (mirror) tma_store_block(&G.tmO, slot_t, row0, col0, c.mat);
-            bulk_commit();
-          }
+          tma_store_block_lane0(&G.tmO, slot, col0, row0, c.mat, lane, true);
+          tma_store_block_lane0(&G.tmO, slot_t, row0, col0, c.mat, lane, mirror);
+          bulk_commit();
         }
         __syncwarp();  // reconverge before the next warp-wide tcgen05.ld
       }
-      if (mode == MODE_XLAST && row0 + lane < G.M)  // one partial per (tile column, half)
+      if (kMode == MODE_XLAST && row0 + lane < G.M)  // one partial per (tile column, half)
         G.rpart[(static_cast<int64_t>(c.mat) * G.tiles_n * 2 + c.tn * 2 + half) * G.M + row0 + lane] = rsum * kUInvScale2;
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive_relaxed_cluster(kPair == 2 ? (acc == 0 ? tempty_target0 : tempty_target1) : TEMPTY_BAR(acc));
-      }
+      mbar_arrive_relaxed_cluster_lane0(kPair == 2 ? (acc == 0 ? tempty_target0 : tempty_target1) : TEMPTY_BAR(acc), lane);
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
     // The outputs are in global memory before the CTA leaves.
-    if (lane == 0) bulk_wait_all();
+    bulk_wait_all();
     __syncwarp();
   } else if (warp == SCHED_WARP) {
     if (lane == 0 && leader) {
@@ -972,10 +986,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         }
         uint4 e = make_uint4(static_cast<uint32_t>(t), 0u, 0u, 0u);
         if (t < p.total_tiles) {
-          const TileCoord c = decode_tile<kPair, kBN>(p, t);
+          const TileCoord c = decode_tile<kPair, kBN, kSym>(p, t);
           const GemmGroup& G = p.g[c.g];
           const int nk = (G.K + BK - 1) / BK;
-          const bool b_is_a = kPair == 2 && G.same_ab && c.tm * TILE_M == c.tn * BN;
+          const bool b_is_a = kSym && kPair == 2 && G.same_ab && c.tm * TILE_M == c.tn * BN;
           e.y = static_cast<uint32_t>(c.mat);
           e.z = static_cast<uint32_t>(c.g) | (static_cast<uint32_t>(c.tm) << 4) | (static_cast<uint32_t>(c.tn) << 18);
           e.w = static_cast<uint32_t>(nk) | (b_is_a ? 0x10000u : 0u);
@@ -1031,26 +1045,39 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
 
 int ns_gemm_smem_bytes(int pair) { return pair == 2 ? Cfg<2, 256>::SMEM_BYTES : Cfg<1, 256>::SMEM_BYTES; }
 
+// f(kernel, shared-memory bytes) of one tile variant's instance for a launch.
+template <int kPair, int kBN, typename F>
+static cudaError_t with_kernel(int mode, int aux, F f) {
+  constexpr int bytes = Cfg<kPair, kBN>::SMEM_BYTES;
+  if (mode == MODE_XLAST) return f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 0>, bytes);
+  if (mode == MODE_DENSE)
+    return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 0>, bytes);
+  if constexpr (kBN == 256)
+    if (aux == 2) return f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 2>, bytes);
+  return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 0>, bytes);
+}
+
 cudaError_t prepare_ns_gemm() {
   auto set = [](auto kernel, int bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  cudaError_t e = set(ns_gemm_kernel<1, 256, false>, Cfg<1, 256>::SMEM_BYTES);
-  if (e == cudaSuccess) e = set(ns_gemm_kernel<1, 256, true>, Cfg<1, 256>::SMEM_BYTES);
-  if (e == cudaSuccess) e = set(ns_gemm_kernel<1, 64, false>, Cfg<1, 64>::SMEM_BYTES);
-  if (e == cudaSuccess) e = set(ns_gemm_kernel<2, 256, false>, Cfg<2, 256>::SMEM_BYTES);
-  if (e == cudaSuccess) e = set(ns_gemm_kernel<2, 256, true>, Cfg<2, 256>::SMEM_BYTES);
-  return e;
+  for (int mode : {MODE_SYM, MODE_DENSE, MODE_XLAST})
+    for (int aux = 0; aux < 3; ++aux) {
+      cudaError_t e = with_kernel<1, 256>(mode, aux, set);
+      if (e == cudaSuccess) e = with_kernel<1, 64>(mode, aux, set);
+      if (e == cudaSuccess) e = with_kernel<2, 256>(mode, aux, set);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 cudaError_t launch_ns_gemm(const GemmParams& p, const GemmTile& t, int grid, cudaStream_t st) {
-  const dim3 g(grid), b(NUM_THREADS);
-  if (t.bn == 64) return launch_pdl(ns_gemm_kernel<1, 64, false>, g, b, Cfg<1, 64>::SMEM_BYTES, st, 1, p);
-  if (t.pair == 2)
-    return launch_pdl(t.aux2 ? ns_gemm_kernel<2, 256, true> : ns_gemm_kernel<2, 256, false>, g, b,
-                      Cfg<2, 256>::SMEM_BYTES, st, 2, p);
-  return launch_pdl(t.aux2 ? ns_gemm_kernel<1, 256, true> : ns_gemm_kernel<1, 256, false>, g, b,
-                    Cfg<1, 256>::SMEM_BYTES, st, 1, p);
+  auto run = [&](auto kernel, int bytes) {
+    return launch_pdl(kernel, dim3(grid), dim3(NUM_THREADS), bytes, st, t.pair, p);
+  };
+  const int mode = p.g[0].mode;
+  if (t.bn == 64) return with_kernel<1, 64>(mode, t.aux, run);
+  return t.pair == 2 ? with_kernel<2, 256>(mode, t.aux, run) : with_kernel<1, 256>(mode, t.aux, run);
 }
 
 }  // namespace meq
