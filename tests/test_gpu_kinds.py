@@ -103,6 +103,15 @@ def test_folded_statistics(meq, shapes, kinds):
     run_kinds(meq, W.custom_workload(shapes, pattern="both", seed=53, kinds=kinds), 2)
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 6, 7, 9, 130, 1367, 4099])
+def test_update_of_odd_rows(meq, n):
+    """Rows that are no multiple of four: groups of four that straddle one or more row ends, both
+    parities of the column in U's rows, matrices of no multiple of four elements, each kind."""
+    shapes = [(37, n), (5, n), (1, n)]
+    kinds = [O.HIDDEN, O.REMAINING_2D, O.VECTOR]
+    run_kinds(meq, W.custom_workload(shapes, pattern="both", seed=n, kinds=kinds), 2)
+
+
 @pytest.mark.parametrize("n", [1, 3, 4, 31, 128, 255, 256, 260, 512, 513, 767, 768, 1000, 1021, 1024])
 def test_remaining_2d_in_one_pass(meq, n):
     """Rows of up to 1024 entries: every width class and its edges, aligned and not, with slabs
