@@ -553,20 +553,17 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
       ops.push_back(c);
       mul = BUF_A;
     }
-    for (int w = 0; w < 2; ++w) {  // U = P X, X' = P X
-      const bool u = w == 0;
-      if (u ? !(last || trajectory) : last) continue;
-      NsOp up;
-      up.mode = u ? MODE_XLAST : MODE_DENSE;
-      up.a = mul, up.b = cx, up.out = u ? BUF_NONE : nx, up.out_is_x = true;
-      up.in16 = dX(k);
-      up.out16 = u ? true : dX(k + step);
-      up.scale = u ? 1.0f / ak : G.alpha / ak;
-      up.c_acc = 1.0f / gs;
-      up.minv_pow = per_matrix ? 1 : 0;
-      if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
-      ops.push_back(up);
-    }
+    NsOp up;  // X' = P X, or U = P X (trajectory: both at once)
+    up.mode = last || trajectory ? MODE_XLAST : MODE_DENSE;
+    up.a = mul, up.b = cx, up.out = last ? BUF_NONE : nx, up.out_is_x = true;
+    up.in16 = dX(k);
+    up.out16 = last ? true : dX(k + step);
+    up.scale = up.mode == MODE_XLAST ? 1.0f / ak : G.alpha / ak;
+    up.c_acc = 1.0f / gs;
+    up.minv_pow = per_matrix ? 1 : 0;
+    if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
+    if (up.mode == MODE_XLAST && !last) up.c_aux = G.alpha;
+    ops.push_back(up);
     cur ^= 1;
     k += step;
   }
@@ -633,6 +630,7 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, const GemmT
     Q.out = base[op.out], Q.out_ld = ld(op.out_is_x), Q.out_mstride = G.s * ld(op.out_is_x);
   } else if (op.mode == MODE_XLAST) {
     Q.out = st->d_u + G.u_base, Q.out_ld = G.un * 2, Q.out_mstride = G.m * G.un * 2;
+    if (op.out != BUF_NONE) Q.out2 = base[op.out], Q.out2_ld = ld(true), Q.out2_mstride = G.s * ld(true);
     Q.rpart = G.rpart;
     Q.cpart = st->d_parts + G.cpart_base;
   }
@@ -706,7 +704,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
       }
       int aux = ops[0].second->aux2 != BUF_NONE ? 2 : 0;
       for (const auto& x : ops)
-        if (x.second->aux != BUF_NONE) aux = std::max(aux, 1);
+        if (x.second->aux != BUF_NONE || (x.second->mode == MODE_XLAST && x.second->out != BUF_NONE)) aux = std::max(aux, 1);
       const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load && aux < 2 &&
                              launch_cost(ops, small, st->num_sms) < launch_cost(ops, large, st->num_sms);
       GemmTile t = use_small ? small : large;
@@ -1453,11 +1451,11 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
   e = launch_row_col_stats(h, rows, cols, eps, o.tie_atol, 1, parts, r, c, &t[0].gamma_r, &t[0].direction, s, &what);
   if (e != cudaSuccess) ms = cuda_fail(nullptr, e, what);
   // k >= 1: one chain of NS products over a one-matrix state fed H with no
-  // momentum history and mu = 0 (so its NS input is H). After each iteration
-  // U = X_k is written as the step writes it and its statistics go to t[k];
-  // then X_k itself, for the next iteration. (One state per k took 3 (1 + ..
-  // + steps) products and as many set-ups: 14.2 ms for 20 iterations of a
-  // 1024 x 2736 matrix, 1.7 ms this way.)
+  // momentum history and mu = 0 (so its NS input is H). The update of each
+  // iteration writes U = X_k as the step writes it, whose statistics go to
+  // t[k], and beside it X_k for the next iteration. (One state per k took
+  // 3 (1 + .. + steps) products and as many set-ups: 14.1 ms for 20 iterations
+  // of a 1024 x 2736 matrix, 1.35 ms this way.)
   meq_state* st = nullptr;
   if (ms == MEQ_OK && steps > 0) {
     o.ns_steps = steps;

@@ -111,6 +111,8 @@ struct GemmGroup {
   void* out;              // DENSE: 16-bit output; XLAST: fp16(kUScale U) in the weight's layout
   int64_t out_ld;         // DENSE / XLAST: output row stride in bytes
   int64_t out_mstride;    // DENSE / XLAST: output matrix stride in bytes
+  void* out2;             // XLAST with aux 1: 16-bit X' (c_aux * U), its row and matrix strides in bytes
+  int64_t out2_ld, out2_mstride;
   const void* aux;        // 16-bit matrix the epilogue adds (same rows and columns as the output), or null
   const void* aux2;       // a second one, in aux's layout, or null
   int64_t aux_ld;         // bytes
@@ -125,7 +127,8 @@ struct GemmGroup {
 // bn columns.
 struct GemmTile {
   int pair, bn;
-  int aux = 0;  // addends of the epilogue: 0, 1 (in some group) or 2 (in every group; 256-column tiles only)
+  int aux = 0;  // addends of the epilogue: 0, 1 (in some group) or 2 (in every group; 256-column tiles only);
+                // XLAST: 1 when X' is written too
 };
 
 // One GEMM launch: one product's shape groups, taken as one tile queue in

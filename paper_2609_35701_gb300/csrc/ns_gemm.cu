@@ -510,7 +510,8 @@ __device__ __forceinline__ void bulk_wait_reads() { asm volatile("cp.async.bulk.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // One instance per kind of launch: kMode (GemmMode) and kAux, the 16-bit
 // matrices added in the epilogue (0: none; 1: one, in some groups; 2: two, in
-// every group, one product of the paired iterations). As runtime values the
+// every group, one product of the paired iterations; of MODE_XLAST, 1: X' is
+// written beside U). As runtime values the
 // operand layout, the output path and the addends cost the producer, the MMA
 // issuer and the epilogue registers and branches in every launch; the chains
 // of dependent instructions are what small launches and launch tails wait for.
@@ -519,6 +520,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
   using C_ = Cfg<kPair, kBN>;
   constexpr int BN = kBN;
   constexpr uint32_t TMEM_COLS = C_::TMEM_COLS;
+  constexpr bool kLast = kMode == MODE_XLAST;
   constexpr bool kSym = kMode == MODE_SYM;  // K-major B, upper-triangle tiles, TMA stores
   constexpr int STAGES = C_::STAGES;
   constexpr int STAGE_BYTES = C_::STAGE_BYTES;
@@ -796,7 +798,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       if (!sched_take_warp(n, e) || static_cast<int>(e.x) >= p.total_tiles) break;
       const TileCoord c = entry_coord(e);
       const GemmGroup& G = p.g[c.g];
-      const bool has_aux = kAux == 2 || (kAux == 1 && G.aux != nullptr);
+      const bool has_aux = kAux == 2 || (kAux == 1 && !kLast && G.aux != nullptr);
       const int row0 = c.tm * TILE_M + static_cast<int>(rank) * BM + q * 32;
       const int R = row0 / 32;  // 32-row block index
       const int rows_valid = min(32, G.M - row0);
@@ -886,7 +888,20 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] *= sc;
         }
-        if (kMode == MODE_XLAST) {
+        if (kLast && kAux == 1) {
+          // the CV trajectory: X' too, in the NS layout, for the next iteration
+          // (X' = alpha' U, alpha' a power of two, so this is the value an
+          // update launch of its own would round)
+          float x[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) x[j] = v[j] * G.c_aux;
+          fill_half_rows(slot, lane, x, G.out_fp16);
+          __syncwarp();
+          store_block64(slot, lane, static_cast<uint8_t*>(G.out2) + static_cast<int64_t>(c.mat) * G.out2_mstride +
+                                        static_cast<int64_t>(row0) * G.out2_ld + col0 * 2, G.out2_ld, rows_valid, 4);
+          __syncwarp();
+        }
+        if (kLast) {
           // U is stored as fp16(kUScale U). The sums of squares are taken from
           // those stored values and scaled back by kUScale^-2 (a power of
           // two) when written, so the statistics describe the U the update
@@ -962,7 +977,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         }
         __syncwarp();  // reconverge before the next warp-wide tcgen05.ld
       }
-      if (kMode == MODE_XLAST && row0 + lane < G.M)  // one partial per (tile column, half)
+      if (kLast && row0 + lane < G.M)  // one partial per (tile column, half)
         G.rpart[(static_cast<int64_t>(c.mat) * G.tiles_n * 2 + c.tn * 2 + half) * G.M + row0 + lane] = rsum * kUInvScale2;
       tc_fence_before();
       __syncwarp();
@@ -1049,7 +1064,8 @@ int ns_gemm_smem_bytes(int pair) { return pair == 2 ? Cfg<2, 256>::SMEM_BYTES : 
 template <int kPair, int kBN, typename F>
 static cudaError_t with_kernel(int mode, int aux, F f) {
   constexpr int bytes = Cfg<kPair, kBN>::SMEM_BYTES;
-  if (mode == MODE_XLAST) return f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 0>, bytes);
+  if (mode == MODE_XLAST)
+    return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 0>, bytes);
   if (mode == MODE_DENSE)
     return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 0>, bytes);
   if constexpr (kBN == 256)
