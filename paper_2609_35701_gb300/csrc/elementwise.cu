@@ -312,19 +312,30 @@ __global__ void __launch_bounds__(kThreads) x0norm_kernel(const MatInfo* __restr
                                                          const float* __restrict__ partials,
                                                          float* __restrict__ ginv, int* __restrict__ nonfinite) {
   pdl_allow_dependents();
-  pdl_wait_predecessor();
   __shared__ float shf[32];
   const MatInfo& M = mats[blockIdx.x];
-  if (M.kind != KIND_HIDDEN) return;
+  if (M.kind != KIND_HIDDEN) {
+    pdl_wait_predecessor();  // every block of the grid waits: its completion stands for its predecessors'
+    return;
+  }
   const int64_t nblk = M.trans ? ((M.m + kCastTile - 1) / kCastTile) * ((M.n + kCastTile - 1) / kCastTile)
                                : (M.m * M.n + kChunk - 1) / kChunk;
-  float acc = 0.f;
-  for (int64_t c = threadIdx.x; c < nblk; c += kThreads) acc += partials[M.xblk_begin + c];
-  const float total = block_sum_f32(acc, shf);
+  const float* part = partials + M.xblk_begin;
+  float* out = ginv + groups[M.group].mbase + M.gidx;
+  pdl_wait_predecessor();
+  float acc[1] = {0.f};
+  int64_t c = threadIdx.x;
+  for (; c + 3 * kThreads < nblk; c += 4 * kThreads) {
+    const float x0 = part[c], x1 = part[c + kThreads], x2 = part[c + 2 * kThreads], x3 = part[c + 3 * kThreads];
+    acc[0] += x0, acc[0] += x1, acc[0] += x2, acc[0] += x3;
+  }
+  for (; c < nblk; c += kThreads) acc[0] += part[c];
+  block_sum_multi<1>(acc, shf);
+  const float total = acc[0];
   if (threadIdx.x == 0) {
     const float nrm = sqrtf(total);
     if (!isfinite(total)) atomicCAS(nonfinite, 0, static_cast<int>(blockIdx.x) + 1);  // first non-finite entry, 1-based
-    ginv[groups[M.group].mbase + M.gidx] = nrm > 0.f ? 1.0f / nrm : 0.f;
+    *out = nrm > 0.f ? 1.0f / nrm : 0.f;
   }
 }
 
@@ -743,14 +754,15 @@ __global__ void __launch_bounds__(kFinThreads, 2) finalize_kernel(const MatInfo*
                                                                unsigned long long* __restrict__ dircount,
                                                                int* __restrict__ nonfinite, int folded) {
   pdl_allow_dependents();
-  pdl_wait_predecessor();
   __shared__ float shf[6 * 32];
   const MatInfo& M = mats[blockIdx.x];
-  const float delta = sc->eps;
+  const float delta = sc->eps;  // uploaded before the step's first kernel
+  const FoldVec v0 = fold_vec(M, 0, parts, rvec, cvec), v1 = fold_vec(M, 1, parts, rvec, cvec);
   float* r = rvec + M.vec_off;
   float* c = cvec + M.vec_off;
   float* s = svec + M.vec_off;
   const float inv_n = 1.0f / static_cast<float>(M.n);
+  pdl_wait_predecessor();
   if (M.kind == KIND_VECTOR) {
     if (threadIdx.x == 0) {
       if (!isfinite(r[0])) atomicCAS(nonfinite, 0, static_cast<int>(blockIdx.x) + 1);
@@ -768,7 +780,7 @@ __global__ void __launch_bounds__(kFinThreads, 2) finalize_kernel(const MatInfo*
       for (int64_t i = threadIdx.x; i < M.m; i += blockDim.x)
         two_sided_row(M, i, static_cast<int>(blockIdx.x), delta, rvec, svec, nonfinite);
     for (int which = M.kind == KIND_HIDDEN ? 0 : 1; which < 2; ++which) {
-      const FoldVec v = fold_vec(M, which, parts, rvec, cvec);
+      const FoldVec v = which == 0 ? v0 : v1;
       for (int64_t j = threadIdx.x; j < v.len; j += blockDim.x) {
         const float rms = sqrtf(strided_sum8(v.parts + j, 0, v.count, v.len) * v.inv);
         v.dst[j] = rms;
