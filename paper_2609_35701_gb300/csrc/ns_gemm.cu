@@ -431,6 +431,14 @@ __device__ __forceinline__ void fill_half_rows(uint8_t* slot, int r, const float
   if (fp16) fill_half_rows<true>(slot, r, v);
   else fill_half_rows<false>(slot, r, v);
 }
+// Two fp32 operations in one instruction, each rounded as fmaf rounds.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(d)
+      : "l"(*reinterpret_cast<uint64_t*>(&a)), "l"(*reinterpret_cast<uint64_t*>(&b)), "l"(*reinterpret_cast<uint64_t*>(&c)));
+  return *reinterpret_cast<float2*>(&d);
+}
 // v = k_acc v + k_aux a (+ k_eye at column j = diag of this lane's row; only
 // the blocks on the diagonal look for it), a being row r of the block in slot.
 template <bool kFp16, bool kDiag>
@@ -444,8 +452,10 @@ __device__ __forceinline__ void add_aux(const uint8_t* slot, int r, float* v, fl
     for (int h = 0; h < 4; ++h) {
       const float2 a = unpack_half2<kFp16>(ws[h]);
       const int j = 8 * k + 2 * h;
-      v[j] = fmaf(k_acc, v[j], fmaf(k_aux, a.x, kDiag && j == diag ? k_eye : 0.f));
-      v[j + 1] = fmaf(k_acc, v[j + 1], fmaf(k_aux, a.y, kDiag && j + 1 == diag ? k_eye : 0.f));
+      const float2 eye = make_float2(kDiag && j == diag ? k_eye : 0.f, kDiag && j + 1 == diag ? k_eye : 0.f);
+      const float2 t = fma2(make_float2(k_aux, k_aux), a, eye);
+      const float2 r = fma2(make_float2(k_acc, k_acc), make_float2(v[j], v[j + 1]), t);
+      v[j] = r.x, v[j + 1] = r.y;
     }
   }
 }
