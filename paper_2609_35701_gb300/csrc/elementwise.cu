@@ -675,8 +675,8 @@ __device__ __forceinline__ FoldVec fold_vec(const MatInfo& M, int which, const f
   if (M.kind == KIND_HIDDEN) {
     const bool cols = (which == 1) != (M.trans != 0);  // which: 0 NS rows, 1 NS columns
     v.parts = parts + (which == 0 ? M.rpart_off : M.cpart_off);
-    v.count = which == 0 ? M.rparts : (M.s + 31) / 32;
-    v.len = which == 0 ? M.s : M.l;
+    v.count = which == 0 ? M.rparts : (M.s() + 31) / 32;
+    v.len = which == 0 ? M.s() : M.l();
     v.dst = (cols ? cvec : rvec) + M.vec_off;
     v.inv = 1.0f / static_cast<float>(cols ? M.m : M.n);
   } else {
@@ -715,7 +715,7 @@ __global__ void __launch_bounds__(kThreads) fold_kernel(const MatInfo* __restric
   const int mi = find_mat(mats, nmat, blk, 6);
   const MatInfo& M = mats[mi];
   const int64_t lb = blk - M.fold_begin;
-  const int64_t first = M.kind == KIND_HIDDEN ? (M.s + kFoldCols - 1) / kFoldCols : (M.m + kThreads - 1) / kThreads;
+  const int64_t first = M.kind == KIND_HIDDEN ? (M.s() + kFoldCols - 1) / kFoldCols : (M.m + kThreads - 1) / kThreads;
   const int which = lb >= first ? 1 : 0;
   if (M.kind == KIND_TWO_SIDED && which == 0) {
     pdl_wait_predecessor();

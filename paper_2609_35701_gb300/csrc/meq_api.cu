@@ -49,9 +49,8 @@ struct Group {
   int64_t mbase = 0;       // first slot of the group in the per-matrix inverse-norm array
   // Fused-statistics partials: the column sums (float offset in the slab), and
   // the row sums, rparts per row, in the X buffer that the last update leaves
-  // idle (CV trajectory, where each update writes U: in the slab).
+  // idle (CV trajectory, where each update writes U and X': in its own scratch).
   int64_t cpart_base = 0;
-  int64_t rpart_base = 0;
   int64_t rparts = 0;
   float* rpart = nullptr;
   std::vector<int> mats;
@@ -97,7 +96,7 @@ struct meq_state {
   std::vector<int> kinds;                     // meq_kind per entry
   int n_hidden = 0;
   meq_options opt{};
-  bool trajectory = false;                    // statistics after every NS iteration
+  float* trajectory_rpart = nullptr;          // CV trajectory (statistics after every NS iteration): the row partials
   int device = 0;
   int num_sms = 0;
   std::vector<MatInfo> mats;
@@ -255,31 +254,30 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     const int64_t m = st->shapes[i].rows, c = st->shapes[i].cols;
     MatInfo& M = st->mats[i];
     M.m = m, M.n = c;
-    M.s = std::min(m, c), M.l = std::max(m, c);
     M.trans = m > c ? 1 : 0;
     M.kind = st->kinds[i];
     M.group = -1;
     if (M.kind != KIND_HIDDEN) continue;
     ++st->n_hidden;
-    auto key = std::make_tuple(M.s, M.l, M.trans);
+    auto key = std::make_tuple(M.s(), M.l(), M.trans);
     auto it = gmap.find(key);
     int g;
     if (it == gmap.end()) {
       g = static_cast<int>(st->groups.size());
       gmap[key] = g;
       Group G;
-      G.s = M.s, G.l = M.l;
+      G.s = M.s(), G.l = M.l();
       G.trans = M.trans;
       G.m = m, G.n = c, G.un = round_up(c, 8);  // whole 16-byte chunks per fp16 row
-      G.lp = round_up(M.l, 64), G.sp = round_up(M.s, 64);
-      G.alpha0 = std::min(pow2_round(std::sqrt(static_cast<double>(M.s) * static_cast<double>(M.l))), 16384.f);
-      G.alpha = std::min(pow2_round(std::sqrt(static_cast<double>(M.l))), 16384.f);
+      G.lp = round_up(M.l(), 64), G.sp = round_up(M.s(), 64);
+      G.alpha0 = std::min(pow2_round(std::sqrt(static_cast<double>(M.s()) * static_cast<double>(M.l()))), 16384.f);
+      G.alpha = std::min(pow2_round(std::sqrt(static_cast<double>(M.l()))), 16384.f);
       st->groups.push_back(G);
     } else {
       g = it->second;
     }
     M.group = g;
-    M.gidx = st->groups[g].count++;
+    M.gidx = static_cast<int32_t>(st->groups[g].count++);
     st->groups[g].mats.push_back(i);
   }
   int64_t mom = 0, u = 0, vec = 0, parts = 0, chunks = 0, hchunks = 0, tiles = 0, rblks = 0, slabs = 0, xblks = 0;
@@ -293,9 +291,6 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
   for (auto& G : st->groups) {  // U is stored group by group: [count][m][un]
     G.u_base = u;
     u += round_up(G.count * G.m * G.un, 64);
-    G.rparts = 2 * ((G.l + 63) / 64);  // at most: 64-column tiles
-    G.rpart_base = parts;
-    if (st->trajectory) parts += round_up(G.count * G.rparts * G.s, 64);
     G.cpart_base = parts;
     parts += round_up(G.count * ((G.s + 31) / 32) * G.l, 64);
   }
@@ -324,12 +319,12 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
       // momentum + X_0: flat chunks of W, or 64 x 64 tiles when X_0 is W transposed
       xblks += M.trans ? ((M.m + kCastTile - 1) / kCastTile) * ((M.n + kCastTile - 1) / kCastTile)
                        : (M.m * M.n + kChunk - 1) / kChunk;
-      folds += (M.s + kFoldCols - 1) / kFoldCols + (M.l + kFoldCols - 1) / kFoldCols;
-      max_parts = std::max(max_parts, 2 * ((M.l + 255) / 256) * M.s + (M.s + 31) / 32 * M.l);
+      folds += (M.s() + kFoldCols - 1) / kFoldCols + (M.l() + kFoldCols - 1) / kFoldCols;
+      max_parts = std::max(max_parts, 2 * ((M.l() + 255) / 256) * M.s() + (M.s() + 31) / 32 * M.l());
     } else {
       M.un = M.n;
       const bool one_pass = M.kind == KIND_TWO_SIDED && M.n <= kRowColMax;
-      M.slab_rows = one_pass ? slab_rows : kColSlab;
+      M.slab_rows = static_cast<int32_t>(one_pass ? slab_rows : kColSlab);
       if (one_pass) rcs += (M.m + M.slab_rows - 1) / M.slab_rows;
       else rblks += (M.m + 7) / 8;  // 8 rows (warps) per block
       if (M.kind == KIND_TWO_SIDED) {
@@ -655,7 +650,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
   st->gemm_tile.clear();
   const GemmTile large{st->opt.ns_cta_pair ? 2 : 1, 256}, small{1, 64};
   int64_t saving = 0;
-  if (pairs_allowed(st->opt) && !st->trajectory)
+  if (pairs_allowed(st->opt) && !st->trajectory_rpart)
     for (const Group& G : st->groups) saving += std::max<int64_t>(0, pair_saving(G)) * G.count;
   const bool pairs = saving >= kPairMinSaving;
   std::vector<int> which;                 // chain of each group: 0 plain, 1 with pairs
@@ -663,7 +658,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
   std::vector<NsOp> A, B;                 // the two chains' products (modes and formats; empty if unused)
   for (const Group& G : st->groups) {
     which.push_back(pairs && pair_saving(G) > 0 ? 1 : 0);
-    chain.push_back(ns_chain(st->opt, G, which.back() == 1, st->trajectory));
+    chain.push_back(ns_chain(st->opt, G, which.back() == 1, st->trajectory_rpart != nullptr));
     (which.back() ? B : A) = chain.back();
   }
   auto joint = [&](size_t i, size_t j) {
@@ -735,8 +730,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
         if (op.mode == MODE_XLAST) {
           // two row partials per tile column
           G.rparts = 2 * ((op_cols(G, op) + t.bn - 1) / t.bn);
-          G.rpart = st->trajectory ? st->d_parts + G.rpart_base
-                                   : reinterpret_cast<float*>(G.x[op.b == BUF_X0 ? 1 : 0]);
+          G.rpart = st->trajectory_rpart ? st->trajectory_rpart : reinterpret_cast<float*>(G.x[op.b == BUF_X0 ? 1 : 0]);
         }
         if (!fill_group(st, G, op, t, Q)) { *why = "cuTensorMapEncodeTiled failed"; return false; }
         Q.tile_begin = tiles;
@@ -766,7 +760,7 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
 extern "C" {
 
 static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
-                             void* cuda_stream, bool trajectory, meq_state** out);
+                             void* cuda_stream, float* trajectory_rpart, meq_state** out);
 
 void meq_default_options(meq_options* o) {
   if (!o) return;
@@ -836,13 +830,14 @@ meq_status meq_init_state(const meq_shape* shapes, int n, const meq_options* opt
 
 meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
                                 void* cuda_stream, meq_state** out) {
-  return init_state(shapes, kinds, n, opt, cuda_stream, false, out);
+  return init_state(shapes, kinds, n, opt, cuda_stream, nullptr, out);
 }
 
-// trajectory: the NS plan gives U's statistics after every iteration
-// (meq_ns_cv_trajectory), not after the last one only.
+// trajectory_rpart (one-matrix state of meq_ns_cv_trajectory, else NULL): the NS
+// plan gives U's statistics after every iteration, not after the last one only;
+// room for 2 * ceil(l / 64) row partials of s floats.
 static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
-                             void* cuda_stream, bool trajectory, meq_state** out) {
+                             void* cuda_stream, float* trajectory_rpart, meq_state** out) {
   if (!out) return fail(nullptr, MEQ_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
   meq_options o;
@@ -878,7 +873,7 @@ static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, c
   st->opt = o;
   st->device = dev;
   st->num_sms = num_sms;
-  st->trajectory = trajectory;
+  st->trajectory_rpart = trajectory_rpart;
 
   Layout L(o.debug_canaries != 0);
   int64_t off_mom, off_u, off_vec4, off_cpart, off_partials, off_counters, off_x0s, off_stats, off_step, off_err, off_mats,
@@ -934,8 +929,10 @@ static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, c
   for (MatInfo& M : st->mats)
     if (M.kind == KIND_HIDDEN) {
       const Group& G = st->groups[M.group];
-      M.rparts = G.rparts;
-      M.rpart_off = (G.rpart - st->d_parts) + M.gidx * G.rparts * G.s;
+      M.rparts = static_cast<int32_t>(G.rparts);
+      // (an offset in floats from the partials' slab, whatever buffer they lie in)
+      const auto at = reinterpret_cast<intptr_t>(G.rpart) - reinterpret_cast<intptr_t>(st->d_parts);
+      M.rpart_off = static_cast<int64_t>(at / static_cast<intptr_t>(sizeof(float))) + M.gidx * G.rparts * G.s;
     }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   std::vector<GroupInfo> gi(st->groups.size());
@@ -1447,11 +1444,12 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
   o.ns_steps = 1;
   if (!valid_options(o, &why)) return fail(nullptr, MEQ_ERR_INVALID_ARG, why);
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  // scratch: r, c, the direction and the two CVs of k = 0, one MatStats per
-  // k >= 1, then the statistics kernels' partial sums
+  // scratch: r, c, the CVs and direction of each k, then the statistics
+  // kernels' partial sums (k = 0) or the NS products' row partials (k >= 1)
   const int64_t rb = round_up(rows * 4, 256), cb = round_up(cols * 4, 256);
   const int64_t tb = round_up(static_cast<int64_t>(sizeof(MatStats)) * (steps + 1), 256);
-  const int64_t pb = round_up(row_col_stats_scratch_floats(rows, cols) * 4, 256);
+  const int64_t rparts = 2 * ((std::max(rows, cols) + 63) / 64) * std::min(rows, cols);
+  const int64_t pb = round_up(std::max(row_col_stats_scratch_floats(rows, cols), rparts) * 4, 256);
   char* tmp = nullptr;
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&tmp), static_cast<size_t>(rb + cb + tb + pb));
   if (e != cudaSuccess) {
@@ -1477,7 +1475,7 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
   meq_state* st = nullptr;
   if (ms == MEQ_OK && steps > 0) {
     o.ns_steps = steps;
-    ms = init_state(&shape, nullptr, 1, &o, cuda_stream, true, &st);
+    ms = init_state(&shape, nullptr, 1, &o, cuda_stream, parts, &st);
   }
   if (ms == MEQ_OK && st) {
     ms = upload_step(st, nullptr, &h, &shape, 1, 0.f, 0.f, 0.f, eps, s);

@@ -38,12 +38,12 @@ constexpr float kUScale = 16384.0f;
 // Per-matrix metadata (device copy built at init).
 struct MatInfo {
   int64_t m, n;          // W layout: rows, cols
-  int64_t s, l;          // oriented NS shape: s = min(m, n), l = max(m, n)
   int32_t trans;         // 1 when the NS layout is W^T (m > n)
   int32_t group;         // shape group (hidden weights)
   int32_t kind;          // 0 hidden, 1 remaining 2D (two-sided), 2 vector
-  int32_t pad_;
-  int64_t gidx;          // index inside its group
+  int32_t rparts;        // row partial sums of squares per NS row: two per tile column of the last update
+  int32_t gidx;          // index inside its group
+  int32_t slab_rows;     // rows per slab (remaining 2D)
   int64_t mom_off;       // float offset of B in the momentum slab
   int64_t u_off;         // element offset of U in the fp16 U slab (row stride un)
   int64_t un;            // U row stride: cols rounded up to 8 (hidden), cols (others)
@@ -53,14 +53,15 @@ struct MatInfo {
   int64_t rblk_begin;    // first 8-row block of the row pass (remaining 2D with long rows, vectors)
   int64_t slab_begin;    // first row slab of the column pass (remaining 2D with long rows)
   int64_t rc_begin;      // first slab of the one-pass form (remaining 2D with rows up to kRowColMax)
-  int64_t slab_rows;     // rows per slab (remaining 2D)
   int64_t tile_begin;    // first cast tile (hidden weights only)
   int64_t xblk_begin;    // first momentum-and-X_0 block (hidden weights only)
   int64_t fold_begin;    // first block of the fold of the partial sums (hidden weights and remaining 2D)
   int64_t rpart_off;     // float offset of NS-row partial sums of squares [rparts][s]
-  int64_t rparts;        // two per tile column of the last update
   int64_t cpart_off;     // float offset of column partial sums of squares: NS columns
                          // [ceil(s/32)][l] (hidden) or normalised columns [slabs][n] (remaining 2D)
+  // oriented NS shape
+  __host__ __device__ int64_t s() const { return m < n ? m : n; }
+  __host__ __device__ int64_t l() const { return m < n ? n : m; }
 };
 
 // Per-group metadata for the elementwise kernels.
