@@ -124,7 +124,11 @@ meq_status meq_state_bytes_kinds(const meq_shape* shapes, const int* kinds, int 
 /* Create the state for n matrices: zeroed momentum (B_{-1} = 0, Algorithm 1)
  * and the workspace, on the current CUDA device. opt may be NULL (defaults).
  * cuda_stream (cudaStream_t, may be NULL) orders the zero-fill. The shape
- * list is copied. On success *out owns device memory until meq_free. */
+ * list is copied. On success *out owns device memory until meq_free.
+ * Entries are updated independently, but the Newton-Schulz products are
+ * planned for the whole list (tile sizes, and whether large weights with
+ * cols != rows run their iterations in pairs), so the rounding of an entry's
+ * update, within the stated tolerances, can depend on the other shapes. */
 meq_status meq_init_state(const meq_shape* shapes, int n, const meq_options* opt,
                           void* cuda_stream, meq_state** out);
 

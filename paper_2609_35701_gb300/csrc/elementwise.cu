@@ -6,7 +6,9 @@
 //                   X_0 scale alpha0 / ||H||_F of Eq. (5).
 //   cast_x0       : X-hat_0 = 16-bit(alpha0 H / ||H||_F) in the oriented NS
 //                   layout (transposed through shared memory for tall W).
-//   finalize      : r, c (Eq. (7)) from the partial sums of squares the last
+//   momentum_x0, x0norm : the default: momentum and an unnormalised bf16 X_0 in
+//                   one pass, then 1 / ||H||_F.
+//   fold, finalize: r, c (Eq. (7)) from the partial sums of squares the last
 //                   NS epilogue wrote, gamma_r, gamma_c (Eq. (8)), the
 //                   direction (Eq. (11)) and the scale vector of Eq. (9).
 //   rowcol, rows, colpart : momentum, row and column statistics of the remaining

@@ -8,10 +8,15 @@
 //   * matrices with the same (s, l) form a group whose X buffers are stacked
 //     [count][s][l_pad] so one 3D TMA tensor map covers the whole group, and
 //     one GEMM launch covers up to kMaxGroups groups;
+//   * each group gets its chain of NS products: GRAM, POLY, XUPD per iteration,
+//     or for large l > s weights two iterations at a time; products of one
+//     kind that are next in both chains share a launch;
 //   * one device arena holds momentum, NS buffers and statistics.
 // Per step (meq_step), on the caller's stream:
 //   upload step scalars + pointer tables, then
-//   momentum_norm, cast_x0, K x (GRAM, POLY, XUPD|XLAST), stats, finalize, apply
+//   momentum (with X_0, its norm or a separate cast), the NS products, [fold,]
+//   finalize, apply; for the other parameter kinds one pass over rows and
+//   columns, or a row and a column pass
 // optionally replayed from a CUDA graph captured at the first step.
 #include <cudaTypedefs.h>
 

@@ -1,7 +1,8 @@
 // Newton-Schulz GEMMs on the sm_103a tensor cores (tcgen05 + TMA + TMEM).
 //
-// One persistent, warp-specialised kernel computes every product of the
-// quintic iteration, Eq. (5) of the paper, for a batch of same-shape groups:
+// Persistent, warp-specialised kernels, instances of one template, compute
+// every product of the quintic iteration, Eq. (5) of the paper, for a batch of
+// same-shape groups:
 //
 //   MODE_SYM  : symmetric s x s products: A = X X^T / alpha^2 (contraction over
 //               l) and, over s, P = a I + b A + c (A A) and the products of the
@@ -11,7 +12,8 @@
 //   MODE_DENSE: X' = P X * (alpha'/alpha) (s x l, contraction over s), and P' P
 //   MODE_XLAST: U = P X / alpha, written as fp16(2^14 U) in the weight's own
 //               layout, with the sums of squares of the stored U's rows and
-//               columns (Eq. (7)) reduced into per-tile partials
+//               columns (Eq. (7)) reduced into per-tile partials (and X'
+//               beside it for the CV trajectory)
 //
 // P X equals a X + (b A + c A^2) X of Eq. (5) exactly in real arithmetic.
 // A and P are symmetric: their launches run only the tiles that hold a 32 x 32
@@ -22,8 +24,8 @@
 // normal range of fp16; the epilogues undo the scale in fp32.
 //
 // Roles (352 threads, one CTA per SM):
-//   warp 0 : TMA producer (one thread), shared-memory ring of 4 stages
-//            (single CTA) or 6 (CTA pair)
+//   warp 0 : TMA producer (one thread), shared-memory ring of 6 stages (CTA
+//            pair, 256 x 256 tiles), 8 (one CTA, 128 x 64) or 4 (128 x 256)
 //   warp 1 : TMEM allocator and tcgen05.mma issuer (one thread; with CTA
 //            pairs, the leader's thread issues cta_group::2 MMAs for both)
 //   warps 2-9 : epilogue; warp w reads TMEM lanes 32*(w%4) .. +31 and takes
@@ -42,7 +44,7 @@
 // dependent integer chain of one thread: measured at 0.35-0.6 us per tile,
 // it left the tensor pipe idle for about 0.5 us between tiles when they did
 // it themselves.
-// Two 128x256 fp32 accumulators (512 TMEM columns) let the epilogue of one
+// Two fp32 accumulators per CTA (512 TMEM columns at 256-column tiles) let the epilogue of one
 // tile overlap the MMAs of the next. The epilogue stages 32 x 32 blocks in
 // swizzled shared memory; the symmetric A and P (each block stored twice)
 // leave by TMA stores, X and U by coalesced 16-byte stores from the threads
