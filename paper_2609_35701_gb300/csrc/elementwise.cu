@@ -325,16 +325,21 @@ __global__ void __launch_bounds__(kThreads) x0norm_kernel(const MatInfo* __restr
   const float* part = partials + M.xblk_begin;
   float* out = ginv + groups[M.group].mbase + M.gidx;
   pdl_wait_predecessor();
-  float acc[1] = {0.f};
+  float acc = 0.f;
   int64_t c = threadIdx.x;
   for (; c + 3 * kThreads < nblk; c += 4 * kThreads) {
     const float x0 = part[c], x1 = part[c + kThreads], x2 = part[c + 2 * kThreads], x3 = part[c + 3 * kThreads];
-    acc[0] += x0, acc[0] += x1, acc[0] += x2, acc[0] += x3;
+    acc += x0, acc += x1, acc += x2, acc += x3;
   }
-  for (; c < nblk; c += kThreads) acc[0] += part[c];
-  block_sum_multi<1>(acc, shf);
-  const float total = acc[0];
+  for (; c < nblk; c += kThreads) acc += part[c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) shf[threadIdx.x >> 5] = acc;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    float total = 0.f;  // the warps one after another: eight adds, fewer cycles than a tree of shuffles
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) total += shf[w];
     const float nrm = sqrtf(total);
     if (!isfinite(total)) atomicCAS(nonfinite, 0, static_cast<int>(blockIdx.x) + 1);  // first non-finite entry, 1-based
     *out = nrm > 0.f ? 1.0f / nrm : 0.f;
