@@ -449,20 +449,24 @@ struct NsOp {
 //   second pair, P' P as a dense one   3 l/s + 6
 // i.e. 45 -> 36 over the five iterations of an FFN weight (l = 8/3 s).
 // Only the five-iteration default with fp16 operands and a fused X_0 takes
-// pairs: its error against fp64 was measured to be no larger than that of the
-// plain form, for these two reasons:
-//   * iteration 0 multiplies by M = P - a I, held in bf16, and adds a X_0 in
-//     fp32 in the epilogue: P's large diagonal is no longer rounded to eight
-//     bits, which pays for what the pairs lose;
-//   * the first pair works with M as well (every singular value is still
-//     small, so P is a I plus a small matrix); in the second pair it is not,
-//     P itself is kept, and P' P is computed whole: mirroring its upper
-//     triangle would force a symmetry that rounding has already broken.
-// Relative error of U~ (numpy emulation, row / column / both / no imbalance):
-//   768 x 2048: 2.57e-3 / 2.76e-3 / 2.88e-3 / 2.25e-3 plain,
-//               2.18e-3 / 2.83e-3 / 2.67e-3 / 2.14e-3 paired;
-// on a GB300, 2048 x 5461 with Student-t scales on both sides (5461 x 2048):
-//               2.41e-3 (2.91e-3) plain, 2.09e-3 (2.83e-3) paired.
+// pairs. Rounding an s x s matrix to 16 bits disturbs each row's norm by the
+// rounding of the diagonal, and the pairs hold three more such matrices per
+// two iterations; so P, A' and P' P are held less a multiple of I, which the
+// epilogues add back in fp32 (aux matrices of the products):
+//   * iteration 0 (bf16) and first pair: every singular value is still small,
+//     P is a I plus a small matrix, held as P - a I;
+//   * second pair: P's diagonal lies between 0.7 and 3.4, near 1.6 where the
+//     input's rows are alike, which is where the rows' statistics are exact
+//     enough to show the rounding: P - kPairP I, A' - kPairA I. There P' P is
+//     computed whole: mirroring its upper triangle would force a symmetry
+//     that rounding has already broken (U~ 2.50e-3 -> 2.58e-3).
+// Error against fp64 over that of the plain chain, numpy emulation, gradients
+// uneven in rows / columns / both / neither, of U~ and of the row RMS:
+//    768 x 2048: 0.83 / 1.00 / 0.91 / 0.93, 0.55 / 0.95 / 0.57 / 0.76
+//   1408 x 5632: 0.89 / 1.02 / 0.94 / 0.88, 0.71 / 1.09 / 0.74 / 0.45
+//   2048 x 5461: 0.99 / 1.11 / 0.99 / 0.87, 1.00 / 1.52 / 0.92 / 0.49
+// (second pair's P, A' and P' P whole: 1408 x 5632, columns, row RMS 1.82).
+constexpr float kPairP = 1.2f, kPairA = 0.8f;
 bool pairs_allowed(const meq_options& o) {
   meq_options d;
   meq_default_options(&d);
@@ -473,9 +477,11 @@ bool pairs_allowed(const meq_options& o) {
 // Pairs take four launches more than the plain chain (about 10 us each), so
 // they are used where they save at least this many k-blocks (256 x 256 x 64;
 // a pair of SMs takes about 0.35 us for one) over the whole state: 10000 take
-// the 76 pairs of a GB300 46 us. Measured steps, plain -> pairs: Llama-130M
-// (17700 saved) 1399 -> 1360 us, Llama-350M 5615 -> 5271 us, four 1B-class
-// layers 5963 -> 5437 us, two 7B-class layers 19930 -> 18000 us.
+// the 76 pairs of a GB300 46 us. Measured steps, plain -> pairs, with the
+// second pair's matrices held whole: Llama-130M (17700 saved) 1399 -> 1360 us,
+// Llama-350M 5615 -> 5271 us, four 1B-class layers 5963 -> 5437 us, two
+// 7B-class layers 19930 -> 18000 us; held less a multiple of I, the pairs cost
+// 28, 55, 18 and 25 us more than that.
 constexpr int64_t kPairMinSaving = 10000;
 
 // k-blocks that the pairs save in one matrix, as the launches run them (whole
@@ -512,7 +518,8 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
     const float ak = (k == 0) ? (fused ? 1.0f : G.alpha0) : G.alpha;
     const bool per_matrix = fused && k == 0;
     const bool pair = pairs && (k == 1 || k == 3);
-    const bool split = pairs && k < 3;  // P is held as M = P - a I
+    // what the matrices are held less of: P - e I, A' - f I
+    const float e = !pairs ? 0.f : k < 3 ? o.ns_a : kPairP, f = pairs && k == 3 ? kPairA : 0.f;
     const int step = pair ? 2 : 1;
     const bool last = k + step == K;
     const NsBuf cx = X(cur), nx = X(cur ^ 1);
@@ -522,34 +529,32 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
     gram.in16 = dX(k), gram.out16 = dA(k);
     gram.scale = gs / (ak * ak), gram.minv_pow = per_matrix ? 2 : 0;
     ops.push_back(gram);
-    NsOp poly;  // P = a I + b A + c A^2 (or M = b A + c A^2)
+    NsOp poly;  // P = a I + b A + c A^2 (less e I: M)
     poly.a = poly.b = BUF_A, poly.out = BUF_P, poly.aux = BUF_A;
     poly.in16 = poly.aux16 = dA(k), poly.out16 = dX(k);
-    poly.c_acc = o.ns_c / gs, poly.c_aux = o.ns_b, poly.c_eye = split ? 0.f : o.ns_a * gs;
+    poly.c_acc = o.ns_c / gs, poly.c_aux = o.ns_b, poly.c_eye = (o.ns_a - e) * gs;
     ops.push_back(poly);
     NsBuf mul = BUF_P;                      // what multiplies X
-    float diag = split ? o.ns_a : 0.f;      // and its identity part, added in the epilogue
+    float diag = e;                         // and its identity part, added in the epilogue
     if (pair) {
-      NsOp q;  // Q = P A (= M A + a A), in the idle X buffer
+      NsOp q;  // Q = P A = M A + e A, in the idle X buffer
       q.a = BUF_P, q.b = BUF_A, q.out = nx, q.c_acc = 1.0f / gs;
-      if (split) q.aux = BUF_A, q.c_aux = o.ns_a;
+      q.aux = BUF_A, q.c_aux = e;
       ops.push_back(q);
-      NsOp a1;  // A' = Q P
+      NsOp a1;  // A' - f I = Q P - f I = Q M + e Q - f I
       a1.a = nx, a1.b = BUF_P, a1.out = BUF_A, a1.c_acc = 1.0f / gs;
-      if (split) a1.aux = nx, a1.c_aux = o.ns_a;
+      a1.aux = nx, a1.c_aux = e, a1.c_eye = -f * gs;
       ops.push_back(a1);
-      NsOp p1 = poly;  // P' (or M') of A'
-      p1.out = nx;
+      NsOp p1 = poly;  // M' = a I + b A' + c A'^2 - e I, in terms of A' - f I
+      p1.out = nx, p1.c_aux = o.ns_b + 2.f * o.ns_c * f;
+      p1.c_eye = (o.ns_a - e + f * (o.ns_b + o.ns_c * f)) * gs;
       ops.push_back(p1);
-      NsOp c;  // P' P, in A's place
+      NsOp c;  // P' P - e^2 I = M' M + e (M + M'), in A's place
       c.a = nx, c.b = BUF_P, c.out = BUF_A, c.c_acc = 1.0f / gs;
-      if (split) {  // less a^2 I: M' M + a (M + M')
-        c.aux = nx, c.c_aux = o.ns_a;
-        c.aux2 = BUF_P, c.c_aux2 = o.ns_a;
-        diag = o.ns_a * o.ns_a;
-      } else {
-        c.mode = MODE_DENSE;
-      }
+      c.aux = nx, c.c_aux = e;
+      c.aux2 = BUF_P, c.c_aux2 = e;
+      if (k == 3) c.mode = MODE_DENSE;
+      diag = e * e;
       ops.push_back(c);
       mul = BUF_A;
     }
@@ -721,8 +726,11 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
         ops.emplace_back(&st->groups[g], &chain[g][at[which[g]]]);
       }
       int aux = ops[0].second->aux2 != BUF_NONE ? 2 : 0;
-      for (const auto& x : ops)
-        if (x.second->aux != BUF_NONE || (x.second->mode == MODE_XLAST && x.second->out != BUF_NONE)) aux = std::max(aux, 1);
+      for (const auto& x : ops) {
+        const bool last = x.second->mode == MODE_XLAST;
+        if (x.second->aux != BUF_NONE) aux = std::max(aux, last ? 2 : 1);
+        if (last && x.second->out != BUF_NONE) aux = 1;
+      }
       const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load && aux < 2 &&
                              launch_cost(ops, small, st->num_sms) < launch_cost(ops, large, st->num_sms);
       GemmTile t = use_small ? small : large;

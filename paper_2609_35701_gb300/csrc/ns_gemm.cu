@@ -523,7 +523,7 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 // One instance per kind of launch: kMode (GemmMode) and kAux, the 16-bit
 // matrices added in the epilogue (0: none; 1: one, in some groups; 2: two, in
 // every group, one product of the paired iterations; of MODE_XLAST, 1: X' is
-// written beside U). As runtime values the
+// written beside U, 2: one matrix, in some groups). As runtime values the
 // operand layout, the output path and the addends cost the producer, the MMA
 // issuer and the epilogue registers and branches in every launch; the chains
 // of dependent instructions are what small launches and launch tails wait for.
@@ -533,6 +533,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
   constexpr int BN = kBN;
   constexpr uint32_t TMEM_COLS = C_::TMEM_COLS;
   constexpr bool kLast = kMode == MODE_XLAST;
+  constexpr bool kAux2 = kAux == 2 && !kLast;
   constexpr bool kSym = kMode == MODE_SYM;  // K-major B, upper-triangle tiles, TMA stores
   constexpr int STAGES = C_::STAGES;
   constexpr int STAGE_BYTES = C_::STAGE_BYTES;
@@ -810,7 +811,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       if (!sched_take_warp(n, e) || static_cast<int>(e.x) >= p.total_tiles) break;
       const TileCoord c = entry_coord(e);
       const GemmGroup& G = p.g[c.g];
-      const bool has_aux = kAux == 2 || (kAux == 1 && !kLast && G.aux != nullptr);
+      const bool has_aux = kAux2 || (kAux == (kLast ? 2 : 1) && G.aux != nullptr);
       const int row0 = c.tm * TILE_M + static_cast<int>(rank) * BM + q * 32;
       const int R = row0 / 32;  // 32-row block index
       const int rows_valid = min(32, G.M - row0);
@@ -851,7 +852,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         const int C = c.tn * (BN / 32) + ch;
         float v[32];
         uint4 aux2[4];
-        if (kAux == 2) {  // each lane its own row
+        if (kAux2) {  // each lane its own row
           const uint8_t* src = static_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
                                static_cast<int64_t>(row0 + min(lane, rows_valid - 1)) * G.aux_ld +
                                static_cast<int64_t>(col0) * 2;
@@ -883,7 +884,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
             else add_aux<false, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
           }
           __syncwarp();  // slot free for the output block
-          if (kAux == 2) {
+          if (kAux2) {
             const float k_aux2 = G.c_aux2;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -899,6 +900,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] *= sc;
+        }
+        if (kLast && kAux == 2 && col0 + 32 > G.N) {  // X's padding columns may hold anything
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (col0 + j >= G.N) v[j] = 0.f;
         }
         if (kLast && kAux == 1) {
           // the CV trajectory: X' too, in the NS layout, for the next iteration
@@ -1076,12 +1082,15 @@ int ns_gemm_smem_bytes(int pair) { return pair == 2 ? Cfg<2, 256>::SMEM_BYTES : 
 template <int kPair, int kBN, typename F>
 static cudaError_t with_kernel(int mode, int aux, F f) {
   constexpr int bytes = Cfg<kPair, kBN>::SMEM_BYTES;
+  if constexpr (kBN == 256)  // the paired iterations' products
+    if (aux == 2)
+      return mode == MODE_XLAST   ? f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 2>, bytes)
+             : mode == MODE_DENSE ? f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 2>, bytes)
+                                  : f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 2>, bytes);
   if (mode == MODE_XLAST)
     return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 0>, bytes);
   if (mode == MODE_DENSE)
     return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 0>, bytes);
-  if constexpr (kBN == 256)
-    if (aux == 2) return f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 2>, bytes);
   return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 0>, bytes);
 }
 
