@@ -443,7 +443,7 @@ def main():
 
     K = 5
     hid = [sh for sh, k in zip(shapes, kinds) if k == W.HIDDEN]   # Newton-Schulz runs on hidden weights only
-    # executed products, symmetric ones as one triangle (paired iterations run fewer than Eq. (5) as written)
+    # executed products, symmetric ones as one triangle
     sym = opt.ns_flops_per_step
     dense = sum(ns_flops(min(r, c), max(r, c), K)[1] for r, c in hid)
     n_gemm_launches = opt.ns_gemm_launches_per_step

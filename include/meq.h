@@ -126,9 +126,8 @@ meq_status meq_state_bytes_kinds(const meq_shape* shapes, const int* kinds, int 
  * cuda_stream (cudaStream_t, may be NULL) orders the zero-fill. The shape
  * list is copied. On success *out owns device memory until meq_free.
  * Entries are updated independently, but the Newton-Schulz products are
- * planned for the whole list (tile sizes, and whether large weights with
- * cols != rows run their iterations in pairs), so the rounding of an entry's
- * update, within the stated tolerances, can depend on the other shapes. */
+ * planned for the whole list (tile sizes), and so is the order of some sums:
+ * the last bits of an entry's statistics can depend on the other shapes. */
 meq_status meq_init_state(const meq_shape* shapes, int n, const meq_options* opt,
                           void* cuda_stream, meq_state** out);
 
@@ -266,10 +265,8 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
  * many of them are Newton-Schulz GEMM launches. */
 int meq_kernels_per_step(const meq_state* st);
 int meq_ns_gemm_launches_per_step(const meq_state* st);
-/* Floating-point operations of those products, the symmetric ones counted as
- * one triangle. Large FFN-like weights run Eq. (5) two iterations at a time
- * (fewer operations, the same polynomial), so this can be less than the
- * count of Eq. (5) as written. */
+/* Floating-point operations of those products (Eq. (5) as written), the
+ * symmetric ones counted as one triangle. */
 double meq_ns_flops_per_step(const meq_state* st);
 
 /* Per-phase timing with CUDA events on the launch stream. While enabled,

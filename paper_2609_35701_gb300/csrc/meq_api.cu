@@ -8,9 +8,7 @@
 //   * matrices with the same (s, l) form a group whose X buffers are stacked
 //     [count][s][l_pad] so one 3D TMA tensor map covers the whole group, and
 //     one GEMM launch covers up to kMaxGroups groups;
-//   * each group gets its chain of NS products: GRAM, POLY, XUPD per iteration,
-//     or for large l > s weights two iterations at a time; products of one
-//     kind that are next in both chains share a launch;
+//   * each group gets its chain of NS products, GRAM, POLY, XUPD per iteration;
 //   * one device arena holds momentum, NS buffers and statistics.
 // Per step (meq_step), on the caller's stream:
 //   upload step scalars + pointer tables, then
@@ -424,80 +422,20 @@ uint32_t make_idesc(bool fp16, bool b_mn_major, int m, int n) {
 bool iter_fp16(const meq_options& o, int k) { return k < 32 && ((o.ns_fp16_mask >> k) & 1u); }
 
 // ------------------------------------------------------- Newton-Schulz plan
-// One product of one shape group. Buffers: the two X buffers, A and P. An X
-// buffer that holds no live iterate also serves as a third s x s buffer (l >= s).
+// One product of one shape group.
 enum NsBuf : int { BUF_X0 = 0, BUF_X1 = 1, BUF_A = 2, BUF_P = 3, BUF_NONE = 4 };
 
 struct NsOp {
-  int mode = MODE_SYM;
+  int mode = MODE_SYM;                 // MODE_SYM: the output is s x s, else s x l
   bool gram = false;                   // contraction over l (operands are X), else over s
-  NsBuf a = BUF_NONE, b = BUF_NONE, out = BUF_NONE, aux = BUF_NONE, aux2 = BUF_NONE;
-  bool out_is_x = false;               // DENSE: the output is s x l (else s x s)
-  bool aux_is_x = false;
+  NsBuf a = BUF_NONE, b = BUF_NONE, out = BUF_NONE, aux = BUF_NONE;
   bool in16 = true, out16 = true, aux16 = true;  // fp16 (else bf16)
-  float scale = 1.f, c_acc = 1.f, c_aux = 0.f, c_aux2 = 0.f, c_eye = 0.f;
+  float scale = 1.f, c_acc = 1.f, c_aux = 0.f, c_eye = 0.f;
   int minv_pow = 0;
 };
 
-// Eq. (5) two iterations at a time. With A = X X^T, P = p(A) = a I + b A + c A^2
-// and X' = P X, the next Gram matrix is A' = X' X'^T = P A P (P and A commute),
-// so P' = p(A') and X'' = (P' P) X need no X': one Gram product over l and one
-// dense product over l fall away for four or so products over s.
-// In units of s^3 fused multiply-adds / 2 (a symmetric product over s is 1):
-//   two plain iterations               6 l/s + 2
-//   first pair, all products symmetric 3 l/s + 5
-//   second pair, P' P as a dense one   3 l/s + 6
-// i.e. 45 -> 36 over the five iterations of an FFN weight (l = 8/3 s).
-// Only the five-iteration default with fp16 operands and a fused X_0 takes
-// pairs. Rounding an s x s matrix to 16 bits disturbs each row's norm by the
-// rounding of the diagonal, and the pairs hold three more such matrices per
-// two iterations; so P, A' and P' P are held less a multiple of I, which the
-// epilogues add back in fp32 (aux matrices of the products):
-//   * iteration 0 (bf16) and first pair: every singular value is still small,
-//     P is a I plus a small matrix, held as P - a I;
-//   * second pair: P's diagonal lies between 0.7 and 3.4, near 1.6 where the
-//     input's rows are alike, which is where the rows' statistics are exact
-//     enough to show the rounding: P - kPairP I, A' - kPairA I. There P' P is
-//     computed whole: mirroring its upper triangle would force a symmetry
-//     that rounding has already broken (U~ 2.50e-3 -> 2.58e-3).
-// Error against fp64 over that of the plain chain, numpy emulation, gradients
-// uneven in rows / columns / both / neither, of U~ and of the row RMS:
-//    768 x 2048: 0.83 / 1.00 / 0.91 / 0.93, 0.55 / 0.95 / 0.57 / 0.76
-//   1408 x 5632: 0.89 / 1.02 / 0.94 / 0.88, 0.71 / 1.09 / 0.74 / 0.45
-//   2048 x 5461: 0.99 / 1.11 / 0.99 / 0.87, 1.00 / 1.52 / 0.92 / 0.49
-// (second pair's P, A' and P' P whole: 1408 x 5632, columns, row RMS 1.82).
-constexpr float kPairP = 1.2f, kPairA = 0.8f;
-bool pairs_allowed(const meq_options& o) {
-  meq_options d;
-  meq_default_options(&d);
-  return o.ns_steps == 5 && o.ns_x0_fused != 0 && (o.ns_fp16_mask & 0x1Fu) == 0x1Fu && o.ns_a == d.ns_a &&
-         o.ns_b == d.ns_b && o.ns_c == d.ns_c;
-}
-
-// Pairs take four launches more than the plain chain (about 10 us each), so
-// they are used where they save at least this many k-blocks (256 x 256 x 64;
-// a pair of SMs takes about 0.35 us for one) over the whole state: 10000 take
-// the 76 pairs of a GB300 46 us. Measured steps, plain -> pairs, with the
-// second pair's matrices held whole: Llama-130M (17700 saved) 1399 -> 1360 us,
-// Llama-350M 5615 -> 5271 us, four 1B-class layers 5963 -> 5437 us, two
-// 7B-class layers 19930 -> 18000 us; held less a multiple of I, the pairs cost
-// 28, 55, 18 and 25 us more than that.
-constexpr int64_t kPairMinSaving = 10000;
-
-// k-blocks that the pairs save in one matrix, as the launches run them (whole
-// upper-triangle tiles, whole k-blocks); 0 below s = 512, where the pairs'
-// error against fp64 was measured to grow (128 x 315: 2.6e-3 -> 2.9e-3; with
-// s = 3 it leaves the tolerance) and there is little to save.
-constexpr int64_t kPairMinS = 512;
-int64_t pair_saving(const Group& G) {
-  if (G.s < kPairMinS) return 0;
-  const int64_t ts = (G.s + 255) / 256, tl = (G.l + 255) / 256, ks = (G.s + 63) / 64, kl = (G.l + 63) / 64;
-  const int64_t sym = ts * (ts + 1) / 2;
-  return 2 * (sym * kl + ts * tl * ks) - 5 * sym * ks - ts * ts * ks;
-}
-
-// The products of one group, in order.
-std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, bool trajectory) {
+// The products of one group, in order: the same kinds and formats for every group.
+std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool trajectory) {
   std::vector<NsOp> ops;
   const int K = o.ns_steps;
   const bool fused = o.ns_x0_fused != 0;
@@ -506,78 +444,38 @@ std::vector<NsOp> ns_chain(const meq_options& o, const Group& G, bool pairs, boo
   // except that a fused X_0 is bf16 (written unnormalised by the momentum pass).
   auto dA = [&](int k) { return iter_fp16(o, k); };
   auto dX = [&](int k) { return (fused && k == 0) ? false : iter_fp16(o, k); };
-  // The paired chain holds its s x s matrices times 2^11: their entries stay
-  // below 32 (|P' P| <= a^2 = 11.9), and those that couple a row of tiny norm
-  // to the others keep fp16's full precision down to 3e-8 instead of 6e-5.
-  // (Unscaled, rows at 1e-4 of the typical norm lost up to 8% of U~.)
-  const float gs = pairs ? 2048.f : 1.f;
-  int cur = 0;
-  auto X = [](int i) { return i ? BUF_X1 : BUF_X0; };
-  for (int k = 0; k < K;) {
+  for (int k = 0; k < K; ++k) {
     // storage scale of X_k; a fused X_0 is unscaled and its 1/||H||_F is applied per matrix
     const float ak = (k == 0) ? (fused ? 1.0f : G.alpha0) : G.alpha;
-    const bool per_matrix = fused && k == 0;
-    const bool pair = pairs && (k == 1 || k == 3);
-    // what the matrices are held less of: P - e I, A' - f I
-    const float e = !pairs ? 0.f : k < 3 ? o.ns_a : kPairP, f = pairs && k == 3 ? kPairA : 0.f;
-    const int step = pair ? 2 : 1;
-    const bool last = k + step == K;
-    const NsBuf cx = X(cur), nx = X(cur ^ 1);
+    const bool per_matrix = fused && k == 0, last = k + 1 == K;
+    const NsBuf cx = k & 1 ? BUF_X1 : BUF_X0, nx = k & 1 ? BUF_X0 : BUF_X1;
     NsOp gram;  // A = X X^T
     gram.gram = true;
     gram.a = gram.b = cx, gram.out = BUF_A;
     gram.in16 = dX(k), gram.out16 = dA(k);
-    gram.scale = gs / (ak * ak), gram.minv_pow = per_matrix ? 2 : 0;
+    gram.scale = 1.0f / (ak * ak), gram.minv_pow = per_matrix ? 2 : 0;
     ops.push_back(gram);
-    NsOp poly;  // P = a I + b A + c A^2 (less e I: M)
+    NsOp poly;  // P = a I + b A + c A^2
     poly.a = poly.b = BUF_A, poly.out = BUF_P, poly.aux = BUF_A;
     poly.in16 = poly.aux16 = dA(k), poly.out16 = dX(k);
-    poly.c_acc = o.ns_c / gs, poly.c_aux = o.ns_b, poly.c_eye = (o.ns_a - e) * gs;
+    poly.c_acc = o.ns_c, poly.c_aux = o.ns_b, poly.c_eye = o.ns_a;
     ops.push_back(poly);
-    NsBuf mul = BUF_P;                      // what multiplies X
-    float diag = e;                         // and its identity part, added in the epilogue
-    if (pair) {
-      NsOp q;  // Q = P A = M A + e A, in the idle X buffer
-      q.a = BUF_P, q.b = BUF_A, q.out = nx, q.c_acc = 1.0f / gs;
-      q.aux = BUF_A, q.c_aux = e;
-      ops.push_back(q);
-      NsOp a1;  // A' - f I = Q P - f I = Q M + e Q - f I
-      a1.a = nx, a1.b = BUF_P, a1.out = BUF_A, a1.c_acc = 1.0f / gs;
-      a1.aux = nx, a1.c_aux = e, a1.c_eye = -f * gs;
-      ops.push_back(a1);
-      NsOp p1 = poly;  // M' = a I + b A' + c A'^2 - e I, in terms of A' - f I
-      p1.out = nx, p1.c_aux = o.ns_b + 2.f * o.ns_c * f;
-      p1.c_eye = (o.ns_a - e + f * (o.ns_b + o.ns_c * f)) * gs;
-      ops.push_back(p1);
-      NsOp c;  // P' P - e^2 I = M' M + e (M + M'), in A's place
-      c.a = nx, c.b = BUF_P, c.out = BUF_A, c.c_acc = 1.0f / gs;
-      c.aux = nx, c.c_aux = e;
-      c.aux2 = BUF_P, c.c_aux2 = e;
-      if (k == 3) c.mode = MODE_DENSE;
-      diag = e * e;
-      ops.push_back(c);
-      mul = BUF_A;
-    }
     NsOp up;  // X' = P X, or U = P X (trajectory: both at once)
     up.mode = last || trajectory ? MODE_XLAST : MODE_DENSE;
-    up.a = mul, up.b = cx, up.out = last ? BUF_NONE : nx, up.out_is_x = true;
+    up.a = BUF_P, up.b = cx, up.out = last ? BUF_NONE : nx;
     up.in16 = dX(k);
-    up.out16 = last ? true : dX(k + step);
+    up.out16 = last ? true : dX(k + 1);
     up.scale = up.mode == MODE_XLAST ? 1.0f / ak : G.alpha / ak;
-    up.c_acc = 1.0f / gs;
     up.minv_pow = per_matrix ? 1 : 0;
-    if (diag != 0.f) up.aux = cx, up.aux_is_x = true, up.aux16 = dX(k), up.c_aux = diag;
     if (up.mode == MODE_XLAST && !last) up.c_aux = G.alpha;
     ops.push_back(up);
-    cur ^= 1;
-    k += step;
   }
   return ops;
 }
 
 // Rows and columns of a product's output, and the length of its contraction.
 int64_t op_rows(const Group& G, const NsOp&) { return G.s; }
-int64_t op_cols(const Group& G, const NsOp& op) { return op.out_is_x ? G.l : G.s; }
+int64_t op_cols(const Group& G, const NsOp& op) { return op.mode == MODE_SYM ? G.s : G.l; }
 int64_t op_depth(const Group& G, const NsOp& op) { return op.gram ? G.l : G.s; }
 
 // Estimated duration (us) of a launch, to choose between 64-column tiles on
@@ -621,19 +519,17 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, const GemmT
   Q.N = static_cast<int32_t>(op_cols(G, op));
   Q.K = static_cast<int32_t>(op_depth(G, op));
   Q.sym = dense ? 0 : 1;
-  Q.same_ab = (!dense && op.a == op.b) ? 1 : 0;
   bool ok = map(&Q.tmA, op.a, op.gram, 64, 128, SW128);
-  if (dense) ok &= map(&Q.tmB, op.b, op.out_is_x, 64, 64, SW128);
+  if (dense) ok &= map(&Q.tmB, op.b, true, 64, 64, SW128);
   else ok &= map(&Q.tmB, op.b, op.gram, 64, b_rows, SW128);
   if (Q.sym) ok &= map(&Q.tmO, op.out, false, 32, 32, SW64);
-  Q.scale = op.aux == BUF_NONE ? op.scale * op.c_acc : op.scale;  // without aux the epilogue takes one factor
-  Q.c_acc = op.c_acc, Q.c_aux = op.c_aux, Q.c_aux2 = op.c_aux2, Q.c_eye = op.c_eye;
+  Q.scale = op.scale;
+  Q.c_acc = op.c_acc, Q.c_aux = op.c_aux, Q.c_eye = op.c_eye;
   if (op.minv_pow) Q.minv = st->d_ginv + G.mbase, Q.minv_pow = op.minv_pow;
   Q.out_fp16 = op.out16, Q.aux_fp16 = op.aux16;
-  if (op.aux != BUF_NONE) Q.aux = base[op.aux], Q.aux_ld = ld(op.aux_is_x), Q.aux_mstride = G.s * ld(op.aux_is_x);
-  if (op.aux2 != BUF_NONE) Q.aux2 = base[op.aux2];
+  if (op.aux != BUF_NONE) Q.aux = base[op.aux], Q.aux_ld = ld(false), Q.aux_mstride = G.s * ld(false);
   if (op.mode == MODE_DENSE) {
-    Q.out = base[op.out], Q.out_ld = ld(op.out_is_x), Q.out_mstride = G.s * ld(op.out_is_x);
+    Q.out = base[op.out], Q.out_ld = ld(true), Q.out_mstride = G.s * ld(true);
   } else if (op.mode == MODE_XLAST) {
     Q.out = st->d_u + G.u_base, Q.out_ld = G.un * 2, Q.out_mstride = G.m * G.un * 2;
     if (op.out != BUF_NONE) Q.out2 = base[op.out], Q.out2_ld = ld(true), Q.out2_mstride = G.s * ld(true);
@@ -651,56 +547,23 @@ bool fill_group(const meq_state* st, const Group& G, const NsOp& op, const GemmT
   return ok;
 }
 
-// Prebuilds the GemmParams of every NS launch of one step. Groups run one of
-// two chains of products (plain, or with pairs of iterations); products of
-// the same kind and operand format that are next in both chains share a launch.
+// Prebuilds the GemmParams of every NS launch of one step.
 bool build_gemm_plan(meq_state* st, std::string* why) {
   st->gemm.clear();
   st->gemm_grid.clear();
   st->gemm_tile.clear();
   const GemmTile large{st->opt.ns_cta_pair ? 2 : 1, 256}, small{1, 64};
-  int64_t saving = 0;
-  if (pairs_allowed(st->opt) && !st->trajectory_rpart)
-    for (const Group& G : st->groups) saving += std::max<int64_t>(0, pair_saving(G)) * G.count;
-  const bool pairs = saving >= kPairMinSaving;
-  std::vector<int> which;                 // chain of each group: 0 plain, 1 with pairs
-  std::vector<std::vector<NsOp>> chain;   // its products
-  std::vector<NsOp> A, B;                 // the two chains' products (modes and formats; empty if unused)
-  for (const Group& G : st->groups) {
-    which.push_back(pairs && pair_saving(G) > 0 ? 1 : 0);
-    chain.push_back(ns_chain(st->opt, G, which.back() == 1, st->trajectory_rpart != nullptr));
-    (which.back() ? B : A) = chain.back();
-  }
-  auto joint = [&](size_t i, size_t j) {
-    return i < A.size() && j < B.size() && A[i].mode == B[j].mode && A[i].in16 == B[j].in16 &&
-           A[i].aux2 == B[j].aux2;
-  };
-  // fewest launches from product i of chain A and j of chain B on
-  std::vector<std::vector<int>> left(A.size() + 1, std::vector<int>(B.size() + 1, 0));
-  for (size_t i = A.size() + 1; i-- > 0;)
-    for (size_t j = B.size() + 1; j-- > 0;) {
-      if (i == A.size() && j == B.size()) continue;
-      int best = 1 << 30;
-      if (joint(i, j)) best = 1 + left[i + 1][j + 1];
-      if (i < A.size()) best = std::min(best, 1 + left[i + 1][j]);
-      if (j < B.size()) best = std::min(best, 1 + left[i][j + 1]);
-      left[i][j] = best;
-    }
-  size_t at[2] = {0, 0};
-  while (at[0] < A.size() || at[1] < B.size()) {
-    bool take[2] = {false, false};
-    if (joint(at[0], at[1]) && left[at[0]][at[1]] == 1 + left[at[0] + 1][at[1] + 1]) take[0] = take[1] = true;
-    else if (at[0] < A.size() && left[at[0]][at[1]] == 1 + left[at[0] + 1][at[1]]) take[0] = true;
-    else take[1] = true;
-    std::vector<int> gs;
-    for (size_t g = 0; g < st->groups.size(); ++g)
-      if (take[which[g]]) gs.push_back(static_cast<int>(g));
+  std::vector<std::vector<NsOp>> chain;   // the products of each group
+  for (const Group& G : st->groups) chain.push_back(ns_chain(st->opt, G, st->trajectory_rpart != nullptr));
+  for (size_t at = 0; !chain.empty() && at < chain[0].size(); ++at) {
+    std::vector<int> gs(st->groups.size());
+    for (size_t g = 0; g < gs.size(); ++g) gs[g] = static_cast<int>(g);
     // Launches of a few rounds of tiles take the longest contractions first,
     // whichever way they walk their tiles, so that the tail is made of short
     // ones (56 weights of a 60M model, 2.2 rounds: Gram launches that met the
     // FFN weights last took 17.6 instead of 15.1 us; at 6.6 rounds, the 130M
     // model, no gain: the order of the groups stays).
-    const auto op_of = [&](int g) -> const NsOp& { return chain[g][at[which[g]]]; };
+    const auto op_of = [&](int g) -> const NsOp& { return chain[g][at]; };
     int64_t all_tiles = 0;
     for (int g : gs)
       all_tiles += tile_count(op_rows(st->groups[g], op_of(g)), op_cols(st->groups[g], op_of(g)),
@@ -723,23 +586,18 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
       std::vector<std::pair<const Group*, const NsOp*>> ops;
       for (int gi = 0; gi < P.ngroups; ++gi) {
         const int g = gs[g0 + gi];
-        ops.emplace_back(&st->groups[g], &chain[g][at[which[g]]]);
+        ops.emplace_back(&st->groups[g], &op_of(g));
       }
-      int aux = ops[0].second->aux2 != BUF_NONE ? 2 : 0;
-      for (const auto& x : ops) {
-        const bool last = x.second->mode == MODE_XLAST;
-        if (x.second->aux != BUF_NONE) aux = std::max(aux, last ? 2 : 1);
-        if (last && x.second->out != BUF_NONE) aux = 1;
-      }
-      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load && aux < 2 &&
+      const bool use_small = st->opt.ns_cta_pair && !st->opt.debug_skip_load &&
                              launch_cost(ops, small, st->num_sms) < launch_cost(ops, large, st->num_sms);
       GemmTile t = use_small ? small : large;
-      t.aux = aux;
+      const NsOp& first = *ops[0].second;
+      t.aux = first.aux != BUF_NONE || (first.mode == MODE_XLAST && first.out != BUF_NONE) ? 1 : 0;
       for (int gi = 0; gi < P.ngroups; ++gi) {
         const int g = gs[g0 + gi];
         GemmGroup& Q = P.g[gi];
         Group& G = st->groups[g];
-        const NsOp& op = chain[g][at[which[g]]];
+        const NsOp& op = op_of(g);
         if (op.mode == MODE_XLAST) {
           // two row partials per tile column
           G.rparts = 2 * ((op_cols(G, op) + t.bn - 1) / t.bn);
@@ -762,8 +620,6 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
       // persistent grid: one CTA (pair) per SM (pair of SMs), never more than the tiles
       st->gemm_grid.push_back(t.pair * std::max(1, std::min(tiles, st->num_sms / t.pair)));
     }
-    for (int c = 0; c < 2; ++c)
-      if (take[c]) ++at[c];
   }
   return true;
 }

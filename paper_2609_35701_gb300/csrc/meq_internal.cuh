@@ -98,24 +98,22 @@ struct GemmGroup {
   int32_t band;           // dense outputs: tile rows per band of the tile order
   int32_t tile_begin;     // first tile of this group in the launch
   int32_t sym;            // 1: symmetric s x s output (upper-triangle tiles, mirrored stores)
-  int32_t same_ab;        // 1: both operands are the same matrix (a diagonal tile loads it once)
   int32_t trans;          // XLAST: 1 when the weight is the transpose of the NS layout
-  // Epilogue: with aux, scale * (c_acc * acc + c_aux * aux) + c_aux2 * aux2 +
-  // c_eye * I (aux2 where given), else scale * acc; scale holds 1/alpha^2
-  // (Gram), alpha_next/alpha (update), 1/alpha (last update) or 1.
+  // Epilogue: with aux (polynomial), c_acc * acc + c_aux * aux + c_eye * I, else
+  // scale * acc; scale holds 1/alpha^2 (Gram), alpha_next/alpha (update) or
+  // 1/alpha (last update).
   float scale;
-  float c_acc, c_aux, c_aux2, c_eye;
+  float c_acc, c_aux, c_eye;
   const float* minv;      // iteration 0 with X_0 unnormalised: 1/||H||_F per matrix of the group
   int32_t minv_pow;       // epilogue scale *= minv^minv_pow (0, 1 or 2)
   int32_t out_fp16;       // 16-bit format of the output (1 = fp16, 0 = bf16)
-  int32_t aux_fp16;       // 16-bit format of aux and aux2
+  int32_t aux_fp16;       // 16-bit format of aux
   void* out;              // DENSE: 16-bit output; XLAST: fp16(kUScale U) in the weight's layout
   int64_t out_ld;         // DENSE / XLAST: output row stride in bytes
   int64_t out_mstride;    // DENSE / XLAST: output matrix stride in bytes
   void* out2;             // XLAST with aux 1: 16-bit X' (c_aux * U), its row and matrix strides in bytes
   int64_t out2_ld, out2_mstride;
-  const void* aux;        // 16-bit matrix the epilogue adds (same rows and columns as the output), or null
-  const void* aux2;       // a second one, in aux's layout, or null
+  const void* aux;        // polynomial: the 16-bit A
   int64_t aux_ld;         // bytes
   int64_t aux_mstride;    // bytes
   float* rpart;           // XLAST: NS-row partial sums of squares, [count][2 * tiles_n][M]
@@ -128,8 +126,7 @@ struct GemmGroup {
 // bn columns.
 struct GemmTile {
   int pair, bn;
-  int aux = 0;  // addends of the epilogue: 0, 1 (in some group) or 2 (in every group; 256-column tiles only);
-                // XLAST: 1 when X' is written too
+  int aux = 0;  // SYM: 1 when the epilogue adds a I + b A (polynomial); XLAST: 1 when X' is written too
 };
 
 // One GEMM launch: one product's shape groups, taken as one tile queue in

@@ -5,11 +5,10 @@
 // same-shape groups:
 //
 //   MODE_SYM  : symmetric s x s products: A = X X^T / alpha^2 (contraction over
-//               l) and, over s, P = a I + b A + c (A A) and the products of the
-//               paired iterations (meq_api.cu); a I + b A is added in fp32 from
-//               the same 16-bit A the product uses, so P is exactly a
+//               l) and P = a I + b A + c (A A) (over s); a I + b A is added in
+//               fp32 from the same 16-bit A the product uses, so P is exactly a
 //               polynomial of that matrix
-//   MODE_DENSE: X' = P X * (alpha'/alpha) (s x l, contraction over s), and P' P
+//   MODE_DENSE: X' = P X * (alpha'/alpha) (s x l, contraction over s)
 //   MODE_XLAST: U = P X / alpha, written as fp16(2^14 U) in the weight's own
 //               layout, with the sums of squares of the stored U's rows and
 //               columns (Eq. (7)) reduced into per-tile partials (and X'
@@ -520,21 +519,20 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_reads() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // Every committed store has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// One instance per kind of launch: kMode (GemmMode) and kAux, the 16-bit
-// matrices added in the epilogue (0: none; 1: one, in some groups; 2: two, in
-// every group, one product of the paired iterations; of MODE_XLAST, 1: X' is
-// written beside U, 2: one matrix, in some groups). As runtime values the
-// operand layout, the output path and the addends cost the producer, the MMA
-// issuer and the epilogue registers and branches in every launch; the chains
-// of dependent instructions are what small launches and launch tails wait for.
+// One instance per kind of launch: kMode (GemmMode) and kAux (MODE_SYM: 1 for
+// the polynomial, whose epilogue adds a I + b A; MODE_XLAST: 1 when X' is
+// written beside U). As runtime values the operand layout, the output path and
+// the addend cost the producer, the MMA issuer and the epilogue registers and
+// branches in every launch; the chains of dependent instructions are what
+// small launches and launch tails wait for.
 template <int kPair, int kBN, int kMode, int kAux>
 __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_constant__ GemmParams p) {
   using C_ = Cfg<kPair, kBN>;
   constexpr int BN = kBN;
   constexpr uint32_t TMEM_COLS = C_::TMEM_COLS;
   constexpr bool kLast = kMode == MODE_XLAST;
-  constexpr bool kAux2 = kAux == 2 && !kLast;
   constexpr bool kSym = kMode == MODE_SYM;  // K-major B, upper-triangle tiles, TMA stores
+  constexpr bool kPoly = kSym && kAux == 1;
   constexpr int STAGES = C_::STAGES;
   constexpr int STAGE_BYTES = C_::STAGE_BYTES;
   constexpr int TILE_M = C_::TILE_M;
@@ -811,7 +809,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       if (!sched_take_warp(n, e) || static_cast<int>(e.x) >= p.total_tiles) break;
       const TileCoord c = entry_coord(e);
       const GemmGroup& G = p.g[c.g];
-      const bool has_aux = kAux2 || (kAux == (kLast ? 2 : 1) && G.aux != nullptr);
       const int row0 = c.tm * TILE_M + static_cast<int>(rank) * BM + q * 32;
       const int R = row0 / 32;  // 32-row block index
       const int rows_valid = min(32, G.M - row0);
@@ -821,7 +818,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       if ((ch0 & 1) != half) ++ch0;                // this warp's chunks: ch % 2 == half
       if (row0 >= G.M) ch0 = nch;
       uint8_t* outm = static_cast<uint8_t*>(G.out) + static_cast<int64_t>(c.mat) * G.out_mstride;
-      // aux block of the chunk, lane L holds 16-byte chunk (L % 4) of rows L/4 + 8i.
+      // A block of the chunk (polynomial), lane L holds 16-byte chunk (L % 4) of rows L/4 + 8i.
       uint4 aux[4];
       const uint8_t* auxm = reinterpret_cast<const uint8_t*>(G.aux) + static_cast<int64_t>(c.mat) * G.aux_mstride;
       auto load_aux = [&](int col0) {
@@ -839,9 +836,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       // What needs no accumulator is requested before waiting for it: the
       // polynomial's first A block, and the output scale (iteration 0 reads
       // its matrix's 1/||H||_F from global memory).
-      if (has_aux && ch0 < nch) load_aux(c.tn * BN + ch0 * 32);
+      if (kPoly && ch0 < nch) load_aux(c.tn * BN + ch0 * 32);
       float sc = G.scale;
-      if (G.minv_pow) {
+      if (!kPoly && G.minv_pow) {
         const float iv = G.minv[c.mat];
         sc *= G.minv_pow == 2 ? iv * iv : iv;
       }
@@ -851,22 +848,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         const int col0 = c.tn * BN + ch * 32;
         const int C = c.tn * (BN / 32) + ch;
         float v[32];
-        uint4 aux2[4];
-        if (kAux2) {  // each lane its own row
-          const uint8_t* src = static_cast<const uint8_t*>(G.aux2) + static_cast<int64_t>(c.mat) * G.aux_mstride +
-                               static_cast<int64_t>(row0 + min(lane, rows_valid - 1)) * G.aux_ld +
-                               static_cast<int64_t>(col0) * 2;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) aux2[k] = __ldg(reinterpret_cast<const uint4*>(src) + k);
-        }
         __syncwarp();  // the load is warp-wide (.sync.aligned)
         tmem_ld_32cols(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * BN + ch * 32), v);
         if (kSym) {
           bulk_wait_reads();  // both slots free (only lane 0 has stores to wait for)
           __syncwarp();
         }
-        if (has_aux) {
-          const float k_acc = sc * G.c_acc, k_aux = sc * G.c_aux, k_eye = G.c_eye;
+        if (kPoly) {
+          const float k_acc = G.c_acc, k_aux = G.c_aux, k_eye = G.c_eye;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int r = (lane >> 2) + 8 * i, k = lane & 3;
@@ -875,7 +864,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           __syncwarp();
           if (ch + 2 < nch) load_aux(col0 + 64);  // in flight while this chunk is processed
           // row0 and col0 are multiples of 32: the diagonal is lane = j of the block C == R
-          const bool diag = kSym && C == R;
+          const bool diag = C == R;
           if (G.aux_fp16) {
             if (diag) add_aux<true, true>(slot, lane, v, k_acc, k_aux, k_eye, lane);
             else add_aux<true, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
@@ -884,27 +873,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
             else add_aux<false, false>(slot, lane, v, k_acc, k_aux, 0.f, 0);
           }
           __syncwarp();  // slot free for the output block
-          if (kAux2) {
-            const float k_aux2 = G.c_aux2;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const uint32_t ws[4] = {aux2[k].x, aux2[k].y, aux2[k].z, aux2[k].w};
-#pragma unroll
-              for (int h = 0; h < 4; ++h) {
-                const float2 a2 = unpack_half2<true>(ws[h]);  // (fp16 chains only)
-                v[8 * k + 2 * h] = fmaf(k_aux2, a2.x, v[8 * k + 2 * h]);
-                v[8 * k + 2 * h + 1] = fmaf(k_aux2, a2.y, v[8 * k + 2 * h + 1]);
-              }
-            }
-          }
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] *= sc;
-        }
-        if (kLast && kAux == 2 && col0 + 32 > G.N) {  // X's padding columns may hold anything
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col0 + j >= G.N) v[j] = 0.f;
         }
         if (kLast && kAux == 1) {
           // the CV trajectory: X' too, in the NS layout, for the next iteration
@@ -1022,7 +993,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           const TileCoord c = decode_tile<kPair, kBN, kSym>(p, t);
           const GemmGroup& G = p.g[c.g];
           const int nk = (G.K + BK - 1) / BK;
-          const bool b_is_a = kSym && kPair == 2 && G.same_ab && c.tm * TILE_M == c.tn * BN;
+          const bool b_is_a = kSym && kPair == 2 && c.tm * TILE_M == c.tn * BN;
           e.y = static_cast<uint32_t>(c.mat);
           e.z = static_cast<uint32_t>(c.g) | (static_cast<uint32_t>(c.tm) << 4) | (static_cast<uint32_t>(c.tn) << 18);
           e.w = static_cast<uint32_t>(nk) | (b_is_a ? 0x10000u : 0u);
@@ -1082,15 +1053,9 @@ int ns_gemm_smem_bytes(int pair) { return pair == 2 ? Cfg<2, 256>::SMEM_BYTES : 
 template <int kPair, int kBN, typename F>
 static cudaError_t with_kernel(int mode, int aux, F f) {
   constexpr int bytes = Cfg<kPair, kBN>::SMEM_BYTES;
-  if constexpr (kBN == 256)  // the paired iterations' products
-    if (aux == 2)
-      return mode == MODE_XLAST   ? f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 2>, bytes)
-             : mode == MODE_DENSE ? f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 2>, bytes)
-                                  : f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 2>, bytes);
   if (mode == MODE_XLAST)
     return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_XLAST, 0>, bytes);
-  if (mode == MODE_DENSE)
-    return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 0>, bytes);
+  if (mode == MODE_DENSE) return f(ns_gemm_kernel<kPair, kBN, MODE_DENSE, 0>, bytes);
   return aux ? f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 1>, bytes) : f(ns_gemm_kernel<kPair, kBN, MODE_SYM, 0>, bytes);
 }
 
@@ -1099,7 +1064,7 @@ cudaError_t prepare_ns_gemm() {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
   for (int mode : {MODE_SYM, MODE_DENSE, MODE_XLAST})
-    for (int aux = 0; aux < 3; ++aux) {
+    for (int aux = 0; aux < 2; ++aux) {
       cudaError_t e = with_kernel<1, 256>(mode, aux, set);
       if (e == cudaSuccess) e = with_kernel<1, 64>(mode, aux, set);
       if (e == cudaSuccess) e = with_kernel<2, 256>(mode, aux, set);
