@@ -265,6 +265,9 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
  * many of them are Newton-Schulz GEMM launches. */
 int meq_kernels_per_step(const meq_state* st);
 int meq_ns_gemm_launches_per_step(const meq_state* st);
+/* Columns of the output tiles of the i-th of those launches: 256, or 64 where
+ * the launch has few tiles (0: no such launch). For tests and profiles. */
+int meq_ns_gemm_tile_columns(const meq_state* st, int i);
 /* Floating-point operations of those products (Eq. (5) as written), the
  * symmetric ones counted as one triangle. */
 double meq_ns_flops_per_step(const meq_state* st);

@@ -1446,6 +1446,10 @@ int meq_ns_gemm_launches_per_step(const meq_state* st) {
   return st ? static_cast<int>(st->gemm.size()) : 0;
 }
 
+int meq_ns_gemm_tile_columns(const meq_state* st, int i) {
+  return st && i >= 0 && static_cast<size_t>(i) < st->gemm_tile.size() ? st->gemm_tile[static_cast<size_t>(i)].bn : 0;
+}
+
 double meq_ns_flops_per_step(const meq_state* st) {
   double f = 0.0;
   if (!st) return f;

@@ -56,6 +56,7 @@ EXPORTED = [
     "meq_read_direction_counts", "meq_reset_direction_counts", "meq_ns_cv_trajectory",
     "meq_check_canaries", "meq_canary_count", "meq_debug_corrupt_canary",
     "meq_step_prepare", "meq_step_apply", "meq_read_update", "meq_ns_flops_per_step",
+    "meq_ns_gemm_tile_columns",
 ]
 HIDDEN, REMAINING_2D, VECTOR = 0, 1, 2  # meq_kind
 RULE_MEQMUON, RULE_MUON = 0, 1          # meq_update_rule
@@ -115,6 +116,8 @@ def _load():
     lib.meq_state_bytes_kinds.restype = I
     lib.meq_ns_gemm_launches_per_step.argtypes = [P]
     lib.meq_ns_gemm_launches_per_step.restype = I
+    lib.meq_ns_gemm_tile_columns.argtypes = [P, I]
+    lib.meq_ns_gemm_tile_columns.restype = I
     lib.meq_ns_flops_per_step.argtypes = [P]
     lib.meq_ns_flops_per_step.restype = D
     lib.meq_read_direction_counts.argtypes = [P, I, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]
@@ -264,6 +267,11 @@ class MeqMuon:
     @property
     def ns_gemm_launches_per_step(self):
         return lib.meq_ns_gemm_launches_per_step(self._st)
+
+    @property
+    def ns_gemm_tile_columns(self):
+        """Tile width of each Newton-Schulz launch (meq_ns_gemm_tile_columns)."""
+        return [lib.meq_ns_gemm_tile_columns(self._st, i) for i in range(self.ns_gemm_launches_per_step)]
 
     @property
     def ns_flops_per_step(self):

@@ -124,25 +124,32 @@ def test_ns_output_is_that_of_the_weight_alone(meq, shape, count):
     [(384, 768), (768, 384), (768, 768), (129, 385)], [(63, 65), (64, 64), (65, 63), (128, 129), (192, 200)],
 ], ids=str)
 def test_tile_variants_agree(meq, shapes):
-    """A state of a few matrices runs its products on 64-column tiles of single CTAs, one of sixty
-    times as many on 256-column tiles of CTA pairs: the same U bit for bit on ragged shapes, and
-    statistics within fp32 summation order (1e-5); the large state staged against the oracle."""
-    many = shapes * 60
+    """A state of one such matrix runs its products on 64-column tiles of single CTAs, one that holds
+    sixty larger ones too on 256-column tiles of CTA pairs, every launch: the same U bit for bit on
+    ragged shapes, and statistics within fp32 summation order (1e-5); the large state staged against
+    the oracle."""
+    import torch
+
+    many = shapes + [(1024, 1024)] * 60 + shapes
     wl = W.custom_workload(shapes, pattern="both", base_sigma=0.01, seed=47)
     Gs, W0 = _to_dev(W.gradients(wl, 0)), _to_dev(W.initial_weights(wl))
-    a, b = meq.MeqMuon(shapes), meq.MeqMuon(many)
-    a.step([w.clone() for w in W0], Gs, LR, MU, WD, EPS)
-    pb = [w.clone() for _ in range(60) for w in W0]
-    b.step(pb, Gs * 60, LR, MU, WD, EPS)
+    b = meq.MeqMuon(many)
+    assert set(b.ns_gemm_tile_columns) == {256}
+    Gbig = torch.randn(1024, 1024, generator=torch.Generator().manual_seed(3)).cuda()
+    pb = [w.clone() for w in W0] + list(torch.zeros(60, 1024, 1024, device="cuda")) + [w.clone() for w in W0]
+    b.step(pb, Gs + [Gbig] * 60 + Gs, LR, MU, WD, EPS)
     for i in range(len(shapes)):
+        a = meq.MeqMuon(shapes[i:i + 1])
+        assert set(a.ns_gemm_tile_columns) == {64}
+        a.step([W0[i].clone()], Gs[i:i + 1], LR, MU, WD, EPS)
         for k in (i, len(many) - len(shapes) + i):
             U = b.read_ns_output(k)
-            assert np.array_equal(a.read_ns_output(i), U), (shapes[i], k)
-            sa, sb = a.read_stats(i), b.read_stats(k)
+            assert np.array_equal(a.read_ns_output(0), U), (shapes[i], k)
+            sa, sb = a.read_stats(0), b.read_stats(k)
             assert PT.max_rel(sa["r"], sb["r"]) <= 1e-5 and PT.max_rel(sa["c"], sb["c"]) <= 1e-5
             PT.check_step(W0[i].cpu().numpy(), Gs[i].cpu().double().numpy(), np.zeros(shapes[i]), pb[k].cpu().numpy(),
                           b.read_momentum(k), U, sb, LR, MU, WD, EPS, Ut_gpu=b.read_update(k))
-    a.close()
+        a.close()
     b.close()
 
 
