@@ -682,7 +682,7 @@ __device__ __forceinline__ FoldVec fold_vec(const MatInfo& M, int which, const f
   if (M.kind == KIND_HIDDEN) {
     const bool cols = (which == 1) != (M.trans != 0);  // which: 0 NS rows, 1 NS columns
     v.parts = parts + (which == 0 ? M.rpart_off : M.cpart_off);
-    v.count = which == 0 ? M.rparts : (M.s() + 31) / 32;
+    v.count = ((which == 0 ? M.l() : M.s()) + 31) / 32;
     v.len = which == 0 ? M.s() : M.l();
     v.dst = (cols ? cvec : rvec) + M.vec_off;
     v.inv = 1.0f / static_cast<float>(cols ? M.m : M.n);

@@ -51,10 +51,9 @@ struct Group {
   int64_t u_base = 0;      // element offset of the group's fp16 U block [count][m][un]
   int64_t mbase = 0;       // first slot of the group in the per-matrix inverse-norm array
   // Fused-statistics partials: the column sums (float offset in the slab), and
-  // the row sums, rparts per row, in the X buffer that the last update leaves
+  // the row sums, ceil(l / 32) per row, in the X buffer that the last update leaves
   // idle (CV trajectory, where each update writes U and X': in its own scratch).
   int64_t cpart_base = 0;
-  int64_t rparts = 0;
   float* rpart = nullptr;
   std::vector<int> mats;
   uint16_t* x[2] = {nullptr, nullptr};
@@ -323,7 +322,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
       xblks += M.trans ? ((M.m + kCastTile - 1) / kCastTile) * ((M.n + kCastTile - 1) / kCastTile)
                        : (M.m * M.n + kChunk - 1) / kChunk;
       folds += (M.s() + kFoldCols - 1) / kFoldCols + (M.l() + kFoldCols - 1) / kFoldCols;
-      max_parts = std::max(max_parts, 2 * ((M.l() + 255) / 256) * M.s() + (M.s() + 31) / 32 * M.l());
+      max_parts = std::max(max_parts, (M.l() + 31) / 32 * M.s() + (M.s() + 31) / 32 * M.l());
     } else {
       M.un = M.n;
       const bool one_pass = M.kind == KIND_TWO_SIDED && M.n <= kRowColMax;
@@ -336,7 +335,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
         parts += round_up(ns * M.n, 64);
         if (!one_pass) slabs += ns * ((M.n + 255) / 256);  // blocks: slab x 256-column chunk
         folds += (M.m + kThreads - 1) / kThreads + (M.n + kFoldCols - 1) / kFoldCols;
-        max_parts = std::max(max_parts, ns * M.n);
+        max_parts = std::max(max_parts, (M.m + M.slab_rows - 1) / M.slab_rows * M.n);
       }
     }
   }
@@ -598,11 +597,8 @@ bool build_gemm_plan(meq_state* st, std::string* why) {
         GemmGroup& Q = P.g[gi];
         Group& G = st->groups[g];
         const NsOp& op = op_of(g);
-        if (op.mode == MODE_XLAST) {
-          // two row partials per tile column
-          G.rparts = 2 * ((op_cols(G, op) + t.bn - 1) / t.bn);
+        if (op.mode == MODE_XLAST)
           G.rpart = st->trajectory_rpart ? st->trajectory_rpart : reinterpret_cast<float*>(G.x[op.b == BUF_X0 ? 1 : 0]);
-        }
         if (!fill_group(st, G, op, t, Q)) { *why = "cuTensorMapEncodeTiled failed"; return false; }
         Q.tile_begin = tiles;
         const int64_t n = int64_t(Q.tiles_per_mat) * Q.count;
@@ -704,7 +700,7 @@ meq_status meq_init_state_kinds(const meq_shape* shapes, const int* kinds, int n
 
 // trajectory_rpart (one-matrix state of meq_ns_cv_trajectory, else NULL): the NS
 // plan gives U's statistics after every iteration, not after the last one only;
-// room for 2 * ceil(l / 64) row partials of s floats.
+// room for ceil(l / 32) row partials of s floats.
 static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, const meq_options* opt,
                              void* cuda_stream, float* trajectory_rpart, meq_state** out) {
   if (!out) return fail(nullptr, MEQ_ERR_INVALID_ARG, "out is NULL");
@@ -798,10 +794,9 @@ static meq_status init_state(const meq_shape* shapes, const int* kinds, int n, c
   for (MatInfo& M : st->mats)
     if (M.kind == KIND_HIDDEN) {
       const Group& G = st->groups[M.group];
-      M.rparts = static_cast<int32_t>(G.rparts);
       // (an offset in floats from the partials' slab, whatever buffer they lie in)
       const auto at = reinterpret_cast<intptr_t>(G.rpart) - reinterpret_cast<intptr_t>(st->d_parts);
-      M.rpart_off = static_cast<int64_t>(at / static_cast<intptr_t>(sizeof(float))) + M.gidx * G.rparts * G.s;
+      M.rpart_off = static_cast<int64_t>(at / static_cast<intptr_t>(sizeof(float))) + M.gidx * ((G.l + 31) / 32) * G.s;
     }
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   std::vector<GroupInfo> gi(st->groups.size());
@@ -1317,7 +1312,7 @@ meq_status meq_ns_cv_trajectory(const float* h, int64_t rows, int64_t cols, int 
   // kernels' partial sums (k = 0) or the NS products' row partials (k >= 1)
   const int64_t rb = round_up(rows * 4, 256), cb = round_up(cols * 4, 256);
   const int64_t tb = round_up(static_cast<int64_t>(sizeof(MatStats)) * (steps + 1), 256);
-  const int64_t rparts = 2 * ((std::max(rows, cols) + 63) / 64) * std::min(rows, cols);
+  const int64_t rparts = (std::max(rows, cols) + 31) / 32 * std::min(rows, cols);
   const int64_t pb = round_up(std::max(row_col_stats_scratch_floats(rows, cols), rparts) * 4, 256);
   char* tmp = nullptr;
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&tmp), static_cast<size_t>(rb + cb + tb + pb));

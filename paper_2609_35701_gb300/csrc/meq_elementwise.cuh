@@ -14,11 +14,12 @@ constexpr int kRowColMax = 1024;   // longest row of the one-pass form: 32 value
 constexpr int kRowColThreads = 512;
 // The partial sums get a launch of their own (fold_kernel) when an entry has
 // more of them than this; below, one finalize block reads them in less time
-// than a launch takes. Statistics phase, one block per entry -> fold, then
-// finalize: 256 x 256 (2.6k partials) 8.5 -> 10.2 us; 56 weights of up to
-// 512 x 1376 (28k) 15.1 -> 13.6 us; Llama-350M (110k) 36.7 -> 31.4 us; two
-// 7B-class layers (1.8M) 318 -> 35 us; two 32000 x 768 embeddings (192k) and
-// the Llama-130M weights 79.7 -> 28.3 us.
+// than a launch takes. Whole steps of one weight, one block per entry -> fold,
+// then finalize (partials): 256 x 256 (4.1k) 74.2 -> 75.1 us; 256 x 512 (8.2k)
+// 82.1 -> 82.4; 200 x 768 (10.2k) 88.1 -> 87.8; 384 x 768 (18.4k) 97.8 -> 96.5;
+// 512 x 1376 (44k) 118.9 -> 115.7; 256 x 4096 (66k) 168.6 -> 161.4; of thirty,
+// 256 x 768 (12.3k) 148.5 -> 148.1. Statistics phase: two 7B-class layers 318 ->
+// 35 us; two 32000 x 768 embeddings and the Llama-130M weights 79.7 -> 28.3 us.
 constexpr int kFoldCols = 128;     // vector entries per block of the fold
 constexpr int64_t kFoldMinParts = 8192;
 

@@ -41,7 +41,6 @@ struct MatInfo {
   int32_t trans;         // 1 when the NS layout is W^T (m > n)
   int32_t group;         // shape group (hidden weights)
   int32_t kind;          // 0 hidden, 1 remaining 2D (two-sided), 2 vector
-  int32_t rparts;        // row partial sums of squares per NS row: two per tile column of the last update
   int32_t gidx;          // index inside its group
   int32_t slab_rows;     // rows per slab (remaining 2D)
   int64_t mom_off;       // float offset of B in the momentum slab
@@ -56,7 +55,7 @@ struct MatInfo {
   int64_t tile_begin;    // first cast tile (hidden weights only)
   int64_t xblk_begin;    // first momentum-and-X_0 block (hidden weights only)
   int64_t fold_begin;    // first block of the fold of the partial sums (hidden weights and remaining 2D)
-  int64_t rpart_off;     // float offset of NS-row partial sums of squares [rparts][s]
+  int64_t rpart_off;     // float offset of NS-row partial sums of squares [ceil(l/32)][s]
   int64_t cpart_off;     // float offset of column partial sums of squares: NS columns
                          // [ceil(s/32)][l] (hidden) or normalised columns [slabs][n] (remaining 2D)
   // oriented NS shape
@@ -116,7 +115,7 @@ struct GemmGroup {
   const void* aux;        // polynomial: the 16-bit A
   int64_t aux_ld;         // bytes
   int64_t aux_mstride;    // bytes
-  float* rpart;           // XLAST: NS-row partial sums of squares, [count][2 * tiles_n][M]
+  float* rpart;           // XLAST: NS-row partial sums of squares, [count][ceil(N/32)][M]
   float* cpart;           // XLAST: NS-column partial sums of squares, [count][ceil(M/32)][N]
   int32_t mode;           // GemmMode of the launch (read from g[0])
   uint32_t idesc;         // tcgen05 instruction descriptor

@@ -11,7 +11,7 @@
 //   MODE_DENSE: X' = P X * (alpha'/alpha) (s x l, contraction over s)
 //   MODE_XLAST: U = P X / alpha, written as fp16(2^14 U) in the weight's own
 //               layout, with the sums of squares of the stored U's rows and
-//               columns (Eq. (7)) reduced into per-tile partials (and X'
+//               columns (Eq. (7)) reduced into partials per 32 (and X'
 //               beside it for the CV trajectory)
 //
 // P X equals a X + (b A + c A^2) X of Eq. (5) exactly in real arithmetic.
@@ -812,7 +812,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
       const int row0 = c.tm * TILE_M + static_cast<int>(rank) * BM + q * 32;
       const int R = row0 / 32;  // 32-row block index
       const int rows_valid = min(32, G.M - row0);
-      float rsum = 0.f;            // XLAST: this lane's row, sum of squares over the tile
       const int nch = min(BN / 32, (G.N - c.tn * BN + 31) / 32);
       int ch0 = kSym ? max(0, R - c.tn * (BN / 32)) : 0;  // blocks strictly below the diagonal come from mirrors
       if ((ch0 & 1) != half) ++ch0;                // this warp's chunks: ch % 2 == half
@@ -914,6 +913,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           // Column sums of squares over the warp's 32 rows: transpose-reduce
           // so that lane j ends with the sum for column col0 + j.
           float sq[32];
+          float rsum = 0.f;  // this lane's row
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             sq[j] = v[j] * v[j];
@@ -931,6 +931,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
           }
           if (col0 + lane < G.N)
             G.cpart[(static_cast<int64_t>(c.mat) * ((G.M + 31) / 32) + R) * G.N + col0 + lane] = sq[0] * kUInvScale2;
+          if (row0 + lane < G.M)  // one partial per 32 columns, whichever the tile's width: so r is the same bit for bit
+            G.rpart[(static_cast<int64_t>(c.mat) * ((G.N + 31) / 32) + C) * G.M + row0 + lane] = rsum * kUInvScale2;
           // 8-element chunks that start below the row length stay inside the
           // padded row (stride = row length rounded up to 8); the slot holds
           // the block (filled above)
@@ -966,8 +968,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
         }
         __syncwarp();  // reconverge before the next warp-wide tcgen05.ld
       }
-      if (kLast && row0 + lane < G.M)  // one partial per (tile column, half)
-        G.rpart[(static_cast<int64_t>(c.mat) * G.tiles_n * 2 + c.tn * 2 + half) * G.M + row0 + lane] = rsum * kUInvScale2;
       tc_fence_before();
       __syncwarp();
       mbar_arrive_relaxed_cluster_lane0(kPair == 2 ? (acc == 0 ? tempty_target0 : tempty_target1) : TEMPTY_BAR(acc), lane);

@@ -103,6 +103,16 @@ def test_folded_statistics(meq, shapes, kinds):
     run_kinds(meq, W.custom_workload(shapes, pattern="both", seed=53, kinds=kinds), 2)
 
 
+@pytest.mark.parametrize("shape,folded", [((256, 256), False), ((256, 512), False), ((200, 768), True), ((768, 200), True),
+                                          ((512, 512), True)], ids=str)
+def test_fold_is_chosen_by_the_partial_sums_there_are(meq, shape, folded):
+    """A weight has ceil(l / 32) s + ceil(s / 32) l partial sums, whichever tiles wrote them; beyond 8192
+    they are folded by a launch of their own (momentum, norm, 15 products, [fold,] finalize, update)."""
+    opt = meq.MeqMuon([shape])
+    assert opt.kernels_per_step == 19 + int(folded)
+    opt.close()
+
+
 @pytest.mark.parametrize("n", [1, 2, 3, 5, 6, 7, 9, 130, 1367, 4099])
 def test_update_of_odd_rows(meq, n):
     """Rows that are no multiple of four: groups of four that straddle one or more row ends, both
