@@ -125,9 +125,9 @@ meq_status meq_state_bytes_kinds(const meq_shape* shapes, const int* kinds, int 
  * and the workspace, on the current CUDA device. opt may be NULL (defaults).
  * cuda_stream (cudaStream_t, may be NULL) orders the zero-fill. The shape
  * list is copied. On success *out owns device memory until meq_free.
- * Entries are updated independently, but the Newton-Schulz products are
- * planned for the whole list (tile sizes), and so is the order of some sums:
- * the last bits of an entry's statistics can depend on the other shapes. */
+ * Entries are updated independently: the launches are planned for the whole
+ * list, but every result of an entry is the same bit for bit whatever else
+ * the list holds (so a list split over several states gives what one gives). */
 meq_status meq_init_state(const meq_shape* shapes, int n, const meq_options* opt,
                           void* cuda_stream, meq_state** out);
 

@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(kFinThreads, 2) finalize_kernel(const MatInfo*
     for (int which = M.kind == KIND_HIDDEN ? 0 : 1; which < 2; ++which) {
       const FoldVec v = which == 0 ? v0 : v1;
       for (int64_t j = threadIdx.x; j < v.len; j += blockDim.x) {
-        const float rms = sqrtf(strided_sum8(v.parts + j, 0, v.count, v.len) * v.inv);
+        const float rms = sqrtf(strided_sum8(v.parts + j, v.count, v.len) * v.inv);
         v.dst[j] = rms;
         if (M.kind == KIND_TWO_SIDED) tvec[M.vec_off + j] = rms > delta ? 1.0f / rms : 0.f;
       }

@@ -225,20 +225,17 @@ bool valid_shapes(const meq_shape* shapes, int n, std::string* why) {
 
 float pow2_round(double x) { return static_cast<float>(std::ldexp(1.0, static_cast<int>(std::lround(std::log2(std::max(x, 1.0)))))); }
 
-// Rows per block of the one-pass form over the remaining 2D parameters: at
-// least kColSlab (the partial sums are sized for that), and as many more as
-// it takes for the blocks, one per SM at a time, to fill whole waves.
-int64_t rowcol_slab_rows(const meq_state* st) {
-  auto blocks = [&](int64_t rows) {
-    int64_t b = 0;
-    for (int i = 0; i < st->n; ++i)
-      if (st->kinds[i] == KIND_TWO_SIDED && st->shapes[i].cols <= kRowColMax) b += (st->shapes[i].rows + rows - 1) / rows;
-    return b;
-  };
+// Rows per block of the one-pass form over a remaining 2D parameter of m rows:
+// at least kColSlab (the partial sums are sized for that), and as many more as
+// it takes for its blocks, one per SM at a time, to fill whole waves. Chosen
+// for each parameter by itself: the slabs set the order of its column sums,
+// which the other parameters are to leave alone.
+int64_t rowcol_slab_rows(int64_t m, int num_sms) {
+  auto blocks = [&](int64_t rows) { return (m + rows - 1) / rows; };
   int64_t rows = kColSlab;
-  const int64_t waves = st->num_sms > 0 ? blocks(rows) / st->num_sms : 0;
+  const int64_t waves = num_sms > 0 ? blocks(rows) / num_sms : 0;
   if (waves > 0)
-    while (blocks(rows) > waves * st->num_sms && rows < 4 * kColSlab) rows += kRowColThreads / 32;
+    while (blocks(rows) > waves * num_sms && rows < 4 * kColSlab) rows += kRowColThreads / 32;
   return rows;
 }
 
@@ -284,7 +281,6 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
   }
   int64_t mom = 0, u = 0, vec = 0, parts = 0, chunks = 0, hchunks = 0, tiles = 0, rblks = 0, slabs = 0, xblks = 0;
   int64_t folds = 0, max_parts = 0, rcs = 0;
-  const int64_t slab_rows = rowcol_slab_rows(st);
   int64_t mslots = 0;
   for (auto& G : st->groups) {
     G.mbase = mslots;
@@ -326,7 +322,7 @@ void plan(meq_state* st, Layout* L, int64_t* off_mom, int64_t* off_u, int64_t* o
     } else {
       M.un = M.n;
       const bool one_pass = M.kind == KIND_TWO_SIDED && M.n <= kRowColMax;
-      M.slab_rows = static_cast<int32_t>(one_pass ? slab_rows : kColSlab);
+      M.slab_rows = static_cast<int32_t>(one_pass ? rowcol_slab_rows(M.m, st->num_sms) : kColSlab);
       if (one_pass) rcs += (M.m + M.slab_rows - 1) / M.slab_rows;
       else rblks += (M.m + 7) / 8;  // 8 rows (warps) per block
       if (M.kind == KIND_TWO_SIDED) {

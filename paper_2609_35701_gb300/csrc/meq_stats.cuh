@@ -6,24 +6,30 @@
 
 namespace meq {
 
-// sum_{k0 <= k < k1} p[k * stride] with eight independent partial sums (term
-// k0 + i goes to partial i % 8) so that the loads overlap; fixed order.
-__device__ __forceinline__ float strided_sum8(const float* __restrict__ p, int64_t k0, int64_t k1, int64_t stride) {
+// sum_{k < count} p[k * stride]: the sums of eight consecutive ranges of
+// ceil(count / 8) terms, side by side so that the loads overlap. The order is
+// that of fold_block, so an entry's statistics are the same bit for bit
+// whether or not the other entries of the state make it fold its partials.
+__device__ __forceinline__ float strided_sum8(const float* __restrict__ p, int64_t count, int64_t stride) {
   float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  int64_t k = k0;
-  for (; k + 8 <= k1; k += 8) {
+  const int n = static_cast<int>(count), per = (n + 7) / 8;
+  const int64_t range = per * stride;
+  int i = 0;
+  for (; i < n - 7 * per; ++i, p += stride) {  // all eight ranges have a term i
 #pragma unroll
-    for (int u = 0; u < 8; ++u) a8[u] += p[(k + u) * stride];
+    for (int u = 0; u < 8; ++u) a8[u] += p[u * range];
   }
+  for (; i < per; ++i, p += stride) {
 #pragma unroll
-  for (int u = 0; u < 7; ++u)
-    if (k + u < k1) a8[u] += p[(k + u) * stride];
+    for (int u = 0; u < 7; ++u)
+      if (u * per + i < n) a8[u] += p[u * range];
+  }
   return ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
 }
 
 // Sums of kFoldCols consecutive entries of partial sums [count][len], by a
 // block of kThreads: four entries per lane, an eighth of the partials per
-// warp, added in a fixed order. Thread t < kFoldCols returns the sum of entry
+// warp, added in a fixed order (strided_sum8's). Thread t < kFoldCols returns the sum of entry
 // j0 + t (if it exists).
 __device__ __forceinline__ float fold_block(const float* __restrict__ parts, int64_t count, int64_t len, int64_t j0,
                                             float (*sh)[kFoldCols]) {

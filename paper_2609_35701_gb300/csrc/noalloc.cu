@@ -162,12 +162,12 @@ __global__ void __launch_bounds__(kFinThreads) na_cv_kernel(int64_t m, int64_t n
     const int64_t nchunks = (n + kNaChunk - 1) / kNaChunk;
     const float* cpart = scratch + nchunks * m;
     for (int64_t i = threadIdx.x; i < m; i += kFinThreads) {
-      const float s = strided_sum8(scratch + i, 0, nchunks, m);
+      const float s = strided_sum8(scratch + i, nchunks, m);
       scratch[i] = s;  // only this thread reads or writes row i's partials
       r[i] = sqrtf(s * (1.0f / static_cast<float>(n)));
     }
     for (int64_t j = threadIdx.x; j < n; j += kFinThreads)
-      c[j] = sqrtf(strided_sum8(cpart + j, 0, nslabs, n) * (1.0f / static_cast<float>(m)));
+      c[j] = sqrtf(strided_sum8(cpart + j, nslabs, n) * (1.0f / static_cast<float>(m)));
     __syncthreads();
   }
   if (frob) {

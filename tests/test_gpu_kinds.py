@@ -113,6 +113,49 @@ def test_fold_is_chosen_by_the_partial_sums_there_are(meq, shape, folded):
     opt.close()
 
 
+def test_an_entry_is_updated_as_if_it_were_alone(meq):
+    """Two steps of a list of every kind (hidden weights with folded and unfolded partial sums, on either
+    tile width; remaining 2D parameters in one pass, with slabs of one and of several waves, and in two
+    passes; a vector), and of each entry in a state of its own: momentum, U, statistics, update and
+    parameters are equal bit for bit."""
+    import torch
+
+    pick = [((256, 256), O.HIDDEN), ((768, 200), O.HIDDEN), ((63, 65), O.HIDDEN), ((768, 2048), O.HIDDEN),
+            ((5000, 96), O.REMAINING_2D), ((30000, 20), O.REMAINING_2D), ((130, 2052), O.REMAINING_2D),
+            ((1, 512), O.VECTOR)]
+    rest = [((1024, 1024), O.HIDDEN)] * 40 + [((27000, 20), O.REMAINING_2D)] * 2
+    gen = torch.Generator().manual_seed(71)
+
+    def data(base):
+        return [torch.randn(s, generator=gen).mul_(base).mul_(torch.logspace(-1, 1, s[0])[:, None]).cuda()
+                for s, _ in pick + rest]
+
+    W0, Gs = data(0.02), [data(0.01), data(0.01)]
+
+    def run(idx):
+        all_ = pick + rest
+        opt = meq.MeqMuon([all_[i][0] for i in idx], kinds=[all_[i][1] for i in idx])
+        p = [W0[i].clone() for i in idx]
+        for G in Gs:
+            opt.step(p, [G[i] for i in idx], LR, MU, WD, EPS)
+        return opt, p
+
+    whole, pw = run(range(len(pick) + len(rest)))
+    for i, (shape, kind) in enumerate(pick):
+        alone, pa = run([i])
+        a, b = alone.read_stats(0), whole.read_stats(i)
+        nr, nc = (shape if kind != O.VECTOR else (1, 0))
+        assert np.array_equal(a["r"][:nr], b["r"][:nr]) and np.array_equal(a["c"][:nc], b["c"][:nc]), shape
+        assert [a[k] for k in ("gamma_r", "gamma_c", "direction")] == [b[k] for k in ("gamma_r", "gamma_c", "direction")]
+        assert np.array_equal(alone.read_momentum(0), whole.read_momentum(i))
+        assert np.array_equal(alone.read_update(0), whole.read_update(i)), shape
+        if kind == O.HIDDEN:
+            assert np.array_equal(alone.read_ns_output(0), whole.read_ns_output(i)), shape
+        assert torch.equal(pa[0], pw[i]), shape
+        alone.close()
+    whole.close()
+
+
 @pytest.mark.parametrize("n", [1, 2, 3, 5, 6, 7, 9, 130, 1367, 4099])
 def test_update_of_odd_rows(meq, n):
     """Rows that are no multiple of four: groups of four that straddle one or more row ends, both
