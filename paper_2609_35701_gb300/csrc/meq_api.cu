@@ -1249,10 +1249,15 @@ static meq_status read_back(meq_state* st, int i, bool raw, float* dst, const ch
   for (int64_t e0 = 0; e == cudaSuccess && e0 < numel; e0 += piece) {
     const int64_t e1 = std::min(numel, e0 + piece);
     e = launch_readback(st->ctx, M, i, raw, e0, e1, scratch, st->last_stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st->last_stream);
+    // The copy is on the stream that writes the scratch again, for the next
+    // piece or in the next step: a cudaMemcpy need not have ended when it
+    // returns if dst is memory of another device.
     if (e == cudaSuccess && !on_device)
-      e = cudaMemcpy(dst + e0, scratch, static_cast<size_t>(e1 - e0) * sizeof(float), cudaMemcpyDefault);
+      e = cudaMemcpyAsync(dst + e0, scratch, static_cast<size_t>(e1 - e0) * sizeof(float), cudaMemcpyDefault,
+                          st->last_stream);
   }
+  const cudaError_t done = cudaStreamSynchronize(st->last_stream);
+  if (e == cudaSuccess) e = done;
   if (tmp) cudaFree(tmp);
   return e == cudaSuccess ? MEQ_OK : cuda_fail(st, e, what);
 }

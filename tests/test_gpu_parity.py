@@ -202,6 +202,39 @@ def test_read_back_in_pieces(meq, shapes, canaries):
     b.close()
 
 
+@pytest.mark.parametrize("shape,kind", [((640, 300), 0), ((3000, 64), 1)], ids=str)
+def test_read_back_is_ordered_on_the_steps_stream(meq, shape, kind):
+    """U (in two pieces) and the update read into pinned and pageable memory while the step's own
+    non-blocking stream is busy, and the next step enqueued right after: what arrives is the last
+    step's, and the next step is the same as without the reads."""
+    import torch
+
+    st = torch.cuda.Stream()
+    gen = torch.Generator().manual_seed(73)
+    G = [(torch.randn(shape, generator=gen) * 0.01).cuda() for _ in range(3)]
+    a, b = (meq.MeqMuon([shape], kinds=[kind], stream=st) for _ in range(2))
+    pa, pb = ([torch.ones(shape, device="cuda")] for _ in range(2))
+    torch.cuda.synchronize()
+    dev = torch.empty(shape, device="cuda")
+    reads = [meq.lib.meq_read_update] + ([meq.lib.meq_read_ns_output] if kind == 0 else [])
+    for t in range(3):
+        a.step(pa, [G[t]], LR, MU, WD, EPS, stream=st)
+        got = []
+        for pinned in (True, False):
+            for read in reads:
+                host = torch.full(shape, float("nan"), pin_memory=pinned)
+                assert read(a._st, 0, host.data_ptr()) == 0
+                got.append(host)
+        b.step(pb, [G[t]], LR, MU, WD, EPS, stream=st)
+        for k, host in enumerate(got):
+            assert reads[k % len(reads)](b._st, 0, dev.data_ptr()) == 0
+            assert torch.equal(dev.cpu(), host), (t, k)
+    torch.cuda.synchronize()
+    assert torch.equal(pa[0], pb[0])
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("pair", [1, 0], ids=["cta_pair", "single_cta"])
 def test_separate_x0_cast(meq, pair):
     """X_0 normalised and cast by its own pass (ns_x0_fused = 0: momentum +
