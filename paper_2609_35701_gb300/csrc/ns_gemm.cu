@@ -460,7 +460,6 @@ __device__ __forceinline__ void add_aux(const uint8_t* slot, int r, float* v, fl
     }
   }
 }
-// The transposed block: element (row j, col r) = v[j] of lane r.
 // Writes the transpose of the 32 x 32 16-bit block in `src` into `dst` (both
 // 64-byte rows of four 16-byte chunks, chunk k of row r at k ^ ((r >> 1) & 3)):
 // ldmatrix .trans reads each 8 x 8 sub-block (g, q) as its transpose and
@@ -623,8 +622,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) ns_gemm_kernel(const __grid_co
   // first wait for the epilogue's outstanding global stores). Its read has
   // completed long before the slot can be written again: entry n + 16 is
   // written after the producer took entry n + 15, by which time every role
-  // has used entry n -- the operand ring holds at most 6 k-blocks and the
-  // accumulators 2 tiles.
+  // has used entry n -- the operand ring holds at most 8 k-blocks, so the MMA
+  // issuer is at most 8 tiles behind the producer, and the accumulators 2
+  // tiles, so the epilogue is at most 2 behind the issuer.
   auto sched_put = [&](int n, uint4 e) -> bool {
     const int i = n & (SCHED_D - 1);
     if (!wait_bounded(SEMPTY_BAR(i), ((n / SCHED_D) & 1) ^ 1u, err, DEV_TIMEOUT_SCHED_PUT, tmo)) return false;
